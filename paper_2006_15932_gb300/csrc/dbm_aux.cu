@@ -32,9 +32,9 @@ __global__ void __launch_bounds__(256)
     const long long N = (long long)nx * ny;
     const long long d = (long long)y * nx + x;
     const long long cell = (long long)(y + GY) * pitch + (x + GX);
-    const Images im = cell_images(x, y, nx, ny, bc_x, bc_y);
-    for (int p = 0; p < nplanes; ++p)
-        store_with_images(f + p * plane, cell, x, y, pitch, im, (real)src[p * N + d]);
+#pragma unroll 8
+    for (int p = 0; p < nplanes; ++p) f[p * plane + cell] = (real)src[p * N + d];
+    images_of_planes(f, plane, nplanes, cell, x, y, nx, ny, pitch, bc_x, bc_y);
 }
 
 template <typename real>
@@ -48,7 +48,26 @@ __global__ void __launch_bounds__(256)
     const long long N = (long long)nx * ny;
     const long long d = (long long)y * nx + x;
     const long long cell = (long long)(y + GY) * pitch + (x + GX);
-    for (int p = 0; p < nplanes; ++p) dst[p * N + d] = (double)f[p * plane + cell];
+    // eight loads in flight; their conversions by bits unless one of them needs
+    // the instruction (uniform over most warps)
+    static_assert(Q % 8 == 0, "planes come in groups of eight");
+    for (int p = 0; p < nplanes; p += 8) {
+        real v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = f[(p + k) * plane + cell];
+        if constexpr (sizeof(real) == 4) {
+            bool bits = true;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) bits = bits && widens_by_bits(v[k]);
+            if (bits) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) dst[(p + k) * N + d] = widen_bits(v[k]);
+                continue;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) dst[(p + k) * N + d] = (double)v[k];
+    }
 }
 
 #define DBM_DISPATCH_S(S_, CALL)             \

@@ -7,9 +7,43 @@
 #pragma once
 #include <stdio.h>
 
+#include <type_traits>
+
 #include "dbm_bf16.cuh"
 
 namespace dbm {
+
+// Ghost images of a cell's stored planes (masks from ghost_mask: comparisons
+// only, and a second look at the cell's own stores on the domain edge; the
+// images used to come from eight integer modulos in every cell: k_set_f on
+// 2048 x 1024 took 207 us, now 159).
+template <typename T>
+__device__ __forceinline__ void images_of_planes(T *f, long long plane, int nplanes, long long cell, int x, int y,
+                                                 int nx, int ny, int pitch, int bc_x, int bc_y)
+{
+    const unsigned mx = ghost_mask(x, nx, bc_x), my = ghost_mask(y, ny, bc_y);
+    if ((mx | my) == 0u) return;
+    for (int p = 0; p < nplanes; ++p) store_images(f + p * plane, x, y, nx, ny, pitch, mx, my, f[p * plane + cell]);
+}
+
+// (double)x on the integer pipe.  The conversion instruction shares the FP64
+// pipe, two lanes per SM and cycle here, and the output kernels convert every
+// value they read or write: exponent and mantissa are moved over instead
+// (k_moments_f32: half its time; k_get_f on 4096^2: 1.05 -> 0.99 ms).
+// Zeros keep their sign; subnormal, infinite and NaN values take the
+// instruction.
+__device__ __forceinline__ bool widens_by_bits(float x)
+{
+    const unsigned a = __float_as_uint(x) & 0x7fffffffu;
+    return a - 1u >= 0x007fffffu && a < 0x7f800000u;
+}
+__device__ __forceinline__ double widen_bits(float x)
+{
+    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+    const unsigned hi = a == 0u ? u : (u & 0x80000000u) | ((a >> 3) + 0x38000000u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(float x) { return widens_by_bits(x) ? widen_bits(x) : (double)x; }
 
 // f = f^eq(rho^s / m^s, u, T), computed in FP64 and rounded to `real`.
 template <typename real, int S>
@@ -24,7 +58,6 @@ __global__ void __launch_bounds__(256)
     const long long N = (long long)c.nx * c.ny;
     const long long d = (long long)y * c.nx + x;
     const long long cell = (long long)(y + GY) * c.pitch + (x + GX);
-    const Images im = cell_images(x, y, c.nx, c.ny, c.bc_x, c.bc_y);
     const double u_x = ux[d], u_y = uy[d], t = T[d];
 #pragma unroll 1
     for (int s = 0; s < S; ++s) {
@@ -34,9 +67,10 @@ __global__ void __launch_bounds__(256)
             double v = 0.0;
 #pragma unroll
             for (int k = 0; k < Q; ++k) v += c.cinv[s][i][k] * fh[k];
-            store_with_images(f + (s * Q + i) * c.plane, cell, x, y, c.pitch, im, (real)v);
+            f[(s * Q + i) * c.plane + cell] = (real)v;
         }
     }
+    images_of_planes(f, c.plane, S * Q, cell, x, y, c.nx, c.ny, c.pitch, c.bc_x, c.bc_y);
 }
 
 // 1 / m^s in FP64, for the conversion of the FP64 input fields.
@@ -62,7 +96,6 @@ __global__ void __launch_bounds__(256)
     const long long N = (long long)c.nx * c.ny;
     const long long d = (long long)y * c.nx + x;
     const long long cell = (long long)(y + GY) * c.pitch + (x + GX);
-    const Images im = cell_images(x, y, c.nx, c.ny, c.bc_x, c.bc_y);
     const float u_x = (float)ux[d], u_y = (float)uy[d];
     const double t = T[d];
 #pragma unroll 1
@@ -70,21 +103,25 @@ __global__ void __launch_bounds__(256)
         float cb[16], o[16];
         fhat_blocks<float>((float)(rho_s[s * N + d] * im_d.v[s]), u_x, u_y, (float)(t * im_d.v[s]), c.dpi[s], cb);
         solve_blocks<float>(c, s, cb, o);
-        for (int i = 0; i < Q; ++i)
-            store_with_images(f + (s * Q + i) * c.plane, cell, x, y, c.pitch, im, feq_of<float>(i, o));
+#pragma unroll
+        for (int i = 0; i < Q; ++i) f[(s * Q + i) * c.plane + cell] = feq_of<float>(i, o);
     }
+    images_of_planes(f, c.plane, S * Q, cell, x, y, c.nx, c.ny, c.pitch, c.bc_x, c.bc_y);
 }
 
 // Source of f for the output kernels: a plain FP64 or FP32 state buffer
 // (the BF16-deviation state has BfSrc, which rebuilds f).
 template <typename real>
 struct PlainSrc {
+    using value = real;
     const real *f;
     long long plane;
+    __device__ __forceinline__ static double widened(float v) { return widen(v); }
+    __device__ __forceinline__ static double widened(double v) { return v; }
     __device__ __forceinline__ void load16(int s, long long cell, double v[Q]) const
     {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) v[i] = (double)f[(s * Q + i) * plane + cell];
+        for (int i = 0; i < Q; ++i) v[i] = widened(f[(s * Q + i) * plane + cell]);
     }
     __device__ __forceinline__ void load16f(int s, long long cell, float v[Q]) const
     {
@@ -93,6 +130,39 @@ struct PlainSrc {
     }
 };
 
+// Sums of one ring of four values in FP64: all (mass), the vector part
+// (rx, ry) and the second moments' part per unit v^2 (axis rings: xx = f0 + f2
+// and yy = f1 + f3; diagonal rings: xx = yy = all and xy).  Additions in place
+// of the 16 products with each velocity component.
+struct RingSums {
+    double all, rx, ry, xx, yy, xy;
+};
+template <bool DIAG>
+__device__ __forceinline__ RingSums ring_sums(const double f[4])
+{
+    RingSums g;
+    const double a = f[0] + f[2], b = f[1] + f[3];
+    g.all = a + b;
+    if (DIAG) {
+        const double d = f[0] - f[2], e = f[3] - f[1];
+        g.rx = d + e;
+        g.ry = d - e;
+        g.xx = g.yy = g.all;
+        g.xy = a - b;
+    } else {
+        g.rx = f[0] - f[2];
+        g.ry = f[1] - f[3];
+        g.xx = a;
+        g.yy = b;
+        g.xy = 0.0;
+    }
+    return g;
+}
+__device__ __forceinline__ RingSums ring_sums(int r, const double f[4])
+{
+    return (r & 1) ? ring_sums<true>(f) : ring_sums<false>(f);
+}
+
 // Species moments of one cell in FP64: n, j = sum f v, E = sum f (v.v+eta^2).
 template <int S, class Src>
 __device__ __forceinline__ void cell_moments(const OutConsts<S> &c, const Src &src, long long cell,
@@ -100,22 +170,17 @@ __device__ __forceinline__ void cell_moments(const OutConsts<S> &c, const Src &s
 {
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        double sn = 0, sx = 0, sy = 0, se = 0;
         double fv[Q];
         src.load16(s, cell, fv);
+        n[s] = jx[s] = jy[s] = en[s] = 0.0;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const double v = fv[i];
-            const int r = i >> 2;
-            sn += v;
-            sx += dir_x(i) * c.vr[s][r] * v;
-            sy += dir_y(i) * c.vr[s][r] * v;
-            se += c.qr[s][r] * v;
+        for (int r = 0; r < 4; ++r) {
+            const RingSums g = ring_sums(r, fv + 4 * r);
+            n[s] += g.all;
+            jx[s] += c.vr[s][r] * g.rx;
+            jy[s] += c.vr[s][r] * g.ry;
+            en[s] += c.qr[s][r] * g.all;
         }
-        n[s] = sn;
-        jx[s] = sx;
-        jy[s] = sy;
-        en[s] = se;
     }
 }
 
@@ -179,16 +244,48 @@ __global__ void __launch_bounds__(256)
     out[(4 * S + 4) * N + d] = ntot * T;
 }
 
+// Kernel parameters of k_moments_f32: the constants as the floats it works
+// with (converting the double ones in the kernel costs the FP64 pipe).
+template <int S>
+struct MomentConsts {
+    float vr[S][4], qr[S][4], m[S], dpi[S];
+    float lam[S], kap[S];  // m / tau, (D + I) / tau
+    int nx, ny, pitch;
+};
+
+template <int S>
+inline MomentConsts<S> moment_consts(const OutConsts<S> &c)
+{
+    MomentConsts<S> k;
+    memset(&k, 0, sizeof(k));
+    for (int s = 0; s < S; ++s) {
+        for (int r = 0; r < 4; ++r) {
+            k.vr[s][r] = (float)c.vr[s][r];
+            k.qr[s][r] = (float)c.qr[s][r];
+        }
+        k.m[s] = (float)c.m[s];
+        k.dpi[s] = (float)c.dpi[s];
+        k.lam[s] = (float)(c.m[s] * c.inv_tau[s]);
+        k.kap[s] = (float)(c.dpi[s] * c.inv_tau[s]);
+    }
+    k.nx = c.nx;
+    k.ny = c.ny;
+    k.pitch = c.pitch;
+    return k;
+}
+
 // The macroscopic fields of a float state (DBM_FP32 or DBM_BF16DEV), in
 // float arithmetic, stored as FP64: the state carries float precision, and
 // on this GPU the FP64 evaluation of k_moments is bound by the FP64 pipe (8 ms
 // for 4096^2 cells against 0.6 ms for the memory traffic).  Species sums by
 // rings as in the step; the mixture temperature's cancelling subtraction in
 // float-float (mixture_T); u^s and T^s from n^s, j^s, E^s with one fused
-// multiply-add each.  Relative error a few float ulps of each field.
+// multiply-add each.  Relative error a few float ulps of each field.  Float
+// constants and widen() keep the FP64 pipe out of it but for one product a
+// cell: 4096^2, two species, 1.27 -> 0.59 ms, the memory time.
 template <int S, class Src>
 __global__ void __launch_bounds__(256)
-    k_moments_f32(const __grid_constant__ OutConsts<S> c, const __grid_constant__ Src src,
+    k_moments_f32(const __grid_constant__ MomentConsts<S> c, const __grid_constant__ Src src,
                   double *__restrict__ out)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -216,39 +313,73 @@ __global__ void __launch_bounds__(256)
                 rx = a + b;
                 ry = a - b;
             }
-            const float v = (float)c.vr[s][r];
             sn += rs;
-            sx = fmaf(v, rx, sx);
-            sy = fmaf(v, ry, sy);
-            se = fmaf((float)c.qr[s][r], rs, se);
+            sx = fmaf(c.vr[s][r], rx, sx);
+            sy = fmaf(c.vr[s][r], ry, sy);
+            se = fmaf(c.qr[s][r], rs, se);
         }
         const bool here = sn != 0.0f;  // an absent species reports zero velocity and temperature
         const float rn = here ? 1.0f / sn : 0.0f;
         const float usx = sx * rn, usy = sy * rn;
-        const float ts = here ? (float)c.m[s] * fmaf(-usx, usx, fmaf(-usy, usy, se * rn)) / (float)c.dpi[s] : 0.0f;
-        out[(4 * s + 0) * N + d] = sn;
-        out[(4 * s + 1) * N + d] = usx;
-        out[(4 * s + 2) * N + d] = usy;
-        out[(4 * s + 3) * N + d] = ts;
-        const float m = (float)c.m[s], lam = (float)(c.m[s] * c.inv_tau[s]);
-        const float kap = (float)(c.dpi[s] * c.inv_tau[s]);
-        rho = fmaf(m, sn, rho);
+        const float ts = here ? c.m[s] * fmaf(-usx, usx, fmaf(-usy, usy, se * rn)) / c.dpi[s] : 0.0f;
+        out[(4 * s + 0) * N + d] = widen(sn);
+        out[(4 * s + 1) * N + d] = widen(usx);
+        out[(4 * s + 2) * N + d] = widen(usy);
+        out[(4 * s + 3) * N + d] = widen(ts);
+        rho = fmaf(c.m[s], sn, rho);
         ntot += sn;
-        w = fmaf(lam, sn, w);
-        wx = fmaf(lam, sx, wx);
-        wy = fmaf(lam, sy, wy);
-        we = fmaf(lam, se, we);
-        wd = fmaf(kap, sn, wd);
+        w = fmaf(c.lam[s], sn, w);
+        wx = fmaf(c.lam[s], sx, wx);
+        wy = fmaf(c.lam[s], sy, wy);
+        we = fmaf(c.lam[s], se, we);
+        wd = fmaf(c.kap[s], sn, wd);
     }
     const float rw = 1.0f / w, ux = wx * rw, uy = wy * rw;
     const float T = mixture_T(we, w, wd, ux, uy);
-    out[(4 * S + 0) * N + d] = rho;
-    out[(4 * S + 1) * N + d] = ux;
-    out[(4 * S + 2) * N + d] = uy;
-    out[(4 * S + 3) * N + d] = T;
-    out[(4 * S + 4) * N + d] = (double)ntot * (double)T;
+    out[(4 * S + 0) * N + d] = widen(rho);
+    out[(4 * S + 1) * N + d] = widen(ux);
+    out[(4 * S + 2) * N + d] = widen(uy);
+    out[(4 * S + 3) * N + d] = widen(T);
+    out[(4 * S + 4) * N + d] = widen(ntot) * widen(T);
 }
 
+// The moments of rows 5..16 of M (xx, xy, yy, q x, q y, xxx, xxy, xyy, yyy,
+// q xx, q xy, q yy) of one species' values.
+template <int S>
+__device__ __forceinline__ void high_moments(const OutConsts<S> &c, int s, const double f[Q], double t[12])
+{
+#pragma unroll
+    for (int k = 0; k < 12; ++k) t[k] = 0.0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const RingSums g = ring_sums(r, f + 4 * r);
+        const double v = c.vr[s][r], q = c.qr[s][r], v2 = v * v, qv = q * v, qv2 = q * v2, v3 = v * v2;
+        t[0] += v2 * g.xx;
+        t[2] += v2 * g.yy;
+        t[3] += qv * g.rx;
+        t[4] += qv * g.ry;
+        t[5] += v3 * g.rx;
+        t[8] += v3 * g.ry;
+        t[9] += qv2 * g.xx;
+        t[11] += qv2 * g.yy;
+        if (r & 1) {
+            t[1] += v2 * g.xy;
+            t[6] += v3 * g.ry;
+            t[7] += v3 * g.rx;
+            t[10] += qv2 * g.xy;
+        }
+    }
+}
+
+// Nonequilibrium moments.  The equilibrium is M^-1 f-hat, so its moments of
+// the 16 monomials of M are f-hat itself, and all twelve moments of the
+// output are among them: Delta = m (M f - f-hat).  Neither f^eq nor a sum
+// over it is needed, and M f comes from ring sums: about 190 FP64 operations
+// per species and cell where summing f - f^eq over the velocities took 1400
+// (the FP64 pipe bounds this kernel: 2048 x 1024, two species, 7.9 -> 1.85
+// ms).
+// Up to two species keep their values in registers until the mixture u and T
+// are known; more load them again.
 template <int S, class Src>
 __global__ void __launch_bounds__(128)
     k_noneq(const __grid_constant__ OutConsts<S> c, const __grid_constant__ Src src,
@@ -264,107 +395,260 @@ __global__ void __launch_bounds__(128)
     cell_moments<S>(c, src, cell, n, jx, jy, en);
     double ux, uy, T;
     cell_mixture<S>(c, n, jx, jy, en, ux, uy, T);
-#pragma unroll 1
+#pragma unroll(S <= 2 ? S : 1)
     for (int s = 0; s < S; ++s) {
-        double fh[Q];
-        fhat16<double>(n[s], ux, uy, T / c.m[s], c.dpi[s], fh);
-        double acc[20];
+        double fc[Q], fh[Q], t[12];
+        double ns = n[0];  // selected, not indexed
 #pragma unroll
-        for (int k = 0; k < 20; ++k) acc[k] = 0.0;
-        const double m = c.m[s];
-        double fc[Q];
+        for (int j = 1; j < S; ++j)
+            if (s == j) ns = n[j];
         src.load16(s, cell, fc);
+        high_moments<S>(c, s, fc, t);
+        fhat16<double>(ns, ux, uy, T / c.m[s], c.dpi[s], fh);
+        const double m = c.m[s], hm = 0.5 * m;
+        double *o = out + 20LL * s * N + d;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            double feq = 0.0;
-#pragma unroll
-            for (int k = 0; k < Q; ++k) feq += c.cinv[s][i][k] * fh[k];
-            const int r = i >> 2;
-            const double vx = dir_x(i) * c.vr[s][r], vy = dir_y(i) * c.vr[s][r];
-            const double q = c.qr[s][r];
-            const double fv = fc[i];
-            const double dm = m * (fv - feq), mf = 0.5 * m * fv, me = 0.5 * m * feq;
-            acc[0] += dm * vx * vx;
-            acc[1] += dm * vx * vy;
-            acc[2] += dm * vy * vy;
-            acc[3] += dm * q * vx;
-            acc[4] += dm * q * vy;
-            acc[5] += dm * vx * vx * vx;
-            acc[6] += dm * vx * vx * vy;
-            acc[7] += dm * vx * vy * vy;
-            acc[8] += dm * vy * vy * vy;
-            acc[9] += dm * q * vx * vx;
-            acc[10] += dm * q * vx * vy;
-            acc[11] += dm * q * vy * vy;
-            acc[12] += mf * vx * vx;
-            acc[13] += mf * vy * vy;
-            acc[14] += me * vx * vx;
-            acc[15] += me * vy * vy;
-            acc[16] += mf * q * vx;
-            acc[17] += mf * q * vy;
-            acc[18] += me * q * vx;
-            acc[19] += me * q * vy;
-        }
-#pragma unroll
-        for (int k = 0; k < 20; ++k) out[(20 * s + k) * N + d] = acc[k];
+        for (int k = 0; k < 12; ++k) o[k * N] = m * (t[k] - fh[4 + k]);
+        o[12 * N] = hm * t[0];
+        o[13 * N] = hm * t[2];
+        o[14 * N] = hm * fh[4];
+        o[15 * N] = hm * fh[6];
+        o[16 * N] = hm * t[3];
+        o[17 * N] = hm * t[4];
+        o[18 * N] = hm * fh[7];
+        o[19 * N] = hm * fh[8];
     }
 }
 
-// Conserved totals: each block sums a fixed, strided subset of cells in a
-// fixed order and reduces them by a fixed tree; the final kernel adds the
-// block partials in block order.  The result is independent of timing.
+// Conserved totals: each block sums a fixed, strided subset of one species'
+// cells in a fixed order and reduces it by a fixed tree; the final kernel
+// adds the block partials in a fixed order.  The result is independent of
+// timing.
+//
+// The totals are linear in f, so a thread only adds up the ring sums of its
+// cells (12 sums a species) and the block forms mass, momentum and energy
+// from them once.  Float states: a ring sum and its running total over 16
+// cells are exact float-float pairs but for the last bits of the low parts
+// (about 2^-47 of the sum, below the rounding of the FP64 total they are
+// added to), on the FP32 pipes; the FP64 pipe, two lanes per SM and cycle,
+// then gets 1.5 additions per species and cell.  Multiplying every value by
+// its weights in FP64 took 190 (4096^2, two species: 8.7 -> 0.65 ms).
+struct FloatPair {
+    float h, l;
+    __device__ __forceinline__ void add(float s, float e)  // += s + e
+    {
+        float e2;
+        h = ff_sum(h, s, e2);
+        l = __fadd_rn(l, __fadd_rn(e, e2));
+    }
+};
+
+// Running sums of one ring: all, rx, ry.
+struct RingTotalF {
+    FloatPair a[3];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) a[k].h = a[k].l = 0.0f;
+    }
+    template <bool DIAG>
+    __device__ __forceinline__ void add(float f0, float f1, float f2, float f3)
+    {
+        float e0, e1, e2, e3, e4;
+        const float a02 = ff_sum(f0, f2, e0), a13 = ff_sum(f1, f3, e1), all = ff_sum(a02, a13, e2);
+        a[0].add(all, __fadd_rn(__fadd_rn(e0, e1), e2));
+        if (DIAG) {
+            const float p = ff_sum(f0, -f2, e0), q = ff_sum(f3, -f1, e1);
+            const float rx = ff_sum(p, q, e2), ry = ff_sum(p, -q, e3);
+            a[1].add(rx, __fadd_rn(__fadd_rn(e0, e1), e2));
+            a[2].add(ry, __fadd_rn(__fsub_rn(e0, e1), e3));
+        } else {
+            const float rx = ff_sum(f0, -f2, e3), ry = ff_sum(f1, -f3, e4);
+            a[1].add(rx, e3);
+            a[2].add(ry, e4);
+        }
+    }
+    // an infinite or NaN total has no error part
+    __device__ __forceinline__ double value(int k) const
+    {
+        return isfinite(a[k].h) ? widen(a[k].h) + widen(a[k].l) : (double)a[k].h;
+    }
+};
+struct RingTotalD {
+    double a[3];
+    __device__ __forceinline__ void clear() { a[0] = a[1] = a[2] = 0.0; }
+    template <bool DIAG>
+    __device__ __forceinline__ void add(double f0, double f1, double f2, double f3)
+    {
+        const double f[4] = {f0, f1, f2, f3};
+        const RingSums g = ring_sums<DIAG>(f);
+        a[0] += g.all;
+        a[1] += g.rx;
+        a[2] += g.ry;
+    }
+    __device__ __forceinline__ double value(int k) const { return a[k]; }
+};
+
+// The values of velocities 4 r .. 4 r + 3 of four cells in a row, v[velocity][cell]
+// (rows start 16-byte aligned; the row's padding covers a ragged last vector).
+__device__ __forceinline__ void load_ring4(const float *p, long long plane, float v[4][4])
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 q = __ldg(reinterpret_cast<const float4 *>(p + i * plane));
+        v[i][0] = q.x, v[i][1] = q.y, v[i][2] = q.z, v[i][3] = q.w;
+    }
+}
+__device__ __forceinline__ void load_ring4(const double *p, long long plane, double v[4][4])
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const double2 q = __ldg(reinterpret_cast<const double2 *>(p + i * plane));
+        const double2 w = __ldg(reinterpret_cast<const double2 *>(p + i * plane) + 1);
+        v[i][0] = q.x, v[i][1] = q.y, v[i][2] = w.x, v[i][3] = w.y;
+    }
+}
+
+template <class Total, typename real>
+__device__ __forceinline__ void total_cells(const PlainSrc<real> &src, int s, long long cell, int live, Total tot[4])
+{
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        real v[4][4];
+        load_ring4(src.f + (s * Q + 4 * r) * src.plane + cell, src.plane, v);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (j >= live) break;
+            if (r & 1)
+                tot[r].template add<true>(v[0][j], v[1][j], v[2][j], v[3][j]);
+            else
+                tot[r].template add<false>(v[0][j], v[1][j], v[2][j], v[3][j]);
+        }
+    }
+}
+template <class Total, int S>
+__device__ __forceinline__ void total_cells(const BfSrc<S> &src, int s, long long cell, int live, Total tot[4])
+{
+#pragma unroll 1
+    for (int j = 0; j < live; ++j) {
+        float f[Q];
+        src.load16f(s, cell + j, f);
+        tot[0].template add<false>(f[0], f[1], f[2], f[3]);
+        tot[1].template add<true>(f[4], f[5], f[6], f[7]);
+        tot[2].template add<false>(f[8], f[9], f[10], f[11]);
+        tot[3].template add<true>(f[12], f[13], f[14], f[15]);
+    }
+}
+
+// Blocks per species: four partials each, within the scratch's CONS_BLOCKS
+// times S + 4.
+constexpr int cons_blocks(int S) { return S == 1 ? 512 : CONS_BLOCKS / 4 * (S + 4) / S; }
+static_assert(4 * 1 * cons_blocks(1) <= CONS_BLOCKS * 5 && 4 * 2 * cons_blocks(2) <= CONS_BLOCKS * 6 &&
+                  4 * 3 * cons_blocks(3) <= CONS_BLOCKS * 7 && 4 * 4 * cons_blocks(4) <= CONS_BLOCKS * 8 &&
+                  4 * 5 * cons_blocks(5) <= CONS_BLOCKS * 9 && 4 * 6 * cons_blocks(6) <= CONS_BLOCKS * 10 &&
+                  4 * 7 * cons_blocks(7) <= CONS_BLOCKS * 11 && 4 * 8 * cons_blocks(8) <= CONS_BLOCKS * 12,
+              "conservation partials exceed the scratch buffer");
+
+__device__ __forceinline__ double warp_total(double v)
+{
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) v += __shfl_down_sync(0xffffffffu, v, w);
+    return v;
+}
+
 template <int S, class Src>
 __global__ void __launch_bounds__(256)
     k_cons_partial(const __grid_constant__ OutConsts<S> c, const __grid_constant__ Src src,
                    double *__restrict__ partial)
 {
-    constexpr int K = S + 4;
-    __shared__ double red[K][256];
-    double acc[K];
+    constexpr bool DOUBLE = std::is_same<typename Src::value, double>::value;
+    using Total = typename std::conditional<DOUBLE, RingTotalD, RingTotalF>::type;
+    constexpr int FLUSH = 4;  // vectors of four cells between additions to the FP64 sums
+    const int s = blockIdx.y;
+    double acc[4][3];
+    Total tot[4];
 #pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] = 0.0;
-    const long long N = (long long)c.nx * c.ny;
-    for (long long d = (long long)blockIdx.x * blockDim.x + threadIdx.x; d < N;
-         d += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(d % c.nx), y = (int)(d / c.nx);
+    for (int r = 0; r < 4; ++r) {
+        acc[r][0] = acc[r][1] = acc[r][2] = 0.0;
+        tot[r].clear();
+    }
+    const unsigned nv = (unsigned)(c.nx + 3) / 4u, count = nv * (unsigned)c.ny;
+    const unsigned stride = gridDim.x * 256u;
+    int held = 0;
+    for (unsigned t = blockIdx.x * 256u + threadIdx.x; t < count; t += stride) {
+        const unsigned y = t / nv, x = 4u * (t - y * nv);
         const long long cell = (long long)(y + GY) * c.pitch + (x + GX);
+        total_cells(src, s, cell, min(4, c.nx - (int)x), tot);
+        if (++held == FLUSH) {
+            held = 0;
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-            const double m = c.m[s];
-            double fv[Q];
-            src.load16(s, cell, fv);
+            for (int r = 0; r < 4; ++r) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const double v = fv[i];
-                const int r = i >> 2;
-                acc[s] += m * v;
-                acc[S] += m * v * (dir_x(i) * c.vr[s][r]);
-                acc[S + 1] += m * v * (dir_y(i) * c.vr[s][r]);
-                acc[S + 2] += 0.5 * m * v * c.qr[s][r];
-                if (c.has_reaction && s == c.fuel) acc[S + 3] += c.Qheat * v / c.abs_a_fuel;
+                for (int k = 0; k < 3; ++k) acc[r][k] += tot[r].value(k);
+                tot[r].clear();
             }
         }
     }
+    __shared__ double red[8][12];
 #pragma unroll
-    for (int k = 0; k < K; ++k) red[k][threadIdx.x] = acc[k];
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double v = warp_total(acc[r][k] + tot[r].value(k));
+            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][3 * r + k] = v;
+        }
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
+    if (threadIdx.x == 0) {
+        double n = 0.0, jx = 0.0, jy = 0.0, en = 0.0;
 #pragma unroll
-            for (int k = 0; k < K; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + w];
-        __syncthreads();
+        for (int r = 0; r < 4; ++r) {
+            double g[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                g[k] = 0.0;
+#pragma unroll
+                for (int w = 0; w < 8; ++w) g[k] += red[w][3 * r + k];
+            }
+            n += g[0];
+            jx += c.vr[s][r] * g[1];
+            jy += c.vr[s][r] * g[2];
+            en += c.qr[s][r] * g[0];
+        }
+        double *p = partial + 4 * ((long long)s * gridDim.x + blockIdx.x);
+        p[0] = n;
+        p[1] = jx;
+        p[2] = jy;
+        p[3] = en;
     }
-    if (threadIdx.x < K) partial[blockIdx.x * K + threadIdx.x] = red[threadIdx.x][0];
 }
 
-static __global__ void k_cons_final(const double *__restrict__ partial, int nblocks, int K,
-                             double *__restrict__ out)
+// One warp per species and sum (128 S threads).
+template <int S>
+static __global__ void __launch_bounds__(128 * S)
+    k_cons_final(const __grid_constant__ OutConsts<S> c, const double *__restrict__ partial, int nblocks,
+                 double *__restrict__ out)
 {
-    const int k = threadIdx.x;
-    if (k >= K) return;
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += partial[b * K + k];
-    out[k] = s;
+    __shared__ double sum[S][4];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, s = w >> 2, k = w & 3;
+    double v = 0.0;
+    for (int b = lane; b < nblocks; b += 32) v += partial[4 * ((long long)s * nblocks + b) + k];
+    v = warp_total(v);
+    if (lane == 0) sum[s][k] = v;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double px = 0.0, py = 0.0, en = 0.0, heat = 0.0;
+    for (int q = 0; q < S; ++q) {
+        const double m = c.m[q];
+        out[q] = m * sum[q][0];
+        px += m * sum[q][1];
+        py += m * sum[q][2];
+        en += 0.5 * m * sum[q][3];
+        if (c.has_reaction && q == c.fuel) heat = c.Qheat * sum[q][0] / c.abs_a_fuel;
+    }
+    out[S] = px;
+    out[S + 1] = py;
+    out[S + 2] = en;
+    out[S + 3] = heat;
 }
 
 inline dim3 cell_grid(const dbm_handle *h, dim3 block)
@@ -377,17 +661,17 @@ inline void set_state_t(dbm_handle *h, void *f, const double *rho_s, const doubl
                         const double *uy, const double *T, cudaStream_t st)
 {
     dim3 b(32, 8);
-    if (sizeof(real) == 4) {
+    if constexpr (sizeof(real) == 4) {
         StepConsts<float, S> c;
         fill_step_consts<float, S>(h, c);
         InvMass<S> im;
         for (int s = 0; s < S; ++s) im.v[s] = 1.0 / h->p.sp[s].m;
         k_set_state_blocks<S><<<cell_grid(h, b), b, 0, st>>>(c, (float *)f, rho_s, ux, uy, T, im);
-        return;
+    } else {
+        OutConsts<S> c;
+        fill_out_consts<S>(h, c);
+        k_set_state<real, S><<<cell_grid(h, b), b, 0, st>>>(c, (real *)f, rho_s, ux, uy, T);
     }
-    OutConsts<S> c;
-    fill_out_consts<S>(h, c);
-    k_set_state<real, S><<<cell_grid(h, b), b, 0, st>>>(c, (real *)f, rho_s, ux, uy, T);
 }
 
 // The source of f for a state buffer of this handle's precision.
@@ -411,10 +695,10 @@ inline void moments_t(dbm_handle *h, const Src &src, double *out, cudaStream_t s
     OutConsts<S> c;
     fill_out_consts<S>(h, c);
     dim3 b(32, 8);
-    if (h->p.precision == DBM_FP64)
+    if constexpr (std::is_same<typename Src::value, double>::value)
         k_moments<S, Src><<<cell_grid(h, b), b, 0, st>>>(c, src, out);
     else
-        k_moments_f32<S, Src><<<cell_grid(h, b), b, 0, st>>>(c, src, out);
+        k_moments_f32<S, Src><<<cell_grid(h, b), b, 0, st>>>(moment_consts<S>(c), src, out);
 }
 
 template <int S, class Src>
@@ -431,8 +715,11 @@ inline void cons_t(dbm_handle *h, const Src &src, double *partial, double *out, 
 {
     OutConsts<S> c;
     fill_out_consts<S>(h, c);
-    k_cons_partial<S, Src><<<CONS_BLOCKS, 256, 0, st>>>(c, src, partial);
-    k_cons_final<<<1, 32, 0, st>>>(partial, CONS_BLOCKS, S + 4, out);
+    const long long vectors = (long long)((h->p.nx + 3) / 4) * h->p.ny;
+    const long long full = (vectors + 255) / 256;
+    const int blocks = (int)(full < cons_blocks(S) ? full : cons_blocks(S));
+    k_cons_partial<S, Src><<<dim3(blocks, S), 256, 0, st>>>(c, src, partial);
+    k_cons_final<S><<<1, 128 * S, 0, st>>>(c, partial, blocks, out);
 }
 
 

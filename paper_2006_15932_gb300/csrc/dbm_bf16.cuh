@@ -110,6 +110,7 @@ __device__ __forceinline__ void bf_cell_f(const StepConsts<float, S> &k, const B
 // Source policy of the FP64 output kernels for a BF16-deviation state.
 template <int S>
 struct BfSrc {
+    using value = float;
     StepConsts<float, S> k;
     BfState st;
     __device__ __forceinline__ void load16(int s, long long cell, double v[Q]) const

@@ -14,7 +14,7 @@ namespace dbm {
 constexpr int Q = 16;
 constexpr int GX = 4;  // ghost columns left of the interior (2 used; 4 keep rows 16-byte aligned)
 constexpr int GY = 2;  // ghost rows above and below the interior
-constexpr int CONS_BLOCKS = 512;          // fixed grid of the conservation reduction
+constexpr int CONS_BLOCKS = 512;          // partials of the conservation reduction, in units of S + 4 doubles
 constexpr size_t SCRATCH_HEAD = 256;      // health flag area at the start of scratch
 // polls of an mbarrier wait for a tile copy before it gives up (each poll
 // may suspend the thread for a while); the first wait of a step can be
