@@ -153,6 +153,14 @@ void fill_out_consts(const dbm_handle *h, OutConsts<S> &c)
 
 namespace dbm {
 
+// Divisors within 2^+-100 take the reciprocal for dividends within 2^+-800:
+// quotient and remainder then stay in the normal range.
+inline ConstDiv const_div(double b)
+{
+    const bool ok = b >= 0x1p-100 && b <= 0x1p100;
+    return ConstDiv{b, 1.0 / b, ok ? 1023u - 800u : 0xffffffffu, ok ? 1600u : 0u};
+}
+
 template <int S>
 void fill_f64_consts(const dbm_handle *h, F64Consts<S> &c)
 {
@@ -160,21 +168,20 @@ void fill_f64_consts(const dbm_handle *h, F64Consts<S> &c)
     const dbm_params &p = h->p;
     for (int s = 0; s < S; ++s) {
         const dbm_species &sp = p.sp[s];
-        for (int i = 0; i < Q; ++i) {
-            for (int k = 0; k < Q; ++k) c.cinv[s][i][k] = h->cinv[s][i][k];
-            const double x = dir_x(i) * sp.v[i >> 2], y = dir_y(i) * sp.v[i >> 2], e = sp.eta[i >> 2];
-            c.vx[s][i] = x;
-            c.vy[s][i] = y;
-            c.q[s][i] = x * x + y * y + e * e;  // host code is built without contraction
+        for (int r = 0; r < 4; ++r) {
+            for (int k = 0; k < Q; ++k) c.row[s][r][k] = h->cinv[s][4 * r][k];
+            const double x = sp.v[r], y = (r & 1) ? sp.v[r] : 0.0, e = sp.eta[r];
+            c.vr[s][r] = x;
+            c.qr[s][r] = x * x + y * y + e * e;  // host code is built without contraction
         }
-        c.m[s] = sp.m;
+        c.md[s] = const_div(sp.m);
+        c.taud[s] = const_div(sp.tau);
         c.I[s] = sp.I;
-        c.tau[s] = sp.tau;
         c.a[s] = sp.a_stoich;
     }
     c.dt = p.dt;
-    c.dx = p.dx;
-    c.dy = p.dy;
+    c.dxd = const_div(p.dx);
+    c.dyd = const_div(p.dy);
     c.ax = p.accel[0];
     c.ay = p.accel[1];
     c.k_ov = p.k_ov;

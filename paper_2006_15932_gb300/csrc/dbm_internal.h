@@ -206,15 +206,24 @@ int set_cuda_error(dbm_handle *h, cudaError_t e, const char *what);
 
 namespace dbm {
 
+// A constant divisor b with y = 1/b rounded to nearest; quotients of dividends
+// with biased exponents lo .. lo + span (and zero) may use y (dbm_step_f64.cu).
+struct ConstDiv {
+    double b, y;
+    unsigned lo, span;
+};
+
 // Kernel parameters of the FP64 reference-order step (dbm_step_f64.cu):
-// per-velocity constants so that every product is formed as in the
-// plain restatement of the paper (same operands, same order).
+// constants such that every product is formed as in the plain restatement
+// of the paper (same operands, same order).
 template <int S>
 struct F64Consts {
-    double cinv[S][Q][Q];
-    double vx[S][Q], vy[S][Q], q[S][Q];  // q = vx*vx + vy*vy + eta*eta
-    double m[S], I[S], tau[S], a[S];
-    double dt, dx, dy, ax, ay;
+    double row[S][4][Q];          // M^-1 of each ring's first velocity, (+,0) or (+,+)
+    double vr[S][4], qr[S][4];    // ring speed; vx*vx + vy*vy + eta*eta
+    ConstDiv md[S], taud[S];      // m, tau
+    double I[S], a[S];
+    ConstDiv dxd, dyd;            // dx, dy
+    double dt, ax, ay;
     double k_ov, Ea_over_R, Qheat;
     int fuel, oxid, has_reaction, has_force;
     int nx, ny, pitch, bc_x, bc_y;

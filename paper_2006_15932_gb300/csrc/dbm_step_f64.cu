@@ -18,194 +18,460 @@
 //     separate terms (Eqs. CollisionTerm, ReactionTerm, ForceTerm);
 //   - NND fluxes H from the split fluxes F+- = (c +- |c|)/2 f;
 //   - f^{n+1} = f + dt (Omega + R + G - d(v_x f)/dx - d(v_y f)/dy).
-// One thread per cell; ghosts of the new state are written as images.
+//
+// What bounds it: the FP64 pipe, two lanes per SM and cycle on this GPU (a
+// warp's instruction occupies it for 16 cycles; 64 FP32 or integer lanes go
+// by meanwhile).  So the work is arranged to issue few FP64 instructions, to
+// fill their 32 lanes, and to reach every SM; everything that rounds the same
+// with less of that pipe is done with less:
+//   - the half of each split flux that is zero is left out, the limiter is a
+//     choice between its arguments on the integer pipe, and its half joins
+//     the flux in one multiply-add (the half of a double is exact);
+//   - in M^-1 f-hat, the entries that vanish by symmetry (at most 1e-31 of
+//     their neighbours as computed) are left out, and the four velocities of
+//     a ring, whose entries differ in sign only, share each product;
+//   - a division by a constant b is a product with 1/b and two multiply-adds
+//     (Markstein 1990: with y = RN(1/b), q = RN(a y), r = RN(a - q b) exact,
+//     RN(q + r y) is the rounded quotient).
+// About 900 FP64 instructions per species and cell; the plain form of the same
+// arithmetic had 2500 (two species, 512 x 384: 2342 us a step, now 745,
+// with the pipe at the rate that back-to-back additions reach, one warp
+// instruction in 19 cycles).
+//
+// A CTA steps CELLS cells (consecutive in row order, so ragged rows leave no
+// lane idle) in phases through shared memory, each with its own split:
+//   1  the 4 moment sums of a cell and species, one thread each (each sum is
+//      a serial chain, the four run side by side);
+//   2  species velocities and weights, one thread per cell and species;
+//   3  mixture u, T and the rate, one thread per cell;
+//   4  f-hat of each term, one thread per cell and species;
+//   5  collision, advection and update, a warp per ring of four velocities:
+//      WIDE, 32 cells with the ring's four velocities in each thread (shared
+//      products); else 8 cells with a velocity per thread, four times as many
+//      CTAs, which a small grid needs to reach every SM and to shorten the
+//      chain of dependent operations (400 x 1, two species: 268 us a step,
+//      now 18).  NARROW_CELLS is where the two cross.
+// Ghosts of the new state are written as images by the edge cells.
 #include "dbm_consts.h"
 #include "dbm_device.cuh"
+#include "dbm_step_impl.cuh"
 
 namespace dbm {
 
-// f-hat_1..16 at (n, u, T) for a species of mass m and extra degrees of
-// freedom I, theta = T/m, D = 2, in the printed form.
-__device__ __forceinline__ void fhat_printed(double n, double ux, double uy, double T, double m, double I,
-                                             double fh[Q])
+// a / d.b rounded to nearest (see above).  Operands whose remainder could
+// leave the normal range, and divisors a host check refuses (span 0), take
+// the division itself.
+__device__ __forceinline__ double div_by(double a, const ConstDiv &d)
 {
-    const double D = 2.0;
-    const double th = T / m;
-    const double u2 = ux * ux + uy * uy;
-    fh[0] = n;
-    fh[1] = n * ux;
-    fh[2] = n * uy;
-    fh[3] = n * ((D + I) * th + u2);
-    fh[4] = n * (th + ux * ux);
-    fh[5] = n * ux * uy;
-    fh[6] = n * (th + uy * uy);
-    fh[7] = n * ux * ((D + I + 2.0) * th + u2);
-    fh[8] = n * uy * ((D + I + 2.0) * th + u2);
-    fh[9] = 3.0 * n * ux * th + n * ux * ux * ux;
-    fh[10] = n * uy * th + n * ux * ux * uy;
-    fh[11] = n * ux * th + n * ux * uy * uy;
-    fh[12] = 3.0 * n * uy * th + n * uy * uy * uy;
-    fh[13] = n * ((D + I + 2.0) * th + u2) * th + n * ux * ux * ((D + I + 4.0) * th + u2);
-    fh[14] = n * ux * uy * ((D + I + 4.0) * th + u2);
-    fh[15] = n * ((D + I + 2.0) * th + u2) * th + n * uy * uy * ((D + I + 4.0) * th + u2);
+    const unsigned hi = (unsigned)__double2hiint(a) & 0x7fffffffu;
+    const bool zero = (hi | (unsigned)__double2loint(a)) == 0u;
+    if ((hi >> 20) - d.lo <= d.span || (zero && d.span != 0u)) {
+        const double q = a * d.y;
+        return fma(fma(-q, d.b, a), d.y, q);
+    }
+    return a / d.b;
 }
 
-template <int S>
-__device__ __forceinline__ void feq_printed(const F64Consts<S> &c, int s, double n, double ux, double uy,
-                                            double T, double feq[Q])
+// minmod(a, b) = (sgn a + sgn b)/2 min(|a|, |b|): one of the arguments or 0,
+// chosen by integer comparisons of the bits.
+__device__ __forceinline__ double minmod_bits(double a, double b)
 {
-    double fh[Q];
-    fhat_printed(n, ux, uy, T, c.m[s], c.I[s], fh);
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+    const long long ma = ia & 0x7fffffffffffffffLL, mb = ib & 0x7fffffffffffffffLL;
+    const long long m = ma < mb ? ia : ib;
+    return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(m);
+}
+
+// d(c f)/dx of one velocity component of magnitude v at the cell p points
+// to; e: element offset of the neighbour downwind (the sign of c times the
+// stride), g0 = v f.  Seen along c, both signs have the same flux
+// H = v f + minmod(...)/2.
+__device__ __forceinline__ double nnd_dflux(double fm2, double fm1, double fp1, double g0, double v,
+                                            const ConstDiv &h)
+{
+    const double gm2 = v * fm2, gm1 = v * fm1, gp1 = v * fp1;
+    const double d0 = gm1 - gm2, d1 = g0 - gm1, d2 = gp1 - g0;
+    const double hr = fma(0.5, minmod_bits(d1, d2), g0), hl = fma(0.5, minmod_bits(d0, d1), gm1);
+    return div_by(hr - hl, h);
+}
+
+// f-hat_1..16 at (n, u, T) for a species of mass m and extra degrees of
+// freedom I, theta = T/m, D = 2, in the printed form; written to
+// fh[k * stride].
+__device__ __forceinline__ void fhat_printed(double n, double ux, double uy, double T, const ConstDiv &m, double I,
+                                             double *fh, int stride)
+{
+    const double D = 2.0;
+    const double th = div_by(T, m);
+    const double u2 = ux * ux + uy * uy;
+    const double a0 = (D + I) * th + u2, a2 = (D + I + 2.0) * th + u2, a4 = (D + I + 4.0) * th + u2;
+    fh[0] = n;
+    fh[1 * stride] = n * ux;
+    fh[2 * stride] = n * uy;
+    fh[3 * stride] = n * a0;
+    fh[4 * stride] = n * (th + ux * ux);
+    fh[5 * stride] = n * ux * uy;
+    fh[6 * stride] = n * (th + uy * uy);
+    fh[7 * stride] = n * ux * a2;
+    fh[8 * stride] = n * uy * a2;
+    fh[9 * stride] = 3.0 * n * ux * th + n * ux * ux * ux;
+    fh[10 * stride] = n * uy * th + n * ux * ux * uy;
+    fh[11 * stride] = n * ux * th + n * ux * uy * uy;
+    fh[12 * stride] = 3.0 * n * uy * th + n * uy * uy * uy;
+    fh[13 * stride] = n * a2 * th + n * ux * ux * a4;
+    fh[14 * stride] = n * ux * uy * a4;
+    fh[15 * stride] = n * a2 * th + n * uy * uy * a4;
+}
+
+// Rows of M^-1.  The row of the ring's first velocity, (+,0) or (+,+), gives
+// every other: along y an axis ring has the x row's entries at the mirrored
+// moments, opposite velocities have the odd moments negated, and on the
+// diagonals the sign of an entry is that of its moment.  Terms are added in
+// the printed order k = 0..15.
+__host__ __device__ constexpr int axis_k(int y, int j)  // moments of an axis row, in order
+{
+    return y ? (j == 0 ? 0 : j == 1 ? 2 : j == 2 ? 3 : j == 3 ? 4 : j == 4 ? 6 : j == 5 ? 8 : j == 6 ? 10 : j == 7 ? 12
+                : j == 8 ? 13 : 15)
+             : (j == 0 ? 0 : j == 1 ? 1 : j == 2 ? 3 : j == 3 ? 4 : j == 4 ? 6 : j == 5 ? 7 : j == 6 ? 9 : j == 7 ? 11
+                : j == 8 ? 13 : 15);
+}
+__host__ __device__ constexpr int axis_c(int y, int j)  // where the x row has that entry
+{
+    return y ? (j == 0 ? 0 : j == 1 ? 1 : j == 2 ? 3 : j == 3 ? 6 : j == 4 ? 4 : j == 5 ? 7 : j == 6 ? 11 : j == 7 ? 9
+                : j == 8 ? 15 : 13)
+             : axis_k(0, j);
+}
+__host__ __device__ constexpr bool axis_odd(int j) { return j == 1 || j == 5 || j == 6 || j == 7; }
+// powers of v_x and v_y (mod 2) in moment k
+__host__ __device__ constexpr bool odd_x(int k) { return k == 1 || k == 5 || k == 7 || k == 9 || k == 11 || k == 14; }
+__host__ __device__ constexpr bool odd_y(int k) { return k == 2 || k == 5 || k == 8 || k == 10 || k == 12 || k == 14; }
+
+// Output of the ring's equilibrium: V = 4 velocities per thread (lane: cell)
+// or V = 1 (velocity `vel` of the ring).  row: 16 entries of the ring's
+// first velocity; fh[k * CELLS]: the cell's moments.
+template <bool DIAG, int V, int CELLS>
+__device__ __forceinline__ void ring_equilibrium(const double *row, const double *fh, int vel, double f[V])
+{
+    if constexpr (DIAG) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        double acc = 0.0;
+        for (int k = 0; k < Q; ++k) {
+            const double t = row[k] * fh[k * CELLS];
 #pragma unroll
-        for (int k = 0; k < Q; ++k) acc += c.cinv[s][i][k] * fh[k];
-        feq[i] = acc;
+            for (int v = 0; v < V; ++v) {
+                const int i = V == 4 ? v : vel;
+                const bool neg = (odd_x(k) && (i == 1 || i == 2)) != (odd_y(k) && (i == 2 || i == 3));
+                const double s = neg ? -t : t;
+                f[v] = k == 0 ? s : f[v] + s;
+            }
+        }
+    } else if constexpr (V == 4) {
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+            for (int j = 0; j < 10; ++j) {
+                const double t = row[axis_c(y, j)] * fh[axis_k(y, j) * CELLS];
+                f[y] = j == 0 ? t : f[y] + t;
+                f[y + 2] = j == 0 ? t : axis_odd(j) ? f[y + 2] - t : f[y + 2] + t;
+            }
+    } else {
+        const bool y = vel & 1, back = vel & 2;
+#pragma unroll
+        for (int j = 0; j < 10; ++j) {
+            const double c = y ? row[axis_c(1, j)] : row[axis_c(0, j)];
+            const double t = c * fh[(y ? axis_k(1, j) : axis_k(0, j)) * CELLS];
+            const double s = axis_odd(j) && back ? -t : t;
+            f[0] = j == 0 ? s : f[0] + s;
+        }
     }
 }
 
-__device__ __forceinline__ double minmod_printed(double a, double b)
+// Moment sum k of a species (n, j_x, j_y, E), terms in velocity order.
+template <int K>
+__device__ __forceinline__ double moment_sum(const double v[4], const double q[4], const double f[Q])
 {
-    const double sa = a > 0.0 ? 1.0 : (a < 0.0 ? -1.0 : 0.0);
-    const double sb = b > 0.0 ? 1.0 : (b < 0.0 ? -1.0 : 0.0);
-    const double fa = fabs(a), fb = fabs(b);
-    return 0.5 * (sa + sb) * (fa < fb ? fa : fb);
+    double sum = 0.0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        if ((K == 1 && dir_x(i) == 0) || (K == 2 && dir_y(i) == 0)) continue;
+        const double w = K == 1 ? dir_x(i) * v[i >> 2] : K == 2 ? dir_y(i) * v[i >> 2] : q[i >> 2];
+        sum = sum + (K == 0 ? f[i] : f[i] * w);
+    }
+    return sum;
 }
 
-// d(c f)/dx at node j from w0..w4 = f_{j-2..j+2}: NND flux difference / h.
-__device__ __forceinline__ double nnd_dflux(double cv, double w0, double w1, double w2, double w3, double w4,
-                                            double h)
-{
-    const double cp = 0.5 * (cv + fabs(cv)), cm = 0.5 * (cv - fabs(cv));
-    const double p0 = cp * w0, p1 = cp * w1, p2 = cp * w2, p3 = cp * w3;
-    const double m1 = cm * w1, m2 = cm * w2, m3 = cm * w3, m4 = cm * w4;
-    const double hr = p2 + 0.5 * minmod_printed(p2 - p1, p3 - p2) + m3 - 0.5 * minmod_printed(m3 - m2, m4 - m3);
-    const double hl = p1 + 0.5 * minmod_printed(p1 - p0, p2 - p1) + m2 - 0.5 * minmod_printed(m2 - m1, m3 - m2);
-    return (hr - hl) / h;
-}
+// Values of a cell and species between phases 2 and 4, and of a cell
+// between 3 and 4.
+enum { W_RHO = 0, W_LAM, W_LX, W_LY, W_ME, W_CAP, W_UX, W_UY, W_TS, W_N };
+enum { M_UX = 0, M_UY, M_T, M_NTOT, M_OMEGA, M_DT, M_COUNT };
+
+__host__ __device__ constexpr int f64_side(int S) { return S >= 2 ? 2 : 1; }  // species side by side in phase 5
 
 template <int S>
-__global__ void __launch_bounds__(128)
+constexpr size_t f64_smem(int cells, int sets)
+{
+    return sizeof(double) * (size_t)cells * (S * Q * sets + S * (4 + W_N) + M_COUNT);
+}
+
+template <int S, bool WIDE>
+__global__ void __launch_bounds__(128 * f64_side(S))
     k_step_f64(const __grid_constant__ F64Consts<S> c, const double *__restrict__ fin,
                double *__restrict__ fout, unsigned *__restrict__ flag)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= c.nx || y >= c.ny) return;
-    const long long P = c.plane, py = c.pitch;
-    const long long cell = (long long)(y + GY) * c.pitch + (x + GX);
+    constexpr int CELLS = WIDE ? 32 : 8, SW = f64_side(S), NT = 128 * SW, V = WIDE ? 4 : 1;
+    extern __shared__ __align__(16) double sm[];
+    double *mom = sm;                          // [S][4][CELLS]
+    double *wts = mom + S * 4 * CELLS;         // [S][W_N][CELLS]
+    double *mix = wts + S * W_N * CELLS;       // [M_COUNT][CELLS]
+    double *fhs = mix + M_COUNT * CELLS;       // [sets][S][Q][CELLS]
+    const long long P = c.plane;
+    const unsigned d0 = blockIdx.x * (unsigned)CELLS, total = (unsigned)c.nx * (unsigned)c.ny;
+    const int tid = threadIdx.x;
+    const bool react = c.has_reaction != 0, force = c.has_force != 0;
+    // a cell past the end takes the last one's values and stores nothing
+    auto locate = [&](int j, unsigned &x, unsigned &y) {
+        const unsigned d = min(d0 + (unsigned)j, total - 1u);
+        y = d / (unsigned)c.nx;
+        x = d - y * (unsigned)c.nx;
+        return (long long)(y + GY) * c.pitch + (x + GX);
+    };
 
-    double n[S], ux[S], uy[S], Ts[S], E[S];
+    // 1. moment sums
+#pragma unroll 1
+    for (int it = tid; it < S * 4 * CELLS; it += NT) {
+        const int j = it % CELLS, k = (it / CELLS) & 3, s = it / (4 * CELLS);
+        unsigned x, y;
+        const long long cell = locate(j, x, y);
+        const double *pl = fin + (long long)s * Q * P + cell;
+        double f[Q], sum;
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-        double sn = 0.0, jx = 0.0, jy = 0.0, se = 0.0;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const double f = fin[(s * Q + i) * P + cell];
-            sn += f;
-            jx += f * c.vx[s][i];
-            jy += f * c.vy[s][i];
-            se += f * c.q[s][i];
-        }
-        n[s] = sn;
-        E[s] = se;
-        if (sn == 0.0) {  // an absent species: zero velocity and temperature
-            ux[s] = 0.0;
-            uy[s] = 0.0;
-            Ts[s] = 0.0;
+        for (int i = 0; i < Q; ++i) f[i] = pl[i * P];
+        if constexpr (WIDE) {  // k is uniform over a warp: no products with 1 or 0
+            if (k == 0)
+                sum = moment_sum<0>(c.vr[s], c.qr[s], f);
+            else if (k == 1)
+                sum = moment_sum<1>(c.vr[s], c.qr[s], f);
+            else if (k == 2)
+                sum = moment_sum<2>(c.vr[s], c.qr[s], f);
+            else
+                sum = moment_sum<3>(c.vr[s], c.qr[s], f);
         } else {
-            ux[s] = jx / sn;
-            uy[s] = jy / sn;
-            Ts[s] = c.m[s] * (se / sn - (ux[s] * ux[s] + uy[s] * uy[s])) / (2.0 + c.I[s]);
+            sum = 0.0;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const double v = c.vr[s][i >> 2], q = c.qr[s][i >> 2];
+                const double wx = dir_x(i) == 0 ? 0.0 : dir_x(i) * v, wy = dir_y(i) == 0 ? 0.0 : dir_y(i) * v;
+                sum += f[i] * (k == 0 ? 1.0 : k == 1 ? wx : k == 2 ? wy : q);
+            }
+        }
+        mom[(s * 4 + k) * CELLS + j] = sum;
+    }
+    __syncthreads();
+
+    // 2. species velocities and the weights of the mixture sums
+#pragma unroll 1
+    for (int it = tid; it < S * CELLS; it += NT) {
+        const int j = it % CELLS, s = it / CELLS;
+        const double *mo = mom + s * 4 * CELLS + j;
+        double *w = wts + s * W_N * CELLS + j;
+        const double sn = mo[0], E = mo[3 * CELLS];
+        double ux = 0.0, uy = 0.0, Ts = 0.0;  // an absent species: zero velocity and temperature
+        if (sn != 0.0) {
+            ux = mo[CELLS] / sn;
+            uy = mo[2 * CELLS] / sn;
+            if (force) Ts = c.md[s].b * (E / sn - (ux * ux + uy * uy)) / (2.0 + c.I[s]);
+        }
+        const double rho = c.md[s].b * sn;
+        w[W_RHO * CELLS] = rho;
+        w[W_LAM * CELLS] = div_by(rho, c.taud[s]);
+        w[W_LX * CELLS] = div_by(rho * ux, c.taud[s]);
+        w[W_LY * CELLS] = div_by(rho * uy, c.taud[s]);
+        w[W_ME * CELLS] = c.md[s].b * E;
+        w[W_CAP * CELLS] = div_by(sn * (2.0 + c.I[s]), c.taud[s]);
+        if (force) {
+            w[W_UX * CELLS] = ux;
+            w[W_UY * CELLS] = uy;
+            w[W_TS * CELLS] = Ts;
         }
     }
-    double w = 0.0, wx = 0.0, wy = 0.0, ntot = 0.0;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-        const double rho = c.m[s] * n[s];
-        w += rho / c.tau[s];
-        wx += rho * ux[s] / c.tau[s];
-        wy += rho * uy[s] / c.tau[s];
-        ntot += fabs(n[s]);
-    }
-    const double Ux = wx / w, Uy = wy / w;
-    const double u2 = Ux * Ux + Uy * Uy;
-    double num = 0.0, den = 0.0;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-        const double rho = c.m[s] * n[s];
-        num += (c.m[s] * E[s] - rho * u2) / c.tau[s];
-        den += n[s] * (2.0 + c.I[s]) / c.tau[s];
-    }
-    const double T = num / den;
+    __syncthreads();
 
-    unsigned bad = 0;
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-        if (!(n[s] >= -1e-6 * ntot) || !isfinite(n[s])) bad |= DBM_HEALTH_DENSITY;
-    if (!(ntot > 0.0)) bad |= DBM_HEALTH_DENSITY;
-    if (!(T > 0.0)) bad |= DBM_HEALTH_TEMPERATURE;
-    if (!isfinite(T) || !isfinite(Ux) || !isfinite(Uy)) bad |= DBM_HEALTH_NONFINITE;
-
-    double omega = 0.0, dTdt = 0.0;
-    if (c.has_reaction) {
-        omega = c.k_ov * n[c.fuel] * n[c.oxid] * exp(-c.Ea_over_R / T);
-        double src = 0.0, cap = 0.0;
+    // 3. mixture velocity and temperature, reaction rate
+    if (tid < CELLS) {
+        const int j = tid;
+        const double *mo = mom + j, *w = wts + j;
+        double sw = 0.0, sx = 0.0, sy = 0.0, ntot = 0.0;
 #pragma unroll
         for (int s = 0; s < S; ++s) {
-            src += (2.0 + c.I[s]) * c.a[s] * omega;
-            cap += n[s] * (2.0 + c.I[s]);
+            sw += w[(s * W_N + W_LAM) * CELLS];
+            sx += w[(s * W_N + W_LX) * CELLS];
+            sy += w[(s * W_N + W_LY) * CELLS];
+            ntot += fabs(mo[s * 4 * CELLS]);
         }
-        dTdt = (c.Qheat * omega - 0.5 * T * src) / (0.5 * cap);
-    }
-
-    const Images im = cell_images(x, y, c.nx, c.ny, c.bc_x, c.bc_y);
-#pragma unroll 1
-    for (int s = 0; s < S; ++s) {
-        const double tau = c.tau[s];
-        double feq[Q], feq_r[Q], g1[Q], g0[Q];
-        feq_printed<S>(c, s, n[s], Ux, Uy, T, feq);
-        const bool react = c.has_reaction != 0, force = c.has_force != 0;
+        const double Ux = sx / sw, Uy = sy / sw;
+        const double u2 = Ux * Ux + Uy * Uy;
+        double num = 0.0, den = 0.0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            num += div_by(w[(s * W_N + W_ME) * CELLS] - w[(s * W_N + W_RHO) * CELLS] * u2, c.taud[s]);
+            den += w[(s * W_N + W_CAP) * CELLS];
+        }
+        const double T = num / den;
+        unsigned bad = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const double n = mo[s * 4 * CELLS];
+            if (!(n >= -1e-6 * ntot) || !isfinite(n)) bad |= DBM_HEALTH_DENSITY;
+        }
+        if (!(ntot > 0.0)) bad |= DBM_HEALTH_DENSITY;
+        if (!(T > 0.0)) bad |= DBM_HEALTH_TEMPERATURE;
+        if (!isfinite(T) || !isfinite(Ux) || !isfinite(Uy)) bad |= DBM_HEALTH_NONFINITE;
+        double omega = 0.0, dTdt = 0.0;
         if (react) {
-            const double nstar = n[s] + tau * c.a[s] * omega;
-            const double Tstar = T + tau * dTdt;
-            if (nstar < -1e-6 * ntot) bad |= DBM_HEALTH_NSTAR;
-            feq_printed<S>(c, s, nstar, Ux, Uy, Tstar, feq_r);
+            omega = c.k_ov * mo[c.fuel * 4 * CELLS] * mo[c.oxid * 4 * CELLS] * exp(-c.Ea_over_R / T);
+            double src = 0.0, cap = 0.0;
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+                src += (2.0 + c.I[s]) * c.a[s] * omega;
+                cap += mo[s * 4 * CELLS] * (2.0 + c.I[s]);
+            }
+            dTdt = (c.Qheat * omega - 0.5 * T * src) / (0.5 * cap);
+        }
+        mix[M_UX * CELLS + j] = Ux;
+        mix[M_UY * CELLS + j] = Uy;
+        mix[M_T * CELLS + j] = T;
+        mix[M_NTOT * CELLS + j] = ntot;
+        mix[M_OMEGA * CELLS + j] = omega;
+        mix[M_DT * CELLS + j] = dTdt;
+        if (bad) raise_flag(flag, bad);
+    }
+    __syncthreads();
+
+    // 4. f-hat of each term: set 0 (n, u, T), then with a reaction (n*, u, T*),
+    // then with a force (n, u-dagger, T^s) and (n, u^s, T^s)
+    constexpr int SET = S * Q * CELLS;
+#pragma unroll 1
+    for (int it = tid; it < S * CELLS; it += NT) {
+        const int j = it % CELLS, s = it / CELLS;
+        const double n = mom[s * 4 * CELLS + j];
+        const double Ux = mix[M_UX * CELLS + j], Uy = mix[M_UY * CELLS + j], T = mix[M_T * CELLS + j];
+        double *fh = fhs + s * Q * CELLS + j;
+        fhat_printed(n, Ux, Uy, T, c.md[s], c.I[s], fh, CELLS);
+        if (react) {
+            const double tau = c.taud[s].b;
+            const double nstar = n + tau * c.a[s] * mix[M_OMEGA * CELLS + j];
+            const double Tstar = T + tau * mix[M_DT * CELLS + j];
+            if (nstar < -1e-6 * mix[M_NTOT * CELLS + j]) raise_flag(flag, DBM_HEALTH_NSTAR);
+            fh += SET;
+            fhat_printed(nstar, Ux, Uy, Tstar, c.md[s], c.I[s], fh, CELLS);
         }
         if (force) {
-            feq_printed<S>(c, s, n[s], ux[s] + c.ax * tau, uy[s] + c.ay * tau, Ts[s], g1);
-            feq_printed<S>(c, s, n[s], ux[s], uy[s], Ts[s], g0);
-        }
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const double *pl = fin + (s * Q + i) * P;
-            const double f = pl[cell];
-            double rhs = -(f - feq[i]) / tau;                   // Omega
-            if (react) rhs = rhs + (feq_r[i] - feq[i]) / tau;   // R
-            if (force) rhs = rhs + (g1[i] - g0[i]) / tau;       // G
-            double adv = 0.0;
-            if (dir_x(i) != 0)
-                adv += nnd_dflux(c.vx[s][i], pl[cell - 2], pl[cell - 1], f, pl[cell + 1], pl[cell + 2], c.dx);
-            if (dir_y(i) != 0)
-                adv += nnd_dflux(c.vy[s][i], pl[cell - 2 * py], pl[cell - py], f, pl[cell + py], pl[cell + 2 * py],
-                                 c.dy);
-            const double fnew = f + c.dt * (rhs - adv);
-            store_with_images(fout + (s * Q + i) * P, cell, x, y, c.pitch, im, fnew);
+            const double tau = c.taud[s].b;
+            const double *w = wts + s * W_N * CELLS + j;
+            const double ux = w[W_UX * CELLS], uy = w[W_UY * CELLS], Ts = w[W_TS * CELLS];
+            fh += SET;
+            fhat_printed(n, ux + c.ax * tau, uy + c.ay * tau, Ts, c.md[s], c.I[s], fh, CELLS);
+            fh += SET;
+            fhat_printed(n, ux, uy, Ts, c.md[s], c.I[s], fh, CELLS);
         }
     }
-    if (bad) raise_flag(flag, bad);
+    __syncthreads();
+
+    // 5. collision, advection and update of one ring per warp
+    const int warp = tid >> 5, lane = tid & 31, r = warp & 3;
+    const int j = lane % CELLS, vel = lane / CELLS;  // vel: 0 when the thread takes all four
+    unsigned x, y;
+    const long long cell = locate(j, x, y);
+    const bool live = d0 + (unsigned)j < total;
+    const unsigned mx = ghost_mask((int)x, c.nx, c.bc_x), my = ghost_mask((int)y, c.ny, c.bc_y);
+    auto ring_step = [&](auto diag_tag, int s) {
+        constexpr bool DIAG = decltype(diag_tag)::value;
+        const double *row = c.row[s][r];
+        const ConstDiv tau = c.taud[s];
+        const double v = c.vr[s][r];
+        double feq[V], rhs[V], f[V], e1[V], e0[V];
+#pragma unroll
+        for (int q = 0; q < V; ++q) f[q] = fin[(s * Q + 4 * r + (V == 4 ? q : vel)) * P + cell];
+        const double *fh = fhs + s * Q * CELLS + j;
+        ring_equilibrium<DIAG, V, CELLS>(row, fh, vel, feq);
+#pragma unroll
+        for (int q = 0; q < V; ++q) rhs[q] = div_by(-(f[q] - feq[q]), tau);  // Omega
+        if (react) {
+            fh += SET;
+            ring_equilibrium<DIAG, V, CELLS>(row, fh, vel, e1);
+#pragma unroll
+            for (int q = 0; q < V; ++q) rhs[q] = rhs[q] + div_by(e1[q] - feq[q], tau);  // R
+        }
+        if (force) {
+            ring_equilibrium<DIAG, V, CELLS>(row, fh + SET, vel, e1);
+            ring_equilibrium<DIAG, V, CELLS>(row, fh + 2 * SET, vel, e0);
+#pragma unroll
+            for (int q = 0; q < V; ++q) rhs[q] = rhs[q] + div_by(e1[q] - e0[q], tau);  // G
+        }
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const int i = V == 4 ? q : vel;
+            const long long plane = (long long)(s * Q + 4 * r + i) * P;
+            const double *pl = fin + plane + cell;
+            const double g0 = v * f[q];
+            double adv;
+            if constexpr (DIAG) {
+                const int ex = (i == 1 || i == 2) ? -1 : 1, ey = (i == 2 || i == 3) ? -c.pitch : c.pitch;
+                adv = nnd_dflux(pl[-2 * ex], pl[-ex], pl[ex], g0, v, c.dxd);
+                adv += nnd_dflux(pl[-2 * ey], pl[-ey], pl[ey], g0, v, c.dyd);
+            } else {
+                const int st = (i & 1) ? c.pitch : 1, e = (i & 2) ? -st : st;
+                adv = nnd_dflux(pl[-2 * e], pl[-e], pl[e], g0, v, (i & 1) ? c.dyd : c.dxd);
+            }
+            const double fnew = f[q] + c.dt * (rhs[q] - adv);
+            if (!live) continue;
+            double *po = fout + plane;
+            po[cell] = fnew;
+            if (mx | my) store_images(po, (int)x, (int)y, c.nx, c.ny, c.pitch, mx, my, fnew);
+        }
+    };
+#pragma unroll 1
+    for (int s = warp >> 2; s < S; s += SW) {
+        if (r & 1)
+            ring_step(std::true_type{}, s);
+        else
+            ring_step(std::false_type{}, s);
+    }
+}
+
+// Grids of up to this many cells take the 8-cell split.
+// Grids of up to this many cells, two 8-cell CTAs per SM, take the 8-cell
+// split (us a step, 8-cell / 32-cell: two species 2048 cells 22.8 / 29.0, 4096
+// cells 33.1 / 29.0; four species under a force 59.7 / 74.1, 114 / 74.1).
+constexpr long long NARROW_CELLS = 16 * 152;
+
+template <int S, bool WIDE>
+static int launch_f64_v(dbm_handle *h, const double *fin, double *fout, cudaStream_t st)
+{
+    constexpr int CELLS = WIDE ? 32 : 8;
+    F64Consts<S> c;
+    fill_f64_consts<S>(h, c);
+    const int sets = 1 + (c.has_reaction ? 1 : 0) + (c.has_force ? 2 : 0);
+    const size_t smem = f64_smem<S>(CELLS, sets);
+    if (smem > 48 * 1024) {
+        static bool attr_set = false;  // per instantiation, set once per process
+        if (!attr_set) {
+            cudaError_t e = cudaFuncSetAttribute(k_step_f64<S, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)f64_smem<S>(CELLS, 4));
+            if (e != cudaSuccess) return set_cuda_error(h, e, "FP64 step kernel shared-memory attribute");
+            attr_set = true;
+        }
+    }
+    const long long cells = (long long)h->p.nx * h->p.ny;
+    k_step_f64<S, WIDE><<<(unsigned)((cells + CELLS - 1) / CELLS), 128 * f64_side(S), smem, st>>>(
+        c, fin, fout, (unsigned *)h->scratch);
+    return set_cuda_error(h, cudaGetLastError(), "FP64 step kernel launch");
 }
 
 template <int S>
 static int launch_f64_t(dbm_handle *h, const double *fin, double *fout, cudaStream_t st)
 {
-    F64Consts<S> c;
-    fill_f64_consts<S>(h, c);
-    dim3 block(32, 4);
-    dim3 grid((h->p.nx + 31) / 32, (h->p.ny + 3) / 4);
-    k_step_f64<S><<<grid, block, 0, st>>>(c, fin, fout, (unsigned *)h->scratch);
-    return set_cuda_error(h, cudaGetLastError(), "FP64 step kernel launch");
+    if ((long long)h->p.nx * h->p.ny <= NARROW_CELLS) return launch_f64_v<S, false>(h, fin, fout, st);
+    return launch_f64_v<S, true>(h, fin, fout, st);
 }
 
 int launch_step_f64(dbm_handle *h, int cur, cudaStream_t st)
