@@ -26,25 +26,6 @@ __device__ __forceinline__ void images_of_planes(T *f, long long plane, int npla
     for (int p = 0; p < nplanes; ++p) store_images(f + p * plane, x, y, nx, ny, pitch, mx, my, f[p * plane + cell]);
 }
 
-// (double)x on the integer pipe.  The conversion instruction shares the FP64
-// pipe, two lanes per SM and cycle here, and the output kernels convert every
-// value they read or write: exponent and mantissa are moved over instead
-// (k_moments_f32: half its time; k_get_f on 4096^2: 1.05 -> 0.99 ms).
-// Zeros keep their sign; subnormal, infinite and NaN values take the
-// instruction.
-__device__ __forceinline__ bool widens_by_bits(float x)
-{
-    const unsigned a = __float_as_uint(x) & 0x7fffffffu;
-    return a - 1u >= 0x007fffffu && a < 0x7f800000u;
-}
-__device__ __forceinline__ double widen_bits(float x)
-{
-    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
-    const unsigned hi = a == 0u ? u : (u & 0x80000000u) | ((a >> 3) + 0x38000000u);
-    return __hiloint2double((int)hi, (int)(u << 29));
-}
-__device__ __forceinline__ double widen(float x) { return widens_by_bits(x) ? widen_bits(x) : (double)x; }
-
 // f = f^eq(rho^s / m^s, u, T), computed in FP64 and rounded to `real`.
 template <typename real, int S>
 __global__ void __launch_bounds__(256)

@@ -90,13 +90,11 @@ __host__ __device__ inline unsigned mix32(unsigned x)
     return x;
 }
 
-template <int S>
-void fill_acc_consts(const dbm_handle *h, const StepConsts<float, S> &c, AccConsts<S> &a)
+template <int S, int MODE>
+void fill_acc_consts(const dbm_handle *h, const StepConsts<float, S> &c, AccConsts<S, MODE> &a)
 {
     memset(&a, 0, sizeof(a));
     const dbm_params &p = h->p;
-    a.thermo64 = p.thermo == DBM_THERMO_FP64;
-    a.stochastic = p.rounding == DBM_ROUND_STOCHASTIC;
     a.seed = mix32((unsigned)h->steps * 0x9e3779b9u + 0x632be5abu) ^ mix32((unsigned)(h->steps >> 32));
     double src = 0.0;
     for (int s = 0; s < S; ++s) {

@@ -64,16 +64,17 @@ struct StepConsts {
 };
 
 // Extra kernel parameters of the FP32 step with its arithmetic options
-// (dbm_params.thermo, dbm_params.rounding): the run-time switches, the
-// seed of the stochastic rounding for this launch, and the constants of the
-// FP64 moment and rate evaluation (the float constants of StepConsts
-// widened, so that both evaluations use the same discrete velocities and
-// weights).  NoAcc stands in for it in the default kernels.
-template <int S>
+// (dbm_params.thermo, dbm_params.rounding; MODE: acc_mode): the seed of the
+// stochastic rounding for this launch, and the constants of the FP64 moment
+// and rate evaluation (the float constants of StepConsts widened, so that
+// both evaluations use the same discrete velocities and weights).  NoAcc
+// stands in for it in the default kernels.
+constexpr int ACC_THERMO64 = 1, ACC_STOCHASTIC = 2;
+template <int S, int MODE>
 struct AccConsts {
     static constexpr bool on = true;
-    int thermo64;    // DBM_THERMO_FP64
-    int stochastic;  // DBM_ROUND_STOCHASTIC
+    static constexpr bool thermo64 = (MODE & ACC_THERMO64) != 0;      // DBM_THERMO_FP64
+    static constexpr bool stochastic = (MODE & ACC_STOCHASTIC) != 0;  // DBM_ROUND_STOCHASTIC
     unsigned seed;   // per launch: hash of the handle's step count
     double vr[S][4], qr[S][4];  // ring speeds and v.v + eta^2, as the float step uses them
     double lam[S], kap[S];      // mixture weights m dt_tau and lam dpi / m
@@ -81,7 +82,7 @@ struct AccConsts {
     double k_ov, Ea_over_R, Qheat, src;
 };
 struct NoAcc {
-    static constexpr bool on = false;
+    static constexpr bool on = false, thermo64 = false, stochastic = false;
 };
 
 // Kernel parameters of the FP64 output / initialisation kernels.
@@ -190,13 +191,16 @@ int launch_conservation_noalloc(dbm_handle *h, const void *f, double *out, cudaS
 
 template <typename real, int S>
 void fill_step_consts(const dbm_handle *h, StepConsts<real, S> &c);
-template <int S>
-void fill_acc_consts(const dbm_handle *h, const StepConsts<float, S> &c, AccConsts<S> &a);
-// the FP32 step runs the kernel with the arithmetic options
-inline bool uses_acc(const dbm_params &p)
+template <int S, int MODE>
+void fill_acc_consts(const dbm_handle *h, const StepConsts<float, S> &c, AccConsts<S, MODE> &a);
+// the arithmetic options of the FP32 step, 0 for none
+inline int acc_mode(const dbm_params &p)
 {
-    return p.precision == DBM_FP32 && (p.thermo != DBM_THERMO_FLOATFLOAT || p.rounding != DBM_ROUND_NEAREST);
+    if (p.precision != DBM_FP32) return 0;
+    return (p.thermo != DBM_THERMO_FLOATFLOAT ? ACC_THERMO64 : 0) |
+           (p.rounding != DBM_ROUND_NEAREST ? ACC_STOCHASTIC : 0);
 }
+inline bool uses_acc(const dbm_params &p) { return acc_mode(p) != 0; }
 template <int S>
 void fill_out_consts(const dbm_handle *h, OutConsts<S> &c);
 

@@ -10,7 +10,7 @@ namespace dbm {
 
 template <int S>
 int launch_step_t(dbm_handle *h, const void *fin, void *fout, cudaStream_t st);
-template <int S, int TX, int TY, int CW, bool ACC>
+template <int S, int TX, int TY, int CW, int MODE>
 int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const void *fin, void *fout, cudaStream_t st);
 template <int S, int TX, int TY>
 int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin,
@@ -32,18 +32,18 @@ static int launch_staged(dbm_handle *h, int cur, const void *fin, void *fout, cu
     return DBM_ERR_INVALID;
 }
 
-// The TMA-staged step of the handle's tile, with (ACC) or without the FP32
-// arithmetic options.
-template <bool ACC>
+// The TMA-staged step of the handle's tile with the FP32 arithmetic options
+// MODE (acc_mode).
+template <int MODE>
 static int launch_tma(dbm_handle *h, const CUtensorMap *tm, const void *fin, void *fout, cudaStream_t st)
 {
     switch (h->p.nspecies) {
-    case 1: return launch_step_tma_t<1, tma_tile_x(1), tma_tile_y(1), 1, ACC>(h, tm, fin, fout, st);
+    case 1: return launch_step_tma_t<1, tma_tile_x(1), tma_tile_y(1), 1, MODE>(h, tm, fin, fout, st);
     case 2:
-        if (h->tma_cw == 2) return launch_step_tma_t<2, PAIR_TX, PAIR_TY, 2, ACC>(h, tm, fin, fout, st);
-        return launch_step_tma_t<2, tma_tile_x(2), tma_tile_y(2), 1, ACC>(h, tm, fin, fout, st);
-    case 3: return launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, ACC>(h, tm, fin, fout, st);
-    case 4: return launch_step_tma_t<4, tma_tile_x(4), tma_tile_y(4), 1, ACC>(h, tm, fin, fout, st);
+        if (h->tma_cw == 2) return launch_step_tma_t<2, PAIR_TX, PAIR_TY, 2, MODE>(h, tm, fin, fout, st);
+        return launch_step_tma_t<2, tma_tile_x(2), tma_tile_y(2), 1, MODE>(h, tm, fin, fout, st);
+    case 3: return launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, MODE>(h, tm, fin, fout, st);
+    case 4: return launch_step_tma_t<4, tma_tile_x(4), tma_tile_y(4), 1, MODE>(h, tm, fin, fout, st);
     }
     return DBM_ERR_INVALID;
 }
@@ -162,7 +162,12 @@ int launch_step(dbm_handle *h, int cur, cudaStream_t st)
     if (h->tma_ok && want != DBM_KERNEL_GENERIC) {
         const CUtensorMap *tm = &h->tmap[cur];
         if (h->tma_staged) return launch_staged(h, cur, fin, fout, st);
-        return uses_acc(h->p) ? launch_tma<true>(h, tm, fin, fout, st) : launch_tma<false>(h, tm, fin, fout, st);
+        switch (acc_mode(h->p)) {
+        case 0: return launch_tma<0>(h, tm, fin, fout, st);
+        case 1: return launch_tma<1>(h, tm, fin, fout, st);
+        case 2: return launch_tma<2>(h, tm, fin, fout, st);
+        default: return launch_tma<3>(h, tm, fin, fout, st);
+        }
     }
     if (uses_acc(h->p)) return DBM_ERR_INVALID;  // the options exist in the TMA-staged kernel only
     if (want != DBM_KERNEL_AUTO && want != DBM_KERNEL_GENERIC) return DBM_ERR_INVALID;

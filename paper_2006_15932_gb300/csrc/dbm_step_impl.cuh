@@ -541,8 +541,10 @@ __device__ __forceinline__ void moments_fp64(const X &xa, const Tile &t, int j, 
         double sn = 0.0, sx = 0.0, sy = 0.0, se = 0.0;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const double f0 = L::get(t.ld(s * Q + 4 * r, 0, 0), j), f1 = L::get(t.ld(s * Q + 4 * r + 1, 0, 0), j);
-            const double f2 = L::get(t.ld(s * Q + 4 * r + 2, 0, 0), j), f3 = L::get(t.ld(s * Q + 4 * r + 3, 0, 0), j);
+            const double f0 = widen(L::get(t.ld(s * Q + 4 * r, 0, 0), j));
+            const double f1 = widen(L::get(t.ld(s * Q + 4 * r + 1, 0, 0), j));
+            const double f2 = widen(L::get(t.ld(s * Q + 4 * r + 2, 0, 0), j));
+            const double f3 = widen(L::get(t.ld(s * Q + 4 * r + 3, 0, 0), j));
             const double rs = (f0 + f2) + (f1 + f3);
             double rx, ry;
             if ((r & 1) == 0) {
@@ -668,12 +670,8 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
     using V = typename Tile::V;
     using L = Lanes<V>;
     static_assert(L::n == 1 || Out::kNoImages, "ghost images are written one cell per thread");
-    // arithmetic options (AccConsts): run-time switches of the option kernel
-    bool t64 = false, sr = false;
-    if constexpr (X::on) {
-        t64 = xa.thermo64 != 0;
-        sr = xa.stochastic != 0;
-    }
+    // arithmetic options, compiled in (AccConsts)
+    constexpr bool t64 = X::thermo64, sr = X::stochastic;
 
     constexpr bool kStaged = is_staged<Tile>::value;
     static_assert(!(kStaged && X::on), "the arithmetic options read every species at once");
@@ -1265,8 +1263,11 @@ __device__ __forceinline__ void halo_store(const HaloRegs<NP, TX, TY, NT> &hr, c
     __syncthreads();
 }
 
-// X: NoAcc for the default arithmetic, AccConsts<S> for the kernel with the
-// thermo and rounding options.
+// X: NoAcc for the default arithmetic, AccConsts<S, MODE> for a kernel with the
+// thermo or rounding option or both.  One kernel per combination: with the
+// options as run-time switches of one kernel, stochastic rounding alone
+// carried the FP64 thermo's registers and code (1024 x 256, three species, us
+// a step: stochastic 81 -> 54, FP64 thermo 163 -> 149, both 197 -> 173).
 template <int S, int TX, int TY, int CW, class X>
 __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     k_step_tma(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
@@ -1326,11 +1327,11 @@ int launch_step_t(dbm_handle *h, const void *fin, void *fout, cudaStream_t st)
     return set_cuda_error(h, cudaGetLastError(), "step kernel launch");
 }
 
-// ACC: the kernel with the thermo and rounding options (AccConsts).
-template <int S, int TX, int TY, int CW, bool ACC>
+// MODE: the thermo and rounding options (acc_mode), 0 for none.
+template <int S, int TX, int TY, int CW, int MODE>
 int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const void *fin, void *fout, cudaStream_t st)
 {
-    using X = typename std::conditional<ACC, AccConsts<S>, NoAcc>::type;
+    using X = typename std::conditional<MODE != 0, AccConsts<S, MODE>, NoAcc>::type;
     constexpr size_t smem = (size_t)(TX + 8) * (TY + 4) * S * Q * sizeof(float);
     static bool attr_set = false;  // per instantiation, set once per process
     if (!attr_set) {
@@ -1342,7 +1343,7 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const void *fin, v
     StepConsts<float, S> c;
     fill_step_consts<float, S>(h, c);
     X xa{};
-    if constexpr (ACC) fill_acc_consts<S>(h, c, xa);
+    if constexpr (MODE != 0) fill_acc_consts<S, MODE>(h, c, xa);
     dim3 block(TX / CW, TY);
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
     k_step_tma<S, TX, TY, CW, X><<<grid, block, smem, st>>>(c, *tmap, (const float *)fin, (float *)fout,
