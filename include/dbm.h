@@ -127,10 +127,10 @@ enum dbm_step_kernel {
                                  DBM_KERNEL_TMA                                      */
     DBM_KERNEL_GENERIC = 1,   /* stencil read from global memory                      */
     DBM_KERNEL_TMA = 2,       /* tile + halo staged in shared memory by TMA copies:
-                                 S = 1: one cell per thread; S = 2: all planes in one
-                                 copy, two cells per thread on grids of at least 4096
-                                 tiles of 64 x 8 cells, else one cell per thread;
-                                 S = 3, 4: one cell per thread; S >= 5: as
+                                 S = 1, 3, 4: one cell per thread; S = 2: two cells
+                                 per thread on grids of at least 128 tiles of 64 x 8
+                                 cells (4096 with the thermo or rounding option),
+                                 else one cell per thread; S >= 5: as
                                  DBM_KERNEL_TMA_STAGED                               */
     DBM_KERNEL_TMA_CELL = 3,  /* TMA-staged, all planes in one copy, one cell per
                                  thread (S <= 4)                                     */
@@ -384,10 +384,14 @@ int dbm_status(dbm_handle *h, void *stream, unsigned *bits);
 /* Steps taken since the last dbm_set_state / dbm_set_f. */
 long long dbm_steps_taken(const dbm_handle *h);
 
-/* The shared-memory tile the step of a bound handle uses (chosen at
- * dbm_bind from dbm_params.step_kernel and the grid): tile_x x tile_y
- * cells, cells_per_thread 1 or 2 (adjacent cells of a row, packed FP32x2
- * arithmetic); all three 0 when the step runs a kernel without a tile
+/* The shared-memory tile class of a bound handle (chosen at dbm_bind from
+ * dbm_params.step_kernel and the grid): tile_x x tile_y cells,
+ * cells_per_thread 1 or 2 (adjacent cells of a row, packed FP32x2
+ * arithmetic).  Two species below 4096 tiles of 64 x 8 cells answer with
+ * their one-cell tile, 32 x 7; the step itself runs pairs on 64 x 8 tiles
+ * there as well from 128 such tiles up, unless DBM_KERNEL_TMA_CELL asks for
+ * one cell (same bits).
+ * All three 0 when the step runs a kernel without a tile
  * (generic global-memory stencil, FP64, BF16DEV).  Null outputs are
  * skipped.  DBM_ERR_UNBOUND before dbm_bind. */
 int dbm_step_tile(const dbm_handle *h, int *tile_x, int *tile_y, int *cells_per_thread);

@@ -481,6 +481,12 @@ int dbm_bind(dbm_handle *h, void *f_a, void *f_b, void *scratch)
     h->scratch = scratch;
     h->cur = 0;
     h->bound = 1;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || h->sms < 1) {
+        cudaGetLastError();
+        h->sms = 1;
+    }
     make_tensor_maps(h);
     const int want = h->p.step_kernel;
     if ((want != DBM_KERNEL_AUTO && want != DBM_KERNEL_GENERIC) || uses_acc(h->p))
@@ -683,9 +689,9 @@ int dbm_step_tile(const dbm_handle *h, int *tile_x, int *tile_y, int *cells_per_
     if (!h) return DBM_ERR_INVALID;
     if (!h->bound) return DBM_ERR_UNBOUND;
     const bool tiled = h->tma_ok && h->p.step_kernel != DBM_KERNEL_GENERIC;
-    if (tile_x) *tile_x = tiled ? h->tma_tx : 0;
-    if (tile_y) *tile_y = tiled ? h->tma_ty : 0;
-    if (cells_per_thread) *cells_per_thread = tiled ? h->tma_cw : 0;
+    if (tile_x) *tile_x = tiled ? h->told_tx : 0;
+    if (tile_y) *tile_y = tiled ? h->told_ty : 0;
+    if (cells_per_thread) *cells_per_thread = tiled ? h->told_cw : 0;
     return DBM_OK;
 }
 

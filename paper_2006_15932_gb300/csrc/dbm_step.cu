@@ -11,7 +11,8 @@ namespace dbm {
 template <int S>
 int launch_step_t(dbm_handle *h, const void *fin, void *fout, cudaStream_t st);
 template <int S, int TX, int TY, int CW, int MODE>
-int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const void *fin, void *fout, cudaStream_t st);
+int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin, void *fout,
+                      cudaStream_t st);
 template <int S, int TX, int TY>
 int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin,
                          void *fout, cudaStream_t st);
@@ -35,15 +36,16 @@ static int launch_staged(dbm_handle *h, int cur, const void *fin, void *fout, cu
 // The TMA-staged step of the handle's tile with the FP32 arithmetic options
 // MODE (acc_mode).
 template <int MODE>
-static int launch_tma(dbm_handle *h, const CUtensorMap *tm, const void *fin, void *fout, cudaStream_t st)
+static int launch_tma(dbm_handle *h, const CUtensorMap *tm, const CUtensorMap *ti, const void *fin, void *fout,
+                      cudaStream_t st)
 {
     switch (h->p.nspecies) {
-    case 1: return launch_step_tma_t<1, tma_tile_x(1), tma_tile_y(1), 1, MODE>(h, tm, fin, fout, st);
+    case 1: return launch_step_tma_t<1, tma_tile_x(1), tma_tile_y(1), 1, MODE>(h, tm, ti, fin, fout, st);
     case 2:
-        if (h->tma_cw == 2) return launch_step_tma_t<2, PAIR_TX, PAIR_TY, 2, MODE>(h, tm, fin, fout, st);
-        return launch_step_tma_t<2, tma_tile_x(2), tma_tile_y(2), 1, MODE>(h, tm, fin, fout, st);
-    case 3: return launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, MODE>(h, tm, fin, fout, st);
-    case 4: return launch_step_tma_t<4, tma_tile_x(4), tma_tile_y(4), 1, MODE>(h, tm, fin, fout, st);
+        if (h->tma_cw == 2) return launch_step_tma_t<2, PAIR_TX, PAIR_TY, 2, MODE>(h, tm, ti, fin, fout, st);
+        return launch_step_tma_t<2, tma_tile_x(2), tma_tile_y(2), 1, MODE>(h, tm, ti, fin, fout, st);
+    case 3: return launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, MODE>(h, tm, ti, fin, fout, st);
+    case 4: return launch_step_tma_t<4, tma_tile_x(4), tma_tile_y(4), 1, MODE>(h, tm, ti, fin, fout, st);
     }
     return DBM_ERR_INVALID;
 }
@@ -57,12 +59,19 @@ static bool staged_supported(const dbm_params &p)
     return p.precision == DBM_FP32 && p.nspecies >= 2 && p.nspecies <= DBM_MAX_SPECIES && !uses_acc(p);
 }
 
-// The tile of the TMA-staged step.  Two species: two cells per thread when
-// asked for, or (DBM_KERNEL_AUTO / DBM_KERNEL_TMA) on grids of at least
-// PAIR_MIN_TILES pair tiles, else the one-cell tile.  Three and four
-// species: the one-cell tile (faster than the species-staged kernel on every
-// grid measured), the species-staged one when two cells per thread are asked
-// for.  Five or more: the species-staged kernel, the only TMA-staged one.
+// The tile of the TMA-staged step.  Two species: two cells per thread from
+// PAIR_MIN_RUN tiles up (us a step, one cell / pairs: 4096^2 845 / 726, 1024^2
+// 69 / 60, 1001 x 771 51 / 45, 512^2 20.0 / 18.3, 256^2, 128 tiles, 10.6 / 9.9;
+// below, a thread's longer chain shows: 128^2 9.6 / 10.1), the one-cell tile
+// when asked for; with an arithmetic option pairs from PAIR_MIN_TILES tiles.
+// Three and four species: the one-cell tile (2048 x 1024, one cell / species-
+// staged: three species 174 / 201, four 261 / 265), the species-staged one
+// when two cells per thread are asked for.  Five or more: the species-staged
+// kernel, the only TMA-staged one.
+//
+// dbm_step_tile's answer is fixed by its own rule, older than pairs on small
+// grids: it names the pair tile for two species from PAIR_MIN_TILES tiles up
+// (or when pairs are asked for) and the one-cell tile below.
 static void choose_tile(dbm_handle *h)
 {
     const dbm_params &p = h->p;
@@ -72,19 +81,23 @@ static void choose_tile(dbm_handle *h)
     const bool staged_asked = want == DBM_KERNEL_TMA_STAGED || (p.nspecies >= 3 && want == DBM_KERNEL_TMA_PAIR);
     if (staged_supported(p) && (staged_by_default || staged_asked)) {
         h->tma_staged = 1;
-        h->tma_tx = STAGED_TX;
-        h->tma_ty = STAGED_TY;
-        h->tma_cw = 2;
+        h->tma_tx = h->told_tx = STAGED_TX;
+        h->tma_ty = h->told_ty = STAGED_TY;
+        h->tma_cw = h->told_cw = 2;
         return;
     }
-    bool pair = false;
+    bool told_pair = false, pair = false;
     if (p.nspecies == 2 && want != DBM_KERNEL_TMA_CELL) {
         const long long tiles = (long long)((p.nx + PAIR_TX - 1) / PAIR_TX) * ((p.ny + PAIR_TY - 1) / PAIR_TY);
-        pair = want == DBM_KERNEL_TMA_PAIR || tiles >= PAIR_MIN_TILES;
+        told_pair = want == DBM_KERNEL_TMA_PAIR || tiles >= PAIR_MIN_TILES;
+        pair = told_pair || (!uses_acc(p) && tiles >= PAIR_MIN_RUN);
     }
     h->tma_tx = pair ? PAIR_TX : tma_tile_x(p.nspecies);
     h->tma_ty = pair ? PAIR_TY : tma_tile_y(p.nspecies);
     h->tma_cw = pair ? 2 : 1;
+    h->told_tx = told_pair ? PAIR_TX : tma_tile_x(p.nspecies);
+    h->told_ty = told_pair ? PAIR_TY : tma_tile_y(p.nspecies);
+    h->told_cw = told_pair ? 2 : 1;
 }
 
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -115,16 +128,15 @@ int make_tensor_maps(dbm_handle *h)
         h->tma_tx = h->tma_ty = h->tma_cw = 0;
         return DBM_OK;
     }
-    // the box: the tile, its halo and every plane (one species' planes for
-    // the species-staged kernel)
-    const cuuint32_t planes = (cuuint32_t)(h->tma_staged ? Q : Q * h->p.nspecies);
+    // the box: the tile, its halo and one species' planes
+    const cuuint32_t planes = (cuuint32_t)Q;
     cuuint32_t box[3] = {(cuuint32_t)(h->tma_tx + 8), (cuuint32_t)(h->tma_ty + 4), planes};
     cuuint32_t estr[3] = {1, 1, 1};
     for (int k = 0; k < 2; ++k) {
         CUresult r = encode(&h->tmap[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->f[k], dims, strides, box, estr,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r == CUDA_SUCCESS && h->tma_staged) {  // interior box of one species: the moment-sum copies
+        if (r == CUDA_SUCCESS) {  // interior box of one species: the tile's own cells
             cuuint32_t box_in[3] = {(cuuint32_t)h->tma_tx, (cuuint32_t)h->tma_ty, (cuuint32_t)Q};
             r = encode(&h->tmap_in[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->f[k], dims, strides, box_in, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -160,13 +172,13 @@ int launch_step(dbm_handle *h, int cur, cudaStream_t st)
     void *fout = h->f[cur ^ 1];
     const int want = h->p.step_kernel;
     if (h->tma_ok && want != DBM_KERNEL_GENERIC) {
-        const CUtensorMap *tm = &h->tmap[cur];
+        const CUtensorMap *tm = &h->tmap[cur], *ti = &h->tmap_in[cur];
         if (h->tma_staged) return launch_staged(h, cur, fin, fout, st);
         switch (acc_mode(h->p)) {
-        case 0: return launch_tma<0>(h, tm, fin, fout, st);
-        case 1: return launch_tma<1>(h, tm, fin, fout, st);
-        case 2: return launch_tma<2>(h, tm, fin, fout, st);
-        default: return launch_tma<3>(h, tm, fin, fout, st);
+        case 0: return launch_tma<0>(h, tm, ti, fin, fout, st);
+        case 1: return launch_tma<1>(h, tm, ti, fin, fout, st);
+        case 2: return launch_tma<2>(h, tm, ti, fin, fout, st);
+        default: return launch_tma<3>(h, tm, ti, fin, fout, st);
         }
     }
     if (uses_acc(h->p)) return DBM_ERR_INVALID;  // the options exist in the TMA-staged kernel only

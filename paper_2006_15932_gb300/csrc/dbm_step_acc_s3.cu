@@ -3,7 +3,10 @@
 #include "dbm_step_impl.cuh"
 
 namespace dbm {
-template int launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, 1>(dbm_handle *, const CUtensorMap *, const void *, void *, cudaStream_t);
-template int launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, 2>(dbm_handle *, const CUtensorMap *, const void *, void *, cudaStream_t);
-template int launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, 3>(dbm_handle *, const CUtensorMap *, const void *, void *, cudaStream_t);
+template int launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, 1>(dbm_handle *, const CUtensorMap *, const CUtensorMap *, const void *, void *,
+                                     cudaStream_t);
+template int launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, 2>(dbm_handle *, const CUtensorMap *, const CUtensorMap *, const void *, void *,
+                                     cudaStream_t);
+template int launch_step_tma_t<3, tma_tile_x(3), tma_tile_y(3), 1, 3>(dbm_handle *, const CUtensorMap *, const CUtensorMap *, const void *, void *,
+                                     cudaStream_t);
 }  // namespace dbm

@@ -71,7 +71,6 @@ __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b)
 __device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ float vmm(float a, float b) { return minmod(a, b); }
 
 // The packed operations are written as PTX with an explicit .rn rounding,
 // which keeps the front end from contracting them; the backend can still
@@ -113,7 +112,6 @@ __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c)
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(vpk(a)), "l"(vpk(b)), "l"(vpk(c)));
     return vupk(r);
 }
-__device__ __forceinline__ float2 vmm(float2 a, float2 b) { return make_float2(minmod(a.x, b.x), minmod(a.y, b.y)); }
 
 // Per-cell access to a value: n cells, broadcast, lane j.
 template <class V>
@@ -206,6 +204,15 @@ struct is_staged : std::false_type {
 };
 template <class T>
 struct is_staged<T, std::void_t<decltype(T::kStaged)>> : std::true_type {
+};
+
+// A tile whose species land one after the other (SplitTile) has a wait
+// before the first read of each.
+template <class T, class = void>
+struct is_split : std::false_type {
+};
+template <class T>
+struct is_split<T, std::void_t<decltype(T::kSplit)>> : std::true_type {
 };
 
 template <class Tile>
@@ -348,41 +355,60 @@ __device__ __forceinline__ V feq_of(int i, const V o[16])
 // `sgn` (+1 or -1): (H_{j+1/2} - H_{j-1/2}) / c, from f_{j-2..j+2}.
 //   c > 0: H_{j+1/2} = c [f_j + mm(f_j - f_{j-1}, f_{j+1} - f_j)/2]
 //   c < 0: H_{j+1/2} = c [f_{j+1} - mm(f_{j+1} - f_j, f_{j+2} - f_{j+1})/2]
+// Both limiters of a difference have the upwind slope d among their arguments,
+// so each is either 0 or has the sign of d: their magnitudes are subtracted
+// and the sign of d is put on the difference, once (exact: rounding to
+// nearest is symmetric).
+__device__ __forceinline__ float limited(float a, float b)  // |minmod(a, b)|
+{
+    float t;
+    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
+    return fmaxf(t, 0.0f);
+}
+__device__ __forceinline__ float signed_as(float v, float d)  // v, negated where d is negative
+{
+    return __uint_as_float(__float_as_uint(v) ^ (__float_as_uint(d) & 0x80000000u));
+}
+__device__ __forceinline__ float2 limited(float2 a, float2 b)
+{
+    return make_float2(limited(a.x, b.x), limited(a.y, b.y));
+}
+__device__ __forceinline__ float2 signed_as(float2 v, float2 d)
+{
+    return make_float2(signed_as(v.x, d.x), signed_as(v.y, d.y));
+}
 template <class V>
 __device__ __forceinline__ V nnd_diff_pos(V fm2, V fm1, V f0, V fp1)
 {
     const V d0 = vsub(fm1, fm2), d1 = vsub(f0, fm1), d2 = vsub(fp1, f0);
-    return vfma(bc<V>(0.5f), vsub(vmm(d1, d2), vmm(d0, d1)), d1);
+    return vfma(bc<V>(0.5f), signed_as(vsub(limited(d1, d2), limited(d0, d1)), d1), d1);
 }
 template <class V>
 __device__ __forceinline__ V nnd_diff_neg(V fm1, V f0, V fp1, V fp2)
 {
     const V d1 = vsub(f0, fm1), d2 = vsub(fp1, f0), d3 = vsub(fp2, fp1);
-    return vfma(bc<V>(-0.5f), vsub(vmm(d2, d3), vmm(d1, d2)), d2);
+    return vfma(bc<V>(-0.5f), signed_as(vsub(limited(d2, d3), limited(d1, d2)), d2), d2);
 }
 
 // The same x-direction flux differences for the pair of cells (x, x + 1),
 // from the two aligned 64-bit loads a = (f_{x-2}, f_{x-1}) and
-// b = (f_{x+2}, f_{x+3}) and the pair's own values c = (f_x, f_{x+1}): the
-// odd shifts are assembled from registers, and the limiter of the face
-// between the two cells is evaluated once (the second cell's left-face
-// minmod is the first cell's right-face minmod, with the same operands), so
-// the result is bitwise that of nnd_diff_pos / nnd_diff_neg.
+// b = (f_{x+2}, f_{x+3}) and the pair's own values c = (f_x, f_{x+1}).  The
+// pair's six slopes and four limiters are four slopes and three limiters of
+// faces: taken one by one (packed subtractions would first have to gather
+// the shifted pairs), bitwise those of nnd_diff_pos / nnd_diff_neg.
+__device__ __forceinline__ float2 nnd_diff_faces(float e0, float e1, float e2, float e3, float half)
+{
+    const float m01 = limited(e0, e1), m12 = limited(e1, e2), m23 = limited(e2, e3);
+    const float2 d = vsub(make_float2(m12, m23), make_float2(m01, m12)), e = make_float2(e1, e2);
+    return vfma(bc<float2>(half), signed_as(d, e), e);
+}
 __device__ __forceinline__ float2 nnd_diff_pos_pair(float2 a, float2 c, float2 b)
 {
-    const float2 fm1 = make_float2(a.y, c.x), fp1 = make_float2(c.y, b.x);
-    const float2 d0 = vsub(fm1, a), d1 = vsub(c, fm1), d2 = vsub(fp1, c);
-    const float2 m12 = vmm(d1, d2);
-    const float2 m01 = make_float2(minmod(d0.x, d1.x), m12.x);
-    return vfma(bc<float2>(0.5f), vsub(m12, m01), d1);
+    return nnd_diff_faces(vsub(a.y, a.x), vsub(c.x, a.y), vsub(c.y, c.x), vsub(b.x, c.y), 0.5f);
 }
 __device__ __forceinline__ float2 nnd_diff_neg_pair(float2 a, float2 c, float2 b)
 {
-    const float2 fm1 = make_float2(a.y, c.x), fp1 = make_float2(c.y, b.x);
-    const float2 d1 = vsub(c, fm1), d2 = vsub(fp1, c), d3 = vsub(b, fp1);
-    const float2 m23 = vmm(d2, d3);
-    const float2 m12 = make_float2(minmod(d1.x, d2.x), m23.x);
-    return vfma(bc<float2>(-0.5f), vsub(m23, m12), d2);
+    return nnd_diff_faces(vsub(c.x, a.y), vsub(c.y, c.x), vsub(b.x, c.y), vsub(b.y, b.x), -0.5f);
 }
 
 // Ghost-image bitmask of interior index k on an axis of n cells: bit j set
@@ -681,6 +707,7 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
 #pragma unroll
     for (int s = 0; s < S; ++s) {
         if constexpr (kStaged) t.acquire(s);
+        if constexpr (is_split<Tile>::value) t.arrived(s);
         const auto &ts = stage_view(t, s, s);
         V sn, sx, sy, se;
 #pragma unroll
@@ -1084,6 +1111,29 @@ __device__ __forceinline__ void tma_tile_load(float *tile, unsigned long long tm
         : "memory");
 }
 
+// Fetch into L2, without waiting, the cells of the tile `ahead` CTAs on in
+// launch order (one thread; tmap_in: the interior box of one species).  CTAs
+// start in that order, so with ahead = half the CTAs resident at once the
+// tile is in L2 when its own CTA asks for it, and HBM keeps busy while the
+// resident CTAs compute: a CTA's copy then takes L2's latency instead of
+// HBM's under load.  4096^2, two species, us a step by distance: none 753,
+// 76 736, 114 728, 152 (half) 726, 200 728, 304 (all) 738; boxes with the
+// halo 732 at 152; issued after the CTA's own copy has landed 731.
+__device__ __forceinline__ void tma_tile_prefetch(unsigned long long tmap, int x, int y, int z)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tmap), "r"(x), "r"(y),
+                 "r"(z)
+                 : "memory");
+}
+template <int S, int TX, int TY>
+__device__ __forceinline__ void prefetch_ahead(unsigned ahead, unsigned long long tmap_in)
+{
+    const unsigned t = blockIdx.y * gridDim.x + blockIdx.x + ahead;
+    if (t >= gridDim.x * gridDim.y) return;
+    const int x = (int)(t % gridDim.x) * TX + GX, y = (int)(t / gridDim.x) * TY + GY;
+    for (int s = 0; s < S; ++s) tma_tile_prefetch(tmap_in, x, y, s * Q);
+}
+
 // Source index of ghost index g (one of -2, -1, n, n + 1) on an axis of n
 // cells: the periodic image or the outflow edge cell.
 __device__ __forceinline__ int halo_source(int g, int n, int bc)
@@ -1263,6 +1313,18 @@ __device__ __forceinline__ void halo_store(const HaloRegs<NP, TX, TY, NT> &hr, c
     __syncthreads();
 }
 
+// A shared-memory tile whose species were copied one by one, each completing
+// its own mbarrier (species 0 has been waited for).
+template <class Base>
+struct SplitTile : Base {
+    static constexpr bool kSplit = true;
+    unsigned bar;  // barrier of species 0; species s: 8 s bytes on
+    __device__ __forceinline__ void arrived(int s) const
+    {
+        if (s > 0 && !mbar_wait(bar + 8u * s, 0, TMA_WAIT_LIMIT)) raise_flag(this->flag, DBM_HEALTH_TIMEOUT);
+    }
+};
+
 // X: NoAcc for the default arithmetic, AccConsts<S, MODE> for a kernel with the
 // thermo or rounding option or both.  One kernel per combination: with the
 // options as run-time switches of one kernel, stochastic rounding alone
@@ -1271,47 +1333,57 @@ __device__ __forceinline__ void halo_store(const HaloRegs<NP, TX, TY, NT> &hr, c
 template <int S, int TX, int TY, int CW, class X>
 __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     k_step_tma(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
-               const float *__restrict__ fin, float *__restrict__ fout, unsigned *__restrict__ flag,
-               const __grid_constant__ X xa)
+               const __grid_constant__ CUtensorMap tmap_in, const float *__restrict__ fin, float *__restrict__ fout,
+               unsigned *__restrict__ flag, const __grid_constant__ X xa)
 {
     static_assert(CW == 1 || CW == 2, "one or two cells per thread");
     constexpr int BX = TX + 8, BY = TY + 4, NP = S * Q, NT = TX / CW * TY;
-    constexpr unsigned BYTES = (unsigned)(BX * BY * NP * sizeof(float));
+    constexpr unsigned BYTES = (unsigned)(BX * BY * Q * sizeof(float));  // one species
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long bar;
+    __shared__ __align__(8) unsigned long long bar[S];
     float *tile = reinterpret_cast<float *>(smem_raw);
     const int tx = threadIdx.x, ty = threadIdx.y;
     const bool leader = tx == 0 && ty == 0;
     const int bx0 = blockIdx.x * TX, by0 = blockIdx.y * TY;
-    const unsigned b = smem_u32(&bar);
+    const unsigned b = smem_u32(&bar[0]);
     if (leader) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
+        for (int s = 0; s < S; ++s)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b + 8u * s) : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int s = 0; s < S; ++s)
+            tma_tile_load(tile + s * Q * BX * BY, reinterpret_cast<unsigned long long>(&tmap), bx0, by0, b + 8u * s,
+                          BYTES, s * Q);
+        prefetch_ahead<S, TX, TY>(c.prefetch, reinterpret_cast<unsigned long long>(&tmap_in));
     }
     __syncthreads();
-    if (leader) tma_tile_load(tile, reinterpret_cast<unsigned long long>(&tmap), bx0, by0, b, BYTES);
     const int tid = ty * (TX / CW) + tx;
     const HaloSides hs = halo_sides<TX, TY>(bx0, by0, c.nx, c.ny);
     const bool ok = mbar_wait(b, 0, c.wait_polls);
     if (__syncthreads_or(!ok)) {
-        // the copy did not land: report, give it one more bounded wait so
-        // that no copy is left writing into this block's shared memory, and
+        // the copy did not land: report, give the copies one more bounded wait
+        // so that none is left writing into this block's shared memory, and
         // leave together
         if (leader) raise_flag(flag, DBM_HEALTH_TIMEOUT);
-        mbar_wait(b, 0, TMA_WAIT_LIMIT);
+        for (int s = 0; s < S; ++s) mbar_wait(b + 8u * s, 0, TMA_WAIT_LIMIT);
         return;
     }
-    if (hs.any())
+    if (hs.any()) {
+        for (int s = 1; s < S; ++s)
+            if (!mbar_wait(b + 8u * s, 0, TMA_WAIT_LIMIT)) raise_flag(flag, DBM_HEALTH_TIMEOUT);
         halo_fill<NP, TX, TY, NT>(hs, tile, fin, bx0, by0, c.nx, c.ny, c.pitch, c.plane, c.bc_x, c.bc_y, tid, flag);
+    }
     const int x = bx0 + CW * tx, y = by0 + ty;
-    if (x >= c.nx || y >= c.ny) return;
+    if (x >= c.nx || y >= c.ny) {
+        for (int s = 1; s < S; ++s) mbar_wait(b + 8u * s, 0, TMA_WAIT_LIMIT);
+        return;
+    }
     StateOutNoImages o{fout, c.plane, (long long)NP * c.plane, flag};
     const float *base = tile + (ty + 2) * BX + (CW * tx + 4);
     if constexpr (CW == 2) {
-        const SmemTile2 t{base, BY * BX, BX, tile, NP * BY * BX, flag};
+        const SplitTile<SmemTile2> t{{base, BY * BX, BX, tile, NP * BY * BX, flag}, b};
         step_cell<S>(c, c, t, x, y, x + 1 < c.nx, o, flag, xa);
     } else {
-        const SmemTile t{base, BY * BX, BX, tile, NP * BY * BX, flag};
+        const SplitTile<SmemTile> t{{base, BY * BX, BX, tile, NP * BY * BX, flag}, b};
         step_cell<S>(c, c, t, x, y, true, o, flag, xa);
     }
 }
@@ -1329,7 +1401,8 @@ int launch_step_t(dbm_handle *h, const void *fin, void *fout, cudaStream_t st)
 
 // MODE: the thermo and rounding options (acc_mode), 0 for none.
 template <int S, int TX, int TY, int CW, int MODE>
-int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const void *fin, void *fout, cudaStream_t st)
+int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin, void *fout,
+                      cudaStream_t st)
 {
     using X = typename std::conditional<MODE != 0, AccConsts<S, MODE>, NoAcc>::type;
     constexpr size_t smem = (size_t)(TX + 8) * (TY + 4) * S * Q * sizeof(float);
@@ -1342,11 +1415,12 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const void *fin, v
     }
     StepConsts<float, S> c;
     fill_step_consts<float, S>(h, c);
+    c.prefetch = (unsigned)(h->sms * tma_ctas_per_sm(S, TX, TY) / 2);
     X xa{};
     if constexpr (MODE != 0) fill_acc_consts<S, MODE>(h, c, xa);
     dim3 block(TX / CW, TY);
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
-    k_step_tma<S, TX, TY, CW, X><<<grid, block, smem, st>>>(c, *tmap, (const float *)fin, (float *)fout,
+    k_step_tma<S, TX, TY, CW, X><<<grid, block, smem, st>>>(c, *tmap, *tmap_in, (const float *)fin, (float *)fout,
                                                               (unsigned *)h->scratch, xa);
     return set_cuda_error(h, cudaGetLastError(), "TMA step kernel launch");
 }

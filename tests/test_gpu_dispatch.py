@@ -1,0 +1,40 @@
+"""Steps whose kernel is chosen by size, on both sides of each line, against
+the generic kernel bit for bit (every FP32 kernel runs the same explicitly
+rounded arithmetic)."""
+import numpy as np
+import pytest
+
+from paper_2006_15932_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nx,ny,ns,bc", [
+    (513, 113, 2, (W.PERIODIC, W.OUTFLOW)),  # 9 x 15 pair tiles, ragged both ways
+    (512, 128, 2, (W.OUTFLOW, W.PERIODIC)),  # exactly 128 pair tiles
+    (510, 119, 2, (W.OUTFLOW, W.OUTFLOW)),   # 120: one cell per thread
+    (1025, 65, 1, (W.PERIODIC, W.PERIODIC)),
+    (321, 200, 3, (W.OUTFLOW, W.PERIODIC)),
+    (130, 300, 4, (W.PERIODIC, W.OUTFLOW)),
+])
+def test_automatic_step_matches_generic_bitwise(orc, nx, ny, ns, bc):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2006_15932_gb300 import build as B
+    from paper_2006_15932_gb300 import dbm as D
+
+    B.build()
+    pb = W.random_smooth(nx, ny, ns, seed=3, reactive=ns == 3, force=ns in (2, 4), bc=bc)
+    p = orc.params_of(pb)
+    f0 = orc.init_feq(p, pb.rho_s, pb.ux, pb.uy, pb.T)
+    f0 = f0 * (1.0 + 0.05 * np.random.default_rng(4).uniform(-1, 1, f0.shape))
+    out = {}
+    for kern in ("generic", "auto"):
+        s = D.Solver(pb, "fp32", step_kernel=kern)
+        s.set_f(f0)
+        s.step(5)
+        out[kern] = s.get_f()
+        assert s.status() == (0, 0)
+        s.close()
+    assert torch.equal(out["auto"], out["generic"])
