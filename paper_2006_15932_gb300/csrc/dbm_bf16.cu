@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(TX / CW * TY, bf16_ctas_per_sm(S, TX, TY))
     const int nthr = TX / CW * TY, tid = ty * (TX / CW) + tx;
     const int bx0 = blockIdx.x * TX, by0 = blockIdx.y * TY;
 
+    chain_begin();
     // phase A: rebuild f for the tile and its halo, one cell per iteration
     // (two cells per iteration in packed FP32x2 measured slower: 18.7
     // against 23.8 G/s on KH 4096^2); a halo cell outside the domain is
@@ -191,10 +192,10 @@ static int step_bf16_t(dbm_handle *h, int cur, cudaStream_t st)
     fill_step_consts<float, S>(h, c);
     dim3 block(BF_TX / BF_CW, BF_TY);
     dim3 grid((h->p.nx + BF_TX - 1) / BF_TX, (h->p.ny + BF_TY - 1) / BF_TY);
-    k_step_bf16<S, BF_TX, BF_TY, BF_CW><<<grid, block, smem, st>>>(c, bf_state(h, h->f[cur]),
-                                                                   bf_state(h, h->f[cur ^ 1]),
-                                                                   (unsigned *)h->scratch);
-    return set_cuda_error(h, cudaGetLastError(), "BF16 step kernel launch");
+    return set_cuda_error(h, launch_chained(k_step_bf16<S, BF_TX, BF_TY, BF_CW>, grid, block, smem, st, c,
+                                            bf_state(h, h->f[cur]), bf_state(h, h->f[cur ^ 1]),
+                                            (unsigned *)h->scratch),
+                          "BF16 step kernel launch");
 }
 
 int launch_step_bf16(dbm_handle *h, int cur, cudaStream_t st)

@@ -8,6 +8,33 @@
 
 namespace dbm {
 
+// Chained launches: a step kernel launched with programmatic serialization
+// may start while the kernel before it on the stream still drains.  It sets
+// up its barriers, lets its own successor do the same, and touches no memory
+// that another kernel reads or writes before chain_begin has returned: by then
+// the kernel before it has completed and its writes are visible.
+__device__ __forceinline__ void chain_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // f-hat_1..16 of the moment relations (section "Discrete Boltzmann model",
 // the f-hat list restating Eqs. relation1..relation7) at (n, u, theta = T/m)
 // with dpi = D + I.  Factored for the GPU; the same polynomials as printed.

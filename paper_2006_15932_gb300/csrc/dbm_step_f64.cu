@@ -235,6 +235,8 @@ __global__ void __launch_bounds__(128 * f64_side(S))
         return (long long)(y + GY) * c.pitch + (x + GX);
     };
 
+    chain_begin();
+
     // 1. moment sums
 #pragma unroll 1
     for (int it = tid; it < S * 4 * CELLS; it += NT) {
@@ -462,9 +464,9 @@ static int launch_f64_v(dbm_handle *h, const double *fin, double *fout, cudaStre
         }
     }
     const long long cells = (long long)h->p.nx * h->p.ny;
-    k_step_f64<S, WIDE><<<(unsigned)((cells + CELLS - 1) / CELLS), 128 * f64_side(S), smem, st>>>(
-        c, fin, fout, (unsigned *)h->scratch);
-    return set_cuda_error(h, cudaGetLastError(), "FP64 step kernel launch");
+    return set_cuda_error(h, launch_chained(k_step_f64<S, WIDE>, dim3((unsigned)((cells + CELLS - 1) / CELLS)),
+                                            dim3(128 * f64_side(S)), smem, st, c, fin, fout, (unsigned *)h->scratch),
+                          "FP64 step kernel launch");
 }
 
 template <int S>

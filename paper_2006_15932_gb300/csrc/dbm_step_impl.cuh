@@ -1350,6 +1350,9 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
         for (int s = 0; s < S; ++s)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b + 8u * s) : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    chain_begin();
+    if (leader) {
         for (int s = 0; s < S; ++s)
             tma_tile_load(tile + s * Q * BX * BY, reinterpret_cast<unsigned long long>(&tmap), bx0, by0, b + 8u * s,
                           BYTES, s * Q);
@@ -1420,9 +1423,9 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
     if constexpr (MODE != 0) fill_acc_consts<S, MODE>(h, c, xa);
     dim3 block(TX / CW, TY);
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
-    k_step_tma<S, TX, TY, CW, X><<<grid, block, smem, st>>>(c, *tmap, *tmap_in, (const float *)fin, (float *)fout,
-                                                              (unsigned *)h->scratch, xa);
-    return set_cuda_error(h, cudaGetLastError(), "TMA step kernel launch");
+    return set_cuda_error(h, launch_chained(k_step_tma<S, TX, TY, CW, X>, grid, block, smem, st, c, *tmap, *tmap_in,
+                                            (const float *)fin, (float *)fout, (unsigned *)h->scratch, xa),
+                          "TMA step kernel launch");
 }
 
 
@@ -1555,6 +1558,7 @@ __global__ void __launch_bounds__(TX / 2 * TY, staged_ctas_per_sm(TX, TY))
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
+    chain_begin();
     const T t{buf,
               buf + (ty + 2) * T::BX + (2 * tx + 4),
               buf + ty * TX + 2 * tx,
@@ -1603,9 +1607,9 @@ int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorM
     fill_step_consts<float, S>(h, c);
     dim3 block(TX / 2, TY);
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
-    k_step_staged<S, TX, TY><<<grid, block, smem, st>>>(c, *tmap, *tmap_in, (const float *)fin, (float *)fout,
-                                                         (unsigned *)h->scratch);
-    return set_cuda_error(h, cudaGetLastError(), "staged step kernel launch");
+    return set_cuda_error(h, launch_chained(k_step_staged<S, TX, TY>, grid, block, smem, st, c, *tmap, *tmap_in,
+                                            (const float *)fin, (float *)fout, (unsigned *)h->scratch),
+                          "staged step kernel launch");
 }
 
 }  // namespace dbm

@@ -38,3 +38,36 @@ def test_automatic_step_matches_generic_bitwise(orc, nx, ny, ns, bc):
         assert s.status() == (0, 0)
         s.close()
     assert torch.equal(out["auto"], out["generic"])
+
+
+@pytest.mark.parametrize("prec,ns", [("fp32", 1), ("fp32", 2), ("fp32", 5), ("fp64", 2), ("bf16dev", 2)])
+def test_chained_steps_captured_and_beside_another_stream(prec, ns):
+    """Steps launched with programmatic serialization: captured into a graph
+    and replayed, and interleaved with a second solver on another stream, they
+    give the bits of plain steps."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2006_15932_gb300 import build as B
+    from paper_2006_15932_gb300 import dbm as D
+
+    B.build()
+    pb = W.random_smooth(131, 67, ns, seed=8)
+    side = torch.cuda.Stream()
+    plain, graphed, beside = (D.Solver(pb, prec, stream=st) for st in (None, None, side))
+    for s in (plain, graphed, beside):
+        s.set_state()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):  # captured, not run: four steps from the first buffer
+        graphed.step(4)
+    graph.replay()
+    graph.replay()
+    for _ in range(4):
+        beside.step(2)
+        plain.step(2)
+    torch.cuda.synchronize()
+    want = plain.get_f()
+    assert torch.equal(graphed.get_f(), want) and torch.equal(beside.get_f(), want)
+    for s in (plain, graphed, beside):
+        assert s.status() == (0, 0)
+        s.close()
