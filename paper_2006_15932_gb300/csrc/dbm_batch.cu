@@ -169,7 +169,7 @@ static int write_tables(dbm_batch *b, cudaStream_t st)
                 const dbm_layout &L = h->lay;
                 cuuint64_t dims[3] = {(cuuint64_t)L.pitch, (cuuint64_t)L.rows, (cuuint64_t)(16 * S)};
                 cuuint64_t strides[2] = {(cuuint64_t)L.pitch * 4, (cuuint64_t)L.plane * 4};
-                cuuint32_t box[3] = {(cuuint32_t)(TX + 8), (cuuint32_t)(TY + 4), (cuuint32_t)(16 * S)};
+                cuuint32_t box[3] = {(cuuint32_t)(TX + 8), (cuuint32_t)(TY + 4), 16};
                 cuuint32_t estr[3] = {1, 1, 1};
                 if (encode(&e.tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, in, dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -187,6 +187,7 @@ static int write_tables(dbm_batch *b, cudaStream_t st)
             blk[par]->t0 = t0;
             blk[par]->nt = (int)b->tiles.size() - t0;
             blk[par]->hot = cs[rep[j]];
+            blk[par]->hot.prefetch = (unsigned)b->resident / 2;  // read by the one-tile-per-CTA form
         }
     }
     b->total_tiles = (int)b->tiles.size();

@@ -115,15 +115,16 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     k_step_batch(const __grid_constant__ BatchChunk<S> P, const BatchTile *__restrict__ tiles)
 {
     constexpr int BX = TX + 8, BY = TY + 4, NP = S * Q, NT = TX / CW * TY;
-    constexpr unsigned BYTES = (unsigned)(BX * BY * NP * sizeof(float));
+    constexpr unsigned BYTES = (unsigned)(BX * BY * Q * sizeof(float));  // one species
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long bar;
+    __shared__ __align__(8) unsigned long long bar[S];
     float *tile = reinterpret_cast<float *>(smem_raw);
     const int tx = threadIdx.x, ty = threadIdx.y;
     const bool leader = tx == 0 && ty == 0;
-    const unsigned b = smem_u32(&bar);
+    const unsigned b = smem_u32(&bar[0]);
     if (leader) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
+        for (int s = 0; s < S; ++s)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b + 8u * s) : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     const int t0 = P.t0 + (PERSIST ? (int)((long long)P.nt * blockIdx.x / gridDim.x) : (int)blockIdx.x);
@@ -141,7 +142,17 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
             // generic proxy; order them before the async-proxy copy that
             // overwrites the same shared memory
             if (t > t0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            tma_tile_load(tile, reinterpret_cast<unsigned long long>(&e.tmap), cur.bx0, cur.by0, b, BYTES);
+            for (int s = 0; s < S; ++s)
+                tma_tile_load(tile + s * Q * BX * BY, reinterpret_cast<unsigned long long>(&e.tmap), cur.bx0, cur.by0,
+                              b + 8u * s, BYTES, s * Q);
+            // one CTA per tile: fetch a later CTA's tile into L2 (prefetch_ahead
+            // has the reasons; here with the halo, by the one descriptor an
+            // instance has)
+            if (!PERSIST && P.hot.prefetch != 0 && blockIdx.x + P.hot.prefetch < gridDim.x) {
+                const BatchTile far = tiles[t0 + (int)P.hot.prefetch];
+                for (int s = 0; s < S; ++s)
+                    tma_tile_prefetch(reinterpret_cast<unsigned long long>(&P.e[far.k].tmap), far.bx0, far.by0, s * Q);
+            }
         }
         const int tid = ty * (TX / CW) + tx;
         const HaloSides hs = halo_sides<TX, TY>(cur.bx0, cur.by0, g.nx, g.ny);
@@ -150,22 +161,26 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
             halo_load(hr, hs, e.fin, cur.bx0, cur.by0, g.nx, g.ny, g.pitch, g.plane, g.bc_x, g.bc_y, tid, e.flag);
         const bool ok = mbar_wait(b, phase, g.wait_polls);
         if (__syncthreads_or(!ok)) {
-            // the copy did not land: report, give it one more bounded wait so
-            // that no copy is left writing into shared memory, leave together
+            // the copy did not land: report, give the copies one more bounded wait
+            // so that none is left writing into shared memory, leave together
             if (leader) raise_flag(e.flag, DBM_HEALTH_TIMEOUT);
-            mbar_wait(b, phase, TMA_WAIT_LIMIT);
+            for (int s = 0; s < S; ++s) mbar_wait(b + 8u * s, phase, TMA_WAIT_LIMIT);
             return;
         }
-        if (hs.any()) halo_store(hr, hs, tile, cur.bx0, cur.by0, g.nx, g.ny, tid, e.flag);
         const int x = cur.bx0 + CW * tx, y = cur.by0 + ty;
-        if (x < g.nx && y < g.ny) {
+        const bool inside = x < g.nx && y < g.ny;
+        if (hs.any() || !inside)
+            for (int s = 1; s < S; ++s)
+                if (!mbar_wait(b + 8u * s, phase, TMA_WAIT_LIMIT)) raise_flag(e.flag, DBM_HEALTH_TIMEOUT);
+        if (hs.any()) halo_store(hr, hs, tile, cur.bx0, cur.by0, g.nx, g.ny, tid, e.flag);
+        if (inside) {
             StateOutNoImages o{e.fout, g.plane, (long long)NP * g.plane, e.flag};
             const float *base = tile + (ty + 2) * BX + (CW * tx + 4);
             if constexpr (CW == 2) {
-                const SmemTile2 st{base, BY * BX, BX, tile, NP * BY * BX, e.flag};
+                const SplitTile<SmemTile2> st{{base, BY * BX, BX, tile, NP * BY * BX, e.flag}, b, phase};
                 step_cell<S>(P.hot, g, st, x, y, x + 1 < g.nx, o, e.flag);
             } else {
-                const SmemTile st{base, BY * BX, BX, tile, NP * BY * BX, e.flag};
+                const SplitTile<SmemTile> st{{base, BY * BX, BX, tile, NP * BY * BX, e.flag}, b, phase};
                 step_cell<S>(P.hot, g, st, x, y, true, o, e.flag);
             }
         }

@@ -1318,10 +1318,11 @@ __device__ __forceinline__ void halo_store(const HaloRegs<NP, TX, TY, NT> &hr, c
 template <class Base>
 struct SplitTile : Base {
     static constexpr bool kSplit = true;
-    unsigned bar;  // barrier of species 0; species s: 8 s bytes on
+    unsigned bar;    // barrier of species 0; species s: 8 s bytes on
+    unsigned phase;  // of this tile's copies
     __device__ __forceinline__ void arrived(int s) const
     {
-        if (s > 0 && !mbar_wait(bar + 8u * s, 0, TMA_WAIT_LIMIT)) raise_flag(this->flag, DBM_HEALTH_TIMEOUT);
+        if (s > 0 && !mbar_wait(bar + 8u * s, phase, TMA_WAIT_LIMIT)) raise_flag(this->flag, DBM_HEALTH_TIMEOUT);
     }
 };
 
@@ -1383,10 +1384,10 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     StateOutNoImages o{fout, c.plane, (long long)NP * c.plane, flag};
     const float *base = tile + (ty + 2) * BX + (CW * tx + 4);
     if constexpr (CW == 2) {
-        const SplitTile<SmemTile2> t{{base, BY * BX, BX, tile, NP * BY * BX, flag}, b};
+        const SplitTile<SmemTile2> t{{base, BY * BX, BX, tile, NP * BY * BX, flag}, b, 0u};
         step_cell<S>(c, c, t, x, y, x + 1 < c.nx, o, flag, xa);
     } else {
-        const SplitTile<SmemTile> t{{base, BY * BX, BX, tile, NP * BY * BX, flag}, b};
+        const SplitTile<SmemTile> t{{base, BY * BX, BX, tile, NP * BY * BX, flag}, b, 0u};
         step_cell<S>(c, c, t, x, y, true, o, flag, xa);
     }
 }

@@ -499,7 +499,8 @@ class Batch:
     """Solvers (FP32, same species count) stepped together: one launch per
     step and chunk of instances, pairs of steps replayed from a CUDA graph.
     The kernel configuration is tuned (``tune``), given (``config``, a dict
-    as returned by ``config()``), or the library's default."""
+    as returned by ``config()``, whose ``by_species`` may hold other values
+    for some species counts), or the library's default."""
 
     def __init__(self, solvers, stream=None, tune=True, config=None):
         import torch
@@ -522,6 +523,7 @@ class Batch:
         self._enter()
         self.b = dbm_batch_create(handles, self._tp, nb, self.stream.cuda_stream)
         if config is not None:
+            config = {**config, **config.get("by_species", {}).get(self.solvers[0].S, {})}
             dbm_batch_set_config(self.b, config["tile"], config.get("cells", 1), config["persistent"], config["promote"],
                                  stream=self.stream.cuda_stream)
         elif tune:

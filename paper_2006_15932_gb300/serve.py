@@ -46,10 +46,14 @@ import numpy as np
 from . import dbm as D
 from . import workloads as W
 
-# kernel configuration of the batched groups (tile shape, launch form, L2
-# promotion): what the tuner picks for the 64-instance mix of sides 64 to
-# 512, and the fastest shape measured on instances of 256^2 to 4096^2
-DEFAULT_CONFIG = {"tile": (64, 4), "cells": 1, "persistent": 0, "promote": 1}
+# kernel configuration of the batched groups (tile shape, cells per thread,
+# launch form, L2 promotion), by species count where it differs: the fastest
+# of the compiled shapes with one CTA per tile on mixes of sides 64 to 512
+# (us a step, best shape / 64 x 4 one cell, the former shape of all: two
+# species, 64 instances 358 / 386; three species, 30 instances of 100 to 400
+# 203 / 221; four 290 / 410; one species 64 x 4 stays)
+DEFAULT_CONFIG = {"tile": (64, 8), "cells": 2, "persistent": 0, "promote": 1,
+                  "by_species": {1: {"tile": (64, 4), "cells": 1}, 3: {"tile": (32, 8), "cells": 1}}}
 
 
 class Admission:
