@@ -24,6 +24,13 @@ constexpr int bf16_ctas_per_sm(int S, int TX, int TY)
     return n > 4 ? 4 : n < 1 ? 1 : n;
 }
 
+// The cell inside 0 .. n-1 that index k of the domain or its halo stands for.
+__device__ __forceinline__ int source_cell(int k, int n, int bc)
+{
+    if (k >= 0 && k < n) return k;
+    return bc == DBM_BC_PERIODIC ? ((k % n) + n) % n : min(max(k, 0), n - 1);
+}
+
 template <int S, int TX, int TY, int CW>
 __global__ void __launch_bounds__(TX / CW * TY, bf16_ctas_per_sm(S, TX, TY))
     k_step_bf16(const __grid_constant__ StepConsts<float, S> c, BfState in, BfState out,
@@ -37,28 +44,36 @@ __global__ void __launch_bounds__(TX / CW * TY, bf16_ctas_per_sm(S, TX, TY))
     const int bx0 = blockIdx.x * TX, by0 = blockIdx.y * TY;
 
     chain_begin();
-    // phase A: rebuild f for the tile and its halo, one cell per iteration
-    // (two cells per iteration in packed FP32x2 measured slower: 18.7
-    // against 23.8 G/s on KH 4096^2); a halo cell outside the domain is
-    // rebuilt from its source cell (periodic wrap, or the edge cell for
-    // outflow), so the stored ghost cells are neither read nor written
-    for (int k = tid; k < BX * BY; k += nthr) {
-        const int rr = k / BX, cc = k % BX;
+    // phase A: rebuild f for the tile and its halo, one species of a pair of
+    // adjacent cells per item, so that the equilibrium runs in packed FP32x2
+    // and the items (720 for two species on 32 x 16) fill the CTA's rounds (whole
+    // pairs, both species, left half of the second round idle and ran slower
+    // than single cells); a halo cell outside the domain is rebuilt from
+    // its source cell (periodic wrap, or the edge cell for outflow), so the
+    // stored ghost cells are neither read nor written.  2048 x 1024, two
+    // species, us a step: single cells 175, this 155.
+    static_assert(TX % 2 == 0, "column 0 of the tile, x0 - 2, is even");
+    // items of a species padded to whole warps: the branch on the species is
+    // uniform, and its constants stay constant-bank operands
+    constexpr int PX = BX / 2, PAIRS = PX * BY, PADDED = (PAIRS + 31) / 32 * 32;
+    for (int k = tid; k < PADDED * S; k += nthr) {
+        const int sk = k / PADDED, kk = k - sk * PADDED;
+        if (kk >= PAIRS) continue;
+        const int rr = kk / PX, cc = 2 * (kk - rr * PX);
         const int x = bx0 - 2 + cc, y = by0 - 2 + rr;
-        const bool ok = x <= c.nx + 1 && y <= c.ny + 1;  // within reach of the stencil
-        const int xs = x >= 0 && x < c.nx ? x
-                       : c.bc_x == DBM_BC_PERIODIC ? ((x % c.nx) + c.nx) % c.nx : min(max(x, 0), c.nx - 1);
-        const int ys = y >= 0 && y < c.ny ? y
-                       : c.bc_y == DBM_BC_PERIODIC ? ((y % c.ny) + c.ny) % c.ny : min(max(y, 0), c.ny - 1);
-        const long long cell = (long long)(ys + GY) * c.pitch + (xs + GX);
-        float *dst = tile + rr * BX + cc;
-        const bool src_ok = ok && in_bounds(cell, in.P, flag);
-#pragma unroll 1
-        for (int s = 0; s < S; ++s) {
-            float f[Q];
-            if (src_ok) bf_cell_f<S>(c, in, s, cell, f);
+        // within reach of the stencil; x + 1 beyond it comes out of the last column in reach
+        const bool ok = x <= c.nx + 1 && y <= c.ny + 1;
+        const int xs0 = source_cell(x, c.nx, c.bc_x), xs1 = source_cell(min(x + 1, c.nx + 1), c.nx, c.bc_x);
+        const long long row = (long long)(source_cell(y, c.ny, c.bc_y) + GY) * c.pitch + GX;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) dst[(s * Q + i) * (BY * BX)] = src_ok ? f[i] : 0.0f;
+        for (int s = 0; s < S; ++s) {
+            if (s != sk) continue;
+            float2 f[Q];
+            if (ok) bf_pair_f<S>(c, in, s, row + xs0, row + xs1, f, flag);
+            float *dst = tile + (s * Q) * (BY * BX) + rr * BX + cc;
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+                *reinterpret_cast<float2 *>(dst + i * (BY * BX)) = ok ? f[i] : make_float2(0.0f, 0.0f);
         }
     }
     __syncthreads();

@@ -107,6 +107,41 @@ __device__ __forceinline__ void bf_cell_f(const StepConsts<float, S> &k, const B
     for (int i = 0; i < Q; ++i) f[i] += __bfloat162float(st.d[(long long)(s * Q + i) * st.P + cell]);
 }
 
+// f of species s at the cells a and b (element offsets), FP32; adjacent cells
+// from an even column on are read as pairs.
+template <int S>
+__device__ __forceinline__ void bf_pair_f(const StepConsts<float, S> &k, const BfState &st, int s, long long a,
+                                          long long b, float2 f[Q], unsigned *flag)
+{
+    float2 n, ux, uy, T;
+    __nv_bfloat162 d[Q];
+    const float *mn = st.mom + (long long)s * st.P, *mu = st.mom + (long long)S * st.P;
+    const __nv_bfloat16 *dev = st.d + (long long)s * Q * st.P;
+    if (!in_bounds(a, st.P, flag) || !in_bounds(b, st.P, flag)) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) f[i] = make_float2(0.0f, 0.0f);
+        return;
+    }
+    if (b == a + 1 && (a & 1) == 0) {
+        n = *reinterpret_cast<const float2 *>(mn + a);
+        ux = *reinterpret_cast<const float2 *>(mu + a);
+        uy = *reinterpret_cast<const float2 *>(mu + st.P + a);
+        T = *reinterpret_cast<const float2 *>(mu + 2 * st.P + a);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) d[i] = *reinterpret_cast<const __nv_bfloat162 *>(dev + i * st.P + a);
+    } else {
+        n = make_float2(mn[a], mn[b]);
+        ux = make_float2(mu[a], mu[b]);
+        uy = make_float2(mu[st.P + a], mu[st.P + b]);
+        T = make_float2(mu[2 * st.P + a], mu[2 * st.P + b]);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) d[i] = __nv_bfloat162(dev[i * st.P + a], dev[i * st.P + b]);
+    }
+    feq_ref<S, float2>(k, s, n, ux, uy, T, f);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = vadd(f[i], __bfloat1622float2(d[i]));
+}
+
 // Source policy of the FP64 output kernels for a BF16-deviation state.
 template <int S>
 struct BfSrc {
