@@ -324,48 +324,85 @@ __global__ void __launch_bounds__(256)
     out[(4 * S + 4) * N + d] = widen(ntot) * widen(T);
 }
 
-// The moments of rows 5..16 of M (xx, xy, yy, q x, q y, xxx, xxy, xyy, yyy,
-// q xx, q xy, q yy) of one species' values.
+// Weights of the nonequilibrium sums, products of the ring constants with m
+// formed on the host: on the FP64 pipe they would be 20 of a species' 250
+// operations.
 template <int S>
-__device__ __forceinline__ void high_moments(const OutConsts<S> &c, int s, const double f[Q], double t[12])
+struct NoneqConsts {
+    OutConsts<S> c;
+    double v2[S][4], qv[S][4], v3[S][4], qv2[S][4];  // m v^2, m q v, m v^3, m q v^2
+    double inv_m[S];
+};
+
+template <int S>
+inline NoneqConsts<S> noneq_consts(const OutConsts<S> &c)
+{
+    NoneqConsts<S> k;
+    memset(&k, 0, sizeof(k));
+    k.c = c;
+    for (int s = 0; s < S; ++s) {
+        for (int r = 0; r < 4; ++r) {
+            const double v = c.vr[s][r], q = c.qr[s][r];
+            k.v2[s][r] = c.m[s] * (v * v);
+            k.qv[s][r] = c.m[s] * (q * v);
+            k.v3[s][r] = c.m[s] * (v * v * v);
+            k.qv2[s][r] = c.m[s] * (q * v * v);
+        }
+        k.inv_m[s] = 1.0 / c.m[s];
+    }
+    return k;
+}
+
+// m times the moments of rows 5..16 of M (xx, xy, yy, q x, q y, xxx, xxy, xyy,
+// yyy, q xx, q xy, q yy) of one species' values.
+template <int S>
+__device__ __forceinline__ void high_moments(const NoneqConsts<S> &k, int s, const double f[Q], double t[12])
 {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) t[k] = 0.0;
+    for (int j = 0; j < 12; ++j) t[j] = 0.0;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const RingSums g = ring_sums(r, f + 4 * r);
-        const double v = c.vr[s][r], q = c.qr[s][r], v2 = v * v, qv = q * v, qv2 = q * v2, v3 = v * v2;
-        t[0] += v2 * g.xx;
-        t[2] += v2 * g.yy;
-        t[3] += qv * g.rx;
-        t[4] += qv * g.ry;
-        t[5] += v3 * g.rx;
-        t[8] += v3 * g.ry;
-        t[9] += qv2 * g.xx;
-        t[11] += qv2 * g.yy;
-        if (r & 1) {
-            t[1] += v2 * g.xy;
-            t[6] += v3 * g.ry;
-            t[7] += v3 * g.rx;
-            t[10] += qv2 * g.xy;
+        if (r & 1) {  // xx and yy are the ring's sum, xxx = xyy, xxy = yyy
+            const double e2 = k.v2[s][r] * g.all, e4 = k.qv2[s][r] * g.all;
+            const double cx = k.v3[s][r] * g.rx, cy = k.v3[s][r] * g.ry;
+            t[0] += e2;
+            t[2] += e2;
+            t[9] += e4;
+            t[11] += e4;
+            t[5] += cx;
+            t[7] += cx;
+            t[6] += cy;
+            t[8] += cy;
+            t[1] += k.v2[s][r] * g.xy;
+            t[10] += k.qv2[s][r] * g.xy;
+        } else {
+            t[0] += k.v2[s][r] * g.xx;
+            t[2] += k.v2[s][r] * g.yy;
+            t[9] += k.qv2[s][r] * g.xx;
+            t[11] += k.qv2[s][r] * g.yy;
+            t[5] += k.v3[s][r] * g.rx;
+            t[8] += k.v3[s][r] * g.ry;
         }
+        t[3] += k.qv[s][r] * g.rx;
+        t[4] += k.qv[s][r] * g.ry;
     }
 }
 
 // Nonequilibrium moments.  The equilibrium is M^-1 f-hat, so its moments of
 // the 16 monomials of M are f-hat itself, and all twelve moments of the
 // output are among them: Delta = m (M f - f-hat).  Neither f^eq nor a sum
-// over it is needed, and M f comes from ring sums: about 190 FP64 operations
+// over it is needed, and M f comes from ring sums: under 200 FP64 operations
 // per species and cell where summing f - f^eq over the velocities took 1400
-// (the FP64 pipe bounds this kernel: 2048 x 1024, two species, 7.9 -> 1.85
-// ms).
-// Up to two species keep their values in registers until the mixture u and T
-// are known; more load them again.
+// (the FP64 pipe bounds this kernel: 2048 x 1024, two species, 7.9 -> 1.63
+// ms).  Up to two species keep their values in registers until the mixture u
+// and T are known; more load them again.
 template <int S, class Src>
 __global__ void __launch_bounds__(128)
-    k_noneq(const __grid_constant__ OutConsts<S> c, const __grid_constant__ Src src,
+    k_noneq(const __grid_constant__ NoneqConsts<S> k, const __grid_constant__ Src src,
             double *__restrict__ out)
 {
+    const OutConsts<S> &c = k.c;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= c.nx || y >= c.ny) return;
@@ -384,20 +421,20 @@ __global__ void __launch_bounds__(128)
         for (int j = 1; j < S; ++j)
             if (s == j) ns = n[j];
         src.load16(s, cell, fc);
-        high_moments<S>(c, s, fc, t);
-        fhat16<double>(ns, ux, uy, T / c.m[s], c.dpi[s], fh);
-        const double m = c.m[s], hm = 0.5 * m;
+        high_moments<S>(k, s, fc, t);
+        // f-hat is linear in n: m f-hat is that of m n
+        fhat16<double>(c.m[s] * ns, ux, uy, T * k.inv_m[s], c.dpi[s], fh);
         double *o = out + 20LL * s * N + d;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) o[k * N] = m * (t[k] - fh[4 + k]);
-        o[12 * N] = hm * t[0];
-        o[13 * N] = hm * t[2];
-        o[14 * N] = hm * fh[4];
-        o[15 * N] = hm * fh[6];
-        o[16 * N] = hm * t[3];
-        o[17 * N] = hm * t[4];
-        o[18 * N] = hm * fh[7];
-        o[19 * N] = hm * fh[8];
+        for (int j = 0; j < 12; ++j) o[j * N] = t[j] - fh[4 + j];
+        o[12 * N] = 0.5 * t[0];
+        o[13 * N] = 0.5 * t[2];
+        o[14 * N] = 0.5 * fh[4];
+        o[15 * N] = 0.5 * fh[6];
+        o[16 * N] = 0.5 * t[3];
+        o[17 * N] = 0.5 * t[4];
+        o[18 * N] = 0.5 * fh[7];
+        o[19 * N] = 0.5 * fh[8];
     }
 }
 
@@ -688,7 +725,7 @@ inline void noneq_t(dbm_handle *h, const Src &src, double *out, cudaStream_t st)
     OutConsts<S> c;
     fill_out_consts<S>(h, c);
     dim3 b(32, 4);
-    k_noneq<S, Src><<<cell_grid(h, b), b, 0, st>>>(c, src, out);
+    k_noneq<S, Src><<<cell_grid(h, b), b, 0, st>>>(noneq_consts<S>(c), src, out);
 }
 
 template <int S, class Src>
