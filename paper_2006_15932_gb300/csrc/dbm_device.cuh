@@ -10,14 +10,20 @@ namespace dbm {
 
 // Chained launches: a step kernel launched with programmatic serialization
 // may start while the kernel before it on the stream still drains.  It sets
-// up its barriers, lets its own successor do the same, and touches no memory
-// that another kernel reads or writes before chain_begin has returned: by then
-// the kernel before it has completed and its writes are visible.
-__device__ __forceinline__ void chain_begin()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// up its barriers and touches no memory that another kernel reads or writes
+// before chain_begin has returned: by then the kernel before it has completed
+// and its writes are visible.  Its own successor may start once every CTA has
+// passed chain_end, which sits late in the step: CTAs that start early take
+// the free SMs and the rest of their grid doubles up on others, which costs
+// a grid of fewer CTAs than the chip holds more than the launch it hides
+// (FP64, 64 x 64, two species: 29 us a step unchained, 54 with the successor
+// let in at once).
+__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_end() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+// Dynamic shared memory that keeps a grid of at most one CTA per SM from
+// doubling up: more than half of an SM's.
+constexpr size_t ALONE_SMEM = 116 * 1024;
 
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)

@@ -42,15 +42,15 @@
 // lane idle) in phases through shared memory, each with its own split:
 //   1  the 4 moment sums of a cell and species, one thread each (each sum is
 //      a serial chain, the four run side by side);
-//   2  species velocities and weights, one thread per cell and species;
-//   3  mixture u, T and the rate, one thread per cell;
-//   4  f-hat of each term, one thread per cell and species;
-//   5  collision, advection and update, a warp per ring of four velocities:
-//      WIDE, 32 cells with the ring's four velocities in each thread (shared
-//      products); else 8 cells with a velocity per thread, four times as many
-//      CTAs, which a small grid needs to reach every SM and to shorten the
-//      chain of dependent operations (400 x 1, two species: 268 us a step,
-//      now 18).  NARROW_CELLS is where the two cross.
+//   2  species velocities and weights;
+//   3  mixture u, T and the rate;
+//   4  f-hat of each term;
+//   5  collision, advection and update, a warp per ring of four velocities.
+// k_step_f64: 32 cells, in phase 5 the ring's four velocities in each thread
+// (shared products).  k_step_f64_small: 4 cells, for grids that leave the chip
+// idle, where the chain of dependent operations is the time: a warp issues an
+// FP64 instruction at most every 64 cycles whatever the others do, so every
+// phase is spread over warps (see there).
 // Ghosts of the new state are written as images by the edge cells.
 #include "dbm_consts.h"
 #include "dbm_device.cuh"
@@ -97,30 +97,40 @@ __device__ __forceinline__ double nnd_dflux(double fm2, double fm1, double fp1, 
 
 // f-hat_1..16 at (n, u, T) for a species of mass m and extra degrees of
 // freedom I, theta = T/m, D = 2, in the printed form; written to
-// fh[k * stride].
+// fh[k * stride].  PART 0..3: a quarter of the work each; -1: all of it.
+template <int PART = -1>
 __device__ __forceinline__ void fhat_printed(double n, double ux, double uy, double T, const ConstDiv &m, double I,
                                              double *fh, int stride)
 {
+    constexpr bool ALL = PART < 0;
     const double D = 2.0;
     const double th = div_by(T, m);
     const double u2 = ux * ux + uy * uy;
     const double a0 = (D + I) * th + u2, a2 = (D + I + 2.0) * th + u2, a4 = (D + I + 4.0) * th + u2;
-    fh[0] = n;
-    fh[1 * stride] = n * ux;
-    fh[2 * stride] = n * uy;
-    fh[3 * stride] = n * a0;
-    fh[4 * stride] = n * (th + ux * ux);
-    fh[5 * stride] = n * ux * uy;
-    fh[6 * stride] = n * (th + uy * uy);
-    fh[7 * stride] = n * ux * a2;
-    fh[8 * stride] = n * uy * a2;
-    fh[9 * stride] = 3.0 * n * ux * th + n * ux * ux * ux;
-    fh[10 * stride] = n * uy * th + n * ux * ux * uy;
-    fh[11 * stride] = n * ux * th + n * ux * uy * uy;
-    fh[12 * stride] = 3.0 * n * uy * th + n * uy * uy * uy;
-    fh[13 * stride] = n * a2 * th + n * ux * ux * a4;
-    fh[14 * stride] = n * ux * uy * a4;
-    fh[15 * stride] = n * a2 * th + n * uy * uy * a4;
+    if (ALL || PART == 0) {
+        fh[0] = n;
+        fh[1 * stride] = n * ux;
+        fh[2 * stride] = n * uy;
+        fh[4 * stride] = n * (th + ux * ux);
+        fh[5 * stride] = n * ux * uy;
+        fh[6 * stride] = n * (th + uy * uy);
+        fh[10 * stride] = n * uy * th + n * ux * ux * uy;
+    }
+    if (ALL || PART == 1) {
+        fh[3 * stride] = n * a0;
+        fh[7 * stride] = n * ux * a2;
+        fh[8 * stride] = n * uy * a2;
+        fh[14 * stride] = n * ux * uy * a4;
+    }
+    if (ALL || PART == 2) {
+        fh[9 * stride] = 3.0 * n * ux * th + n * ux * ux * ux;
+        fh[11 * stride] = n * ux * th + n * ux * uy * uy;
+        fh[12 * stride] = 3.0 * n * uy * th + n * uy * uy * uy;
+    }
+    if (ALL || PART == 3) {
+        fh[13 * stride] = n * a2 * th + n * ux * ux * a4;
+        fh[15 * stride] = n * a2 * th + n * uy * uy * a4;
+    }
 }
 
 // Rows of M^-1.  The row of the ring's first velocity, (+,0) or (+,+), gives
@@ -212,12 +222,12 @@ constexpr size_t f64_smem(int cells, int sets)
     return sizeof(double) * (size_t)cells * (S * Q * sets + S * (4 + W_N) + M_COUNT);
 }
 
-template <int S, bool WIDE>
+template <int S>
 __global__ void __launch_bounds__(128 * f64_side(S))
     k_step_f64(const __grid_constant__ F64Consts<S> c, const double *__restrict__ fin,
                double *__restrict__ fout, unsigned *__restrict__ flag)
 {
-    constexpr int CELLS = WIDE ? 32 : 8, SW = f64_side(S), NT = 128 * SW, V = WIDE ? 4 : 1;
+    constexpr int CELLS = 32, SW = f64_side(S), NT = 128 * SW, V = 4;
     extern __shared__ __align__(16) double sm[];
     double *mom = sm;                          // [S][4][CELLS]
     double *wts = mom + S * 4 * CELLS;         // [S][W_N][CELLS]
@@ -247,24 +257,15 @@ __global__ void __launch_bounds__(128 * f64_side(S))
         double f[Q], sum;
 #pragma unroll
         for (int i = 0; i < Q; ++i) f[i] = pl[i * P];
-        if constexpr (WIDE) {  // k is uniform over a warp: no products with 1 or 0
-            if (k == 0)
-                sum = moment_sum<0>(c.vr[s], c.qr[s], f);
-            else if (k == 1)
-                sum = moment_sum<1>(c.vr[s], c.qr[s], f);
-            else if (k == 2)
-                sum = moment_sum<2>(c.vr[s], c.qr[s], f);
-            else
-                sum = moment_sum<3>(c.vr[s], c.qr[s], f);
-        } else {
-            sum = 0.0;
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const double v = c.vr[s][i >> 2], q = c.qr[s][i >> 2];
-                const double wx = dir_x(i) == 0 ? 0.0 : dir_x(i) * v, wy = dir_y(i) == 0 ? 0.0 : dir_y(i) * v;
-                sum += f[i] * (k == 0 ? 1.0 : k == 1 ? wx : k == 2 ? wy : q);
-            }
-        }
+        // k is uniform over a warp: no products with 1 or 0
+        if (k == 0)
+            sum = moment_sum<0>(c.vr[s], c.qr[s], f);
+        else if (k == 1)
+            sum = moment_sum<1>(c.vr[s], c.qr[s], f);
+        else if (k == 2)
+            sum = moment_sum<2>(c.vr[s], c.qr[s], f);
+        else
+            sum = moment_sum<3>(c.vr[s], c.qr[s], f);
         mom[(s * 4 + k) * CELLS + j] = sum;
     }
     __syncthreads();
@@ -378,9 +379,11 @@ __global__ void __launch_bounds__(128 * f64_side(S))
     }
     __syncthreads();
 
+    chain_end();
+
     // 5. collision, advection and update of one ring per warp
     const int warp = tid >> 5, lane = tid & 31, r = warp & 3;
-    const int j = lane % CELLS, vel = lane / CELLS;  // vel: 0 when the thread takes all four
+    const int j = lane;
     unsigned x, y;
     const long long cell = locate(j, x, y);
     const bool live = d0 + (unsigned)j < total;
@@ -392,26 +395,26 @@ __global__ void __launch_bounds__(128 * f64_side(S))
         const double v = c.vr[s][r];
         double feq[V], rhs[V], f[V], e1[V], e0[V];
 #pragma unroll
-        for (int q = 0; q < V; ++q) f[q] = fin[(s * Q + 4 * r + (V == 4 ? q : vel)) * P + cell];
+        for (int q = 0; q < V; ++q) f[q] = fin[(s * Q + 4 * r + q) * P + cell];
         const double *fh = fhs + s * Q * CELLS + j;
-        ring_equilibrium<DIAG, V, CELLS>(row, fh, vel, feq);
+        ring_equilibrium<DIAG, V, CELLS>(row, fh, 0, feq);
 #pragma unroll
         for (int q = 0; q < V; ++q) rhs[q] = div_by(-(f[q] - feq[q]), tau);  // Omega
         if (react) {
             fh += SET;
-            ring_equilibrium<DIAG, V, CELLS>(row, fh, vel, e1);
+            ring_equilibrium<DIAG, V, CELLS>(row, fh, 0, e1);
 #pragma unroll
             for (int q = 0; q < V; ++q) rhs[q] = rhs[q] + div_by(e1[q] - feq[q], tau);  // R
         }
         if (force) {
-            ring_equilibrium<DIAG, V, CELLS>(row, fh + SET, vel, e1);
-            ring_equilibrium<DIAG, V, CELLS>(row, fh + 2 * SET, vel, e0);
+            ring_equilibrium<DIAG, V, CELLS>(row, fh + SET, 0, e1);
+            ring_equilibrium<DIAG, V, CELLS>(row, fh + 2 * SET, 0, e0);
 #pragma unroll
             for (int q = 0; q < V; ++q) rhs[q] = rhs[q] + div_by(e1[q] - e0[q], tau);  // G
         }
 #pragma unroll
         for (int q = 0; q < V; ++q) {
-            const int i = V == 4 ? q : vel;
+            const int i = q;
             const long long plane = (long long)(s * Q + 4 * r + i) * P;
             const double *pl = fin + plane + cell;
             const double g0 = v * f[q];
@@ -441,39 +444,296 @@ __global__ void __launch_bounds__(128 * f64_side(S))
 }
 
 // Grids of up to this many cells take the 8-cell split.
-// Grids of up to this many cells, two 8-cell CTAs per SM, take the 8-cell
-// split (us a step, 8-cell / 32-cell: two species 2048 cells 22.8 / 29.0, 4096
-// cells 33.1 / 29.0; four species under a force 59.7 / 74.1, 114 / 74.1).
-constexpr long long NARROW_CELLS = 16 * 152;
-
-template <int S, bool WIDE>
-static int launch_f64_v(dbm_handle *h, const double *fin, double *fout, cudaStream_t st)
+template <int S>
+static int launch_f64_wide(dbm_handle *h, const F64Consts<S> &c, int sets, const double *fin, double *fout,
+                           cudaStream_t st)
 {
-    constexpr int CELLS = WIDE ? 32 : 8;
-    F64Consts<S> c;
-    fill_f64_consts<S>(h, c);
-    const int sets = 1 + (c.has_reaction ? 1 : 0) + (c.has_force ? 2 : 0);
+    constexpr int CELLS = 32;
     const size_t smem = f64_smem<S>(CELLS, sets);
     if (smem > 48 * 1024) {
         static bool attr_set = false;  // per instantiation, set once per process
         if (!attr_set) {
-            cudaError_t e = cudaFuncSetAttribute(k_step_f64<S, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaError_t e = cudaFuncSetAttribute(k_step_f64<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)f64_smem<S>(CELLS, 4));
             if (e != cudaSuccess) return set_cuda_error(h, e, "FP64 step kernel shared-memory attribute");
             attr_set = true;
         }
     }
     const long long cells = (long long)h->p.nx * h->p.ny;
-    return set_cuda_error(h, launch_chained(k_step_f64<S, WIDE>, dim3((unsigned)((cells + CELLS - 1) / CELLS)),
+    return set_cuda_error(h, launch_chained(k_step_f64<S>, dim3((unsigned)((cells + CELLS - 1) / CELLS)),
                                             dim3(128 * f64_side(S)), smem, st, c, fin, fout, (unsigned *)h->scratch),
                           "FP64 step kernel launch");
 }
 
+// ---------------------------------------------------------------------------
+// The FP64 step of a small grid: 4 cells per CTA.
+//
+// Four phase warps run phases 1 to 4, each split so that no warp has more
+// than about 20 FP64 instructions in a row: the products of the moment sums
+// by value and the sums by moment, one quantity of a species per warp, f-hat
+// in four parts.  Meanwhile the ring warps (a ring each; 16 lanes, 4 cells by 4
+// velocities, per species, two species a warp) form the advection terms, which
+// need no moments, and after the last phase the equilibrium and the update.
+// One CTA's chain is then about 11 000 cycles where one thread per item of
+// each phase and 8 cells took 38 000 (two species, us a step: 400 x 1
+// 17.7 -> 9.8; three reacting 31 -> 18).
+// ---------------------------------------------------------------------------
+
+constexpr int SMALL_CELLS = 4;
+__host__ __device__ constexpr int small_ring_warps(int S) { return 4 * ((S + 1) / 2); }
+
+template <int S>
+__global__ void __launch_bounds__(128 + 32 * small_ring_warps(S))
+    k_step_f64_small(const __grid_constant__ F64Consts<S> c, const double *__restrict__ fin,
+                     double *__restrict__ fout, unsigned *__restrict__ flag)
+{
+    constexpr int C = SMALL_CELLS, PHASE = 128;
+    __shared__ double val[S][3][Q][C];     // f, f v (the ring's speed), f q
+    __shared__ double mom[S][4][C];        // n, j_x, j_y, E
+    __shared__ double wts[S][W_N][C];
+    __shared__ double mix[M_COUNT][C];
+    __shared__ double den[C], term[S][C];
+    __shared__ double fhs[4][S][Q][C];
+    const long long P = c.plane;
+    const unsigned d0 = blockIdx.x * (unsigned)C, total = (unsigned)c.nx * (unsigned)c.ny;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool react = c.has_reaction != 0, force = c.has_force != 0;
+    auto locate = [&](int j, unsigned &x, unsigned &y) {
+        const unsigned d = min(d0 + (unsigned)j, total - 1u);
+        y = d / (unsigned)c.nx;
+        x = d - y * (unsigned)c.nx;
+        return (long long)(y + GY) * c.pitch + (x + GX);
+    };
+    chain_begin();
+
+    if (tid < PHASE) {
+        auto phase_sync = [] { asm volatile("barrier.sync 1, 128;" ::: "memory"); };
+        // 1. values and their products, one per thread; then the sums
+#pragma unroll 1
+        for (int it = tid; it < S * Q * C; it += PHASE) {
+            const int j = it & 3, i = (it >> 2) & 15, s = it >> 6;
+            unsigned x, y;
+            const double f = fin[(long long)(s * Q + i) * P + locate(j, x, y)];
+            val[s][0][i][j] = f;
+            val[s][1][i][j] = f * c.vr[s][i >> 2];
+            val[s][2][i][j] = f * c.qr[s][i >> 2];
+        }
+        phase_sync();
+        {  // warp q and its upper half take species q and q + 4; lane: cell and moment
+            const int j = lane & 3, k = (lane >> 2) & 3, s = warp + 4 * (lane >> 4);
+            if (s < S) {
+                double sum = 0.0;
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const double f = val[s][k == 0 ? 0 : k == 3 ? 2 : 1][i][j];
+                    const int d = k == 1 ? dir_x(i) : k == 2 ? dir_y(i) : 1;
+                    sum = sum + (d < 0 ? -f : d == 0 ? 0.0 : f);
+                }
+                mom[s][k][j] = sum;
+            }
+        }
+        phase_sync();
+        // 2. one quantity per warp; lane: cell and species
+        const int j = lane & 3, s = lane >> 2;
+        const bool mine = s < S;
+        const int q = mine ? s : 0;  // species constants of an idle lane
+        if (mine) {
+            const double sn = mom[s][0][j];
+            const double rho = c.md[q].b * sn;
+            if (warp == 0) {
+                const double ux = sn != 0.0 ? mom[s][1][j] / sn : 0.0;  // an absent species: zero velocity
+                wts[s][W_UX][j] = ux;
+                wts[s][W_LX][j] = div_by(rho * ux, c.taud[q]);
+            } else if (warp == 1) {
+                const double uy = sn != 0.0 ? mom[s][2][j] / sn : 0.0;
+                wts[s][W_UY][j] = uy;
+                wts[s][W_LY][j] = div_by(rho * uy, c.taud[q]);
+            } else if (warp == 2) {
+                wts[s][W_RHO][j] = rho;
+                wts[s][W_LAM][j] = div_by(rho, c.taud[q]);
+                wts[s][W_ME][j] = c.md[q].b * mom[s][3][j];
+            } else {
+                wts[s][W_CAP][j] = div_by(sn * (2.0 + c.I[q]), c.taud[q]);
+            }
+        }
+        phase_sync();
+        // 3. mixture u, the denominator of T
+        if (lane < C) {
+            if (warp <= 1) {
+                double sw = 0.0, sx = 0.0;
+#pragma unroll
+                for (int k = 0; k < S; ++k) {
+                    sw += wts[k][W_LAM][lane];
+                    sx += wts[k][warp == 0 ? W_LX : W_LY][lane];
+                }
+                mix[M_UX + warp][lane] = sx / sw;
+            } else if (warp == 2) {
+                double d = 0.0, ntot = 0.0;
+#pragma unroll
+                for (int k = 0; k < S; ++k) {
+                    d += wts[k][W_CAP][lane];
+                    ntot += fabs(mom[k][0][lane]);
+                }
+                den[lane] = d;
+                mix[M_NTOT][lane] = ntot;
+            }
+        }
+        if (force && warp == 3 && mine) {
+            const double sn = mom[s][0][j];
+            double Ts = 0.0;
+            if (sn != 0.0) {
+                const double ux = wts[s][W_UX][j], uy = wts[s][W_UY][j];
+                Ts = c.md[q].b * (mom[s][3][j] / sn - (ux * ux + uy * uy)) / (2.0 + c.I[q]);
+            }
+            wts[s][W_TS][j] = Ts;
+        }
+        phase_sync();
+        if (warp == 0) {
+            if (mine) {
+                const double Ux = mix[M_UX][j], Uy = mix[M_UY][j];
+                const double u2 = Ux * Ux + Uy * Uy;
+                term[s][j] = div_by(wts[s][W_ME][j] - wts[s][W_RHO][j] * u2, c.taud[q]);
+            }
+            __syncwarp();
+            if (lane < C) {
+                const double Ux = mix[M_UX][lane], Uy = mix[M_UY][lane], ntot = mix[M_NTOT][lane];
+                double num = 0.0;
+#pragma unroll
+                for (int k = 0; k < S; ++k) num += term[k][lane];
+                const double T = num / den[lane];
+                unsigned bad = 0;
+#pragma unroll
+                for (int k = 0; k < S; ++k) {
+                    const double n = mom[k][0][lane];
+                    if (!(n >= -1e-6 * ntot) || !isfinite(n)) bad |= DBM_HEALTH_DENSITY;
+                }
+                if (!(ntot > 0.0)) bad |= DBM_HEALTH_DENSITY;
+                if (!(T > 0.0)) bad |= DBM_HEALTH_TEMPERATURE;
+                if (!isfinite(T) || !isfinite(Ux) || !isfinite(Uy)) bad |= DBM_HEALTH_NONFINITE;
+                double omega = 0.0, dTdt = 0.0;
+                if (react) {
+                    omega = c.k_ov * mom[c.fuel][0][lane] * mom[c.oxid][0][lane] * exp(-c.Ea_over_R / T);
+                    double src = 0.0, cap = 0.0;
+#pragma unroll
+                    for (int k = 0; k < S; ++k) {
+                        src += (2.0 + c.I[k]) * c.a[k] * omega;
+                        cap += mom[k][0][lane] * (2.0 + c.I[k]);
+                    }
+                    dTdt = (c.Qheat * omega - 0.5 * T * src) / (0.5 * cap);
+                }
+                mix[M_T][lane] = T;
+                mix[M_OMEGA][lane] = omega;
+                mix[M_DT][lane] = dTdt;
+                if (bad) raise_flag(flag, bad);
+            }
+        }
+        phase_sync();
+        // 4. f-hat: a part per warp; lane: cell and species
+        if (mine) {
+            const double n = mom[s][0][j], Ux = mix[M_UX][j], Uy = mix[M_UY][j], T = mix[M_T][j];
+            const double tau = c.taud[q].b;
+            auto part = [&](int set, double n_, double ux, double uy, double t) {
+                double *fh = &fhs[set][s][0][j];
+                if (warp == 0)
+                    fhat_printed<0>(n_, ux, uy, t, c.md[q], c.I[q], fh, C);
+                else if (warp == 1)
+                    fhat_printed<1>(n_, ux, uy, t, c.md[q], c.I[q], fh, C);
+                else if (warp == 2)
+                    fhat_printed<2>(n_, ux, uy, t, c.md[q], c.I[q], fh, C);
+                else
+                    fhat_printed<3>(n_, ux, uy, t, c.md[q], c.I[q], fh, C);
+            };
+            part(0, n, Ux, Uy, T);
+            if (react) {
+                const double nstar = n + tau * c.a[q] * mix[M_OMEGA][j];
+                if (warp == 0 && nstar < -1e-6 * mix[M_NTOT][j]) raise_flag(flag, DBM_HEALTH_NSTAR);
+                part(1, nstar, Ux, Uy, T + tau * mix[M_DT][j]);
+            }
+            if (force) {
+                const double ux = wts[s][W_UX][j], uy = wts[s][W_UY][j], Ts = wts[s][W_TS][j];
+                part(2, n, ux + c.ax * tau, uy + c.ay * tau, Ts);
+                part(3, n, ux, uy, Ts);
+            }
+        }
+        __syncthreads();
+        chain_end();
+        return;
+    }
+
+    // 5. a ring per warp, a velocity of a cell and species per lane
+    const int r = warp & 3, j = lane & 3, i = (lane >> 2) & 3;
+    const int s = 2 * ((warp - 4) >> 2) + (lane >> 4);
+    const bool mine = s < S;
+    const int q = mine ? s : 0;
+    unsigned x, y;
+    const long long cell = locate(j, x, y);
+    const long long plane = (long long)(q * Q + 4 * r + i) * P;
+    const double *pl = fin + plane + cell;
+    const double f = pl[0], v = c.vr[q][r];
+    double adv;
+    {
+        const double g0 = v * f;
+        if (r & 1) {
+            const int ex = (i == 1 || i == 2) ? -1 : 1, ey = (i == 2 || i == 3) ? -c.pitch : c.pitch;
+            adv = nnd_dflux(pl[-2 * ex], pl[-ex], pl[ex], g0, v, c.dxd);
+            adv += nnd_dflux(pl[-2 * ey], pl[-ey], pl[ey], g0, v, c.dyd);
+        } else {
+            const int st = (i & 1) ? c.pitch : 1, e = (i & 2) ? -st : st;
+            const ConstDiv h = (i & 1) ? c.dyd : c.dxd;
+            adv = nnd_dflux(pl[-2 * e], pl[-e], pl[e], g0, v, h);
+        }
+    }
+    __syncthreads();
+    chain_end();
+    auto equilibrium = [&](int set) {
+        double e[1];
+        if (r & 1)
+            ring_equilibrium<true, 1, C>(c.row[q][r], &fhs[set][q][0][j], i, e);
+        else
+            ring_equilibrium<false, 1, C>(c.row[q][r], &fhs[set][q][0][j], i, e);
+        return e[0];
+    };
+    const ConstDiv tau = c.taud[q];
+    const double feq = equilibrium(0);
+    double rhs = div_by(-(f - feq), tau);                                 // Omega
+    if (react) rhs = rhs + div_by(equilibrium(1) - feq, tau);             // R
+    if (force) {
+        const double g1 = equilibrium(2), g0 = equilibrium(3);
+        rhs = rhs + div_by(g1 - g0, tau);                                 // G
+    }
+    const double fnew = f + c.dt * (rhs - adv);
+    if (!mine || d0 + (unsigned)j >= total) return;
+    double *po = fout + plane;
+    po[cell] = fnew;
+    const unsigned mx = ghost_mask((int)x, c.nx, c.bc_x), my = ghost_mask((int)y, c.ny, c.bc_y);
+    if (mx | my) store_images(po, (int)x, (int)y, c.nx, c.ny, c.pitch, mx, my, fnew);
+}
+
+// Grids of up to this many cells take the 4-cell kernel (us a step, 4 cells /
+// 32 cells: two species 2048 cells 20.2 / 25.7, 3000 cells 27.6 / 25.8; four under
+// a force 63 / 71, 76 / 71).
+constexpr long long SMALL_GRID = 16 * 152;
+
 template <int S>
 static int launch_f64_t(dbm_handle *h, const double *fin, double *fout, cudaStream_t st)
 {
-    if ((long long)h->p.nx * h->p.ny <= NARROW_CELLS) return launch_f64_v<S, false>(h, fin, fout, st);
-    return launch_f64_v<S, true>(h, fin, fout, st);
+    F64Consts<S> c;
+    fill_f64_consts<S>(h, c);
+    const long long cells = (long long)h->p.nx * h->p.ny;
+    if (cells > SMALL_GRID)
+        return launch_f64_wide<S>(h, c, 1 + (c.has_reaction ? 1 : 0) + (c.has_force ? 2 : 0), fin, fout, st);
+    static bool attr_set = false;  // per instantiation, set once per process
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(k_step_f64_small<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)ALONE_SMEM);
+        if (e != cudaSuccess) return set_cuda_error(h, e, "FP64 small-grid step kernel shared-memory attribute");
+        attr_set = true;
+    }
+    const long long ctas = (cells + SMALL_CELLS - 1) / SMALL_CELLS;
+    return set_cuda_error(h, launch_chained(k_step_f64_small<S>, dim3((unsigned)ctas),
+                                            dim3(128 + 32 * small_ring_warps(S)), ctas <= h->sms ? ALONE_SMEM : 0, st, c,
+                                            fin, fout, (unsigned *)h->scratch),
+                          "FP64 small-grid step kernel launch");
 }
 
 int launch_step_f64(dbm_handle *h, int cur, cudaStream_t st)

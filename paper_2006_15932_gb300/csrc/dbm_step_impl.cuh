@@ -872,6 +872,7 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
 #pragma unroll(S <= 3 ? S : 1)
     for (int s = 0; s < S; ++s) {
         if constexpr (kStaged) t.acquire(S + s);
+        if (s == S - 1) chain_end();
         const auto &ts = stage_view(t, S + s, s);
         V f0[Q];
 #pragma unroll

@@ -1,4 +1,4 @@
-"""The FP64 step's two splits (8 cells per CTA on small grids, 32 on the
+"""The FP64 step's two kernels (4 cells per CTA on small grids, 32 on the
 rest) at their edges against the FP64 oracle.
 
 Tolerance: the kernel evaluates every formula in the oracle's order, each
