@@ -109,6 +109,7 @@ struct dbm_handle {
     int tma_cw;           // fixed at dbm_bind
     int told_tx, told_ty, told_cw;  // what dbm_step_tile answers (choose_tile)
     int tma_staged;       // the species-staged step (one species per copy)
+    int tma_half;         // two threads per pair of cells (k_step_half)
     int sms;              // SMs of the device current at dbm_bind
     double cinv[DBM_MAX_SPECIES][16][16];  // host FP64 M^-1 per species
     double eqA[DBM_MAX_SPECIES][4][4];     // symmetry blocks of M^-1
@@ -164,6 +165,10 @@ constexpr int PAIR_TX = 64, PAIR_TY = 8;
 #endif
 constexpr int STAGED_TX = DBM_STAGED_TX, STAGED_TY = DBM_STAGED_TY;
 constexpr long long PAIR_MIN_TILES = 4096, PAIR_MIN_RUN = 128;
+// Small grids of two and four species: two threads per pair of cells on
+// SMALL_TX x SMALL_TY tiles (k_step_half; 32 x 8 on 128^2, two species, 6.6 us
+// a step against 6.2).
+constexpr int SMALL_TX = 32, SMALL_TY = 4;
 
 // CTAs of a TX x TY tile kernel that fit on one SM at once, limited by
 // shared memory (the tile plus halo of 16 S float planes, and 1 KB reserved

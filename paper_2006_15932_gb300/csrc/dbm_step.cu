@@ -14,6 +14,9 @@ template <int S, int TX, int TY, int CW, int MODE>
 int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin, void *fout,
                       cudaStream_t st);
 template <int S, int TX, int TY>
+int launch_step_half_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin, void *fout,
+                       cudaStream_t st);
+template <int S, int TX, int TY>
 int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin,
                          void *fout, cudaStream_t st);
 
@@ -39,6 +42,9 @@ template <int MODE>
 static int launch_tma(dbm_handle *h, const CUtensorMap *tm, const CUtensorMap *ti, const void *fin, void *fout,
                       cudaStream_t st)
 {
+    if (h->tma_half)
+        return h->p.nspecies == 2 ? launch_step_half_t<2, SMALL_TX, SMALL_TY>(h, tm, ti, fin, fout, st)
+                                  : launch_step_half_t<4, SMALL_TX, SMALL_TY>(h, tm, ti, fin, fout, st);
     switch (h->p.nspecies) {
     case 1: return launch_step_tma_t<1, tma_tile_x(1), tma_tile_y(1), 1, MODE>(h, tm, ti, fin, fout, st);
     case 2:
@@ -59,15 +65,22 @@ static bool staged_supported(const dbm_params &p)
     return p.precision == DBM_FP32 && p.nspecies >= 2 && p.nspecies <= DBM_MAX_SPECIES && !uses_acc(p);
 }
 
-// The tile of the TMA-staged step.  Two species: two cells per thread from
-// PAIR_MIN_RUN tiles up (us a step, one cell / pairs: 4096^2 845 / 726, 1024^2
-// 69 / 60, 1001 x 771 51 / 45, 512^2 20.0 / 18.3, 256^2, 128 tiles, 10.6 / 9.9;
-// below, a thread's longer chain shows: 128^2 9.6 / 10.1), the one-cell tile
-// when asked for; with an arithmetic option pairs from PAIR_MIN_TILES tiles.
-// Three and four species: the one-cell tile (2048 x 1024, one cell / species-
-// staged: three species 174 / 201, four 261 / 265), the species-staged one
-// when two cells per thread are asked for.  Five or more: the species-staged
-// kernel, the only TMA-staged one.
+// The tile of the TMA-staged step, without the arithmetic options:
+// two species: two cells per thread from PAIR_MIN_RUN tiles up (us a step,
+//   one cell / pairs: 4096^2 845 / 726, 1024^2 68 / 60, 1001 x 771 51 / 45,
+//   512^2 20.0 / 17.7, 256^2, 128 tiles, 9.1 / 8.1), below that two threads per
+//   pair, whose chain is the shortest (one cell / two threads: 256 x 200 9.1 /
+//   6.4, 128^2 7.4 / 5.8, 64^2 7.4 / 4.4, 400 x 1 6.6 / 5.3);
+// one and three species: one cell per thread (three species, two threads per
+//   pair: 128^2 7.5 / 8.0, 256^2 9.9 / 14.6; species-staged: 2048 x 1024 174 /
+//   201);
+// four: one cell per thread (2048 x 1024 261, species-staged 265), two threads
+//   per pair on grids of at most a small tile per SM (128^2 10.7 / 8.3, 777 x
+//   413 62 / 91);
+// five or more: the species-staged kernel, the only TMA-staged one.
+// DBM_KERNEL_TMA_CELL asks for one cell per thread, DBM_KERNEL_TMA_PAIR and
+// _STAGED for two.  With an option: two species pairs from PAIR_MIN_TILES
+// tiles up, else one cell.
 //
 // dbm_step_tile's answer is fixed by its own rule, older than pairs on small
 // grids: it names the pair tile for two species from PAIR_MIN_TILES tiles up
@@ -76,7 +89,7 @@ static void choose_tile(dbm_handle *h)
 {
     const dbm_params &p = h->p;
     const int want = p.step_kernel;
-    h->tma_staged = 0;
+    h->tma_staged = h->tma_half = 0;
     const bool staged_by_default = p.nspecies > 4 && want != DBM_KERNEL_TMA_CELL;
     const bool staged_asked = want == DBM_KERNEL_TMA_STAGED || (p.nspecies >= 3 && want == DBM_KERNEL_TMA_PAIR);
     if (staged_supported(p) && (staged_by_default || staged_asked)) {
@@ -92,8 +105,12 @@ static void choose_tile(dbm_handle *h)
         told_pair = want == DBM_KERNEL_TMA_PAIR || tiles >= PAIR_MIN_TILES;
         pair = told_pair || (!uses_acc(p) && tiles >= PAIR_MIN_RUN);
     }
-    h->tma_tx = pair ? PAIR_TX : tma_tile_x(p.nspecies);
-    h->tma_ty = pair ? PAIR_TY : tma_tile_y(p.nspecies);
+    if (!uses_acc(p) && want != DBM_KERNEL_TMA_CELL && !pair) {
+        const long long small = (long long)((p.nx + SMALL_TX - 1) / SMALL_TX) * ((p.ny + SMALL_TY - 1) / SMALL_TY);
+        h->tma_half = p.nspecies == 2 || (p.nspecies == 4 && small <= h->sms);
+    }
+    h->tma_tx = pair ? PAIR_TX : h->tma_half ? SMALL_TX : tma_tile_x(p.nspecies);
+    h->tma_ty = pair ? PAIR_TY : h->tma_half ? SMALL_TY : tma_tile_y(p.nspecies);
     h->tma_cw = pair ? 2 : 1;
     h->told_tx = told_pair ? PAIR_TX : tma_tile_x(p.nspecies);
     h->told_ty = told_pair ? PAIR_TY : tma_tile_y(p.nspecies);

@@ -215,6 +215,17 @@ template <class T>
 struct is_split<T, std::void_t<decltype(T::kSplit)>> : std::true_type {
 };
 
+// A tile whose pairs of cells are stepped by two threads (HalfTile): thread
+// kHalf owns rings 2 kHalf and 2 kHalf + 1.  -1: one thread owns all four.
+template <class T, class = void>
+struct half_of {
+    static constexpr int v = -1;
+};
+template <class T>
+struct half_of<T, std::void_t<decltype(T::kHalf)>> {
+    static constexpr int v = T::kHalf;
+};
+
 template <class Tile>
 __device__ __forceinline__ decltype(auto) stage_view(const Tile &t, int k, int s)
 {
@@ -680,6 +691,24 @@ static_assert(dir_x(0) == 1 && dir_y(1) == 1 && dir_x(2) == -1 && dir_y(3) == -1
                   dir_x(6) == -1 && dir_y(6) == -1 && dir_x(7) == 1 && dir_y(7) == -1,
               "D2V16 ring order");
 
+// Sums of ring r of species s at the thread's cells: all four values, and the
+// x and y vector parts.
+template <class Tile, class V>
+__device__ __forceinline__ void ring_terms(const Tile &t, int s, int r, V &rs, V &rx, V &ry)
+{
+    const V f0 = t.ld(s * Q + 4 * r, 0, 0), f1 = t.ld(s * Q + 4 * r + 1, 0, 0);
+    const V f2 = t.ld(s * Q + 4 * r + 2, 0, 0), f3 = t.ld(s * Q + 4 * r + 3, 0, 0);
+    rs = vadd(vadd(f0, f2), vadd(f1, f3));
+    if ((r & 1) == 0) {
+        rx = vsub(f0, f2);
+        ry = vsub(f1, f3);
+    } else {
+        const V a = vsub(f0, f2), b = vsub(f3, f1);
+        rx = vadd(a, b);
+        ry = vsub(a, b);
+    }
+}
+
 // The whole update of cell (x, y), or of the cells (x, y) and (x + 1, y)
 // when the tile delivers pairs (Tile::V = float2; `two` false when x + 1 is
 // outside the domain: that half is computed but neither stored nor checked).
@@ -702,28 +731,39 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
     constexpr bool kStaged = is_staged<Tile>::value;
     static_assert(!(kStaged && X::on), "the arithmetic options read every species at once");
 
+    constexpr int kHalf = half_of<Tile>::v;
+    static_assert(kHalf < 0 || (!kStaged && !X::on), "two threads per pair: the default arithmetic, every species at once");
+    // ring r, velocity i: this thread's
+    const auto my_ring = [](int r) { return kHalf < 0 || (r >> 1) == kHalf; };
+
     // 1. species moments, by ring sums
     V n[S], nf = bc<V>(0.0f), no = bc<V>(0.0f), cap, w, wx, wy, we, wd;
+    V rall[S][4], rvx[S][4], rvy[S][4];  // ring sums: of all values, of the vector part
+    if constexpr (kHalf >= 0) {          // every own ring sum before the first exchange
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            t.arrived(s);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (my_ring(r)) ring_terms(t, s, r, rall[s][r], rvx[s][r], rvy[s][r]);
+        }
+        if constexpr (kHalf == 1) t.partials_wait();
+    }
 #pragma unroll
     for (int s = 0; s < S; ++s) {
         if constexpr (kStaged) t.acquire(s);
-        if constexpr (is_split<Tile>::value) t.arrived(s);
+        if constexpr (is_split<Tile>::value && kHalf < 0) t.arrived(s);
         const auto &ts = stage_view(t, s, s);
         V sn, sx, sy, se;
+        if constexpr (kHalf == 1) t.take(s, sn, sx, sy, se);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const V f0 = ts.ld(s * Q + 4 * r, 0, 0), f1 = ts.ld(s * Q + 4 * r + 1, 0, 0);
-            const V f2 = ts.ld(s * Q + 4 * r + 2, 0, 0), f3 = ts.ld(s * Q + 4 * r + 3, 0, 0);
-            const V rs = vadd(vadd(f0, f2), vadd(f1, f3));
-            V rx, ry;
-            if ((r & 1) == 0) {
-                rx = vsub(f0, f2);
-                ry = vsub(f1, f3);
-            } else {
-                const V a = vsub(f0, f2), b = vsub(f3, f1);
-                rx = vadd(a, b);
-                ry = vsub(a, b);
-            }
+            if (!my_ring(r)) continue;
+            V rs, rx, ry;
+            if constexpr (kHalf >= 0)
+                rs = rall[s][r], rx = rvx[s][r], ry = rvy[s][r];
+            else
+                ring_terms(ts, s, r, rs, rx, ry);
             if (r == 0) {
                 sn = rs;
                 sx = vmul(bc<V>(c.vr[s][0]), rx);
@@ -737,6 +777,10 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
             }
         }
         if constexpr (kStaged) t.release(s);
+        if constexpr (kHalf == 0) {  // the other thread of the pair adds its rings and goes on to the mixture
+            t.give(s, sn, sx, sy, se);
+            continue;
+        }
         n[s] = sn;
         if (s == g.fuel) nf = sn;  // selects, no runtime-indexed register array
         if (s == g.oxid) no = sn;
@@ -754,13 +798,17 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
     }
 
     // 2. mixture velocity and temperature (per cell: division, float-float T)
-    V rw, T;
+    V rw, T, ux, uy, om = bc<V>(0.0f), dT = bc<V>(0.0f), a;  // a: sum_s |n^s|
+    unsigned bad = 0;
+    if constexpr (kHalf == 0) t.partials_done();
+    if constexpr (kHalf != 0) {
 #pragma unroll
     for (int j = 0; j < L::n; ++j) L::set(rw, j, 1.0f / L::get(w, j));
-    V ux = vmul(wx, rw), uy = vmul(wy, rw);
+    ux = vmul(wx, rw), uy = vmul(wy, rw);
 #pragma unroll
     for (int j = 0; j < L::n; ++j)
         L::set(T, j, mixture_T(L::get(we, j), L::get(w, j), L::get(wd, j), L::get(ux, j), L::get(uy, j)));
+    }
     // DBM_THERMO_FP64: n^s, u and T from double sums replace the float ones
     double n64[S][L::n], T64[L::n], cap64[L::n], om64[L::n], dT64[L::n];
     unsigned hcell[L::n];  // per-cell hash of the stochastic rounding
@@ -806,8 +854,7 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
         }
     }
 
-    unsigned bad = 0;
-    V a;  // sum_s |n^s|
+    if constexpr (kHalf != 0) {
 #pragma unroll
     for (int j = 0; j < L::n; ++j) {
         float aj = 0.0f;
@@ -823,9 +870,9 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
             if (!isfinite(L::get(T, j) + L::get(ux, j) + L::get(uy, j))) bad |= DBM_HEALTH_NONFINITE;
         }
     }
+    }
 
     // 3. reaction: omega_ov and T' (state after a time tau^s)
-    V om = bc<V>(0.0f), dT = bc<V>(0.0f);
     if constexpr (X::on) {
         if (t64 && g.has_reaction) {  // the Arrhenius rate and T' in double
 #pragma unroll
@@ -842,7 +889,7 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
             }
         }
     }
-    if (g.has_reaction && !t64) {
+    if (kHalf != 0 && g.has_reaction && !t64) {
 #pragma unroll
         for (int j = 0; j < L::n; ++j) {
             const float Tj = L::get(T, j);
@@ -853,6 +900,9 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
                        __fmul_rn(0.5f, L::get(cap, j)));
         }
     }
+
+    if constexpr (kHalf == 1) t.template give_mixture<S>(n, ux, uy, T, om, dT);
+    if constexpr (kHalf == 0) t.template take_mixture<S>(n, ux, uy, T, om, dT);
 
     Site w_;
     w_.x = x;
@@ -876,7 +926,8 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
         const auto &ts = stage_view(t, S + s, s);
         V f0[Q];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) f0[i] = ts.ld(s * Q + i, 0, 0);
+        for (int i = 0; i < Q; ++i)
+            if (my_ring(i >> 2)) f0[i] = ts.ld(s * Q + i, 0, 0);
         // species density from step 1 (selected, not indexed)
         V ns = n[0];
 #pragma unroll
@@ -914,7 +965,8 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
                 }
 #pragma unroll
                 for (int j = 0; j < L::n; ++j)
-                    if ((j == 0 || two) && L::get(nr, j) < -1e-6f * L::get(a, j)) bad |= DBM_HEALTH_NSTAR;
+                    if (kHalf != 0 && (j == 0 || two) && L::get(nr, j) < -1e-6f * L::get(a, j))
+                        bad |= DBM_HEALTH_NSTAR;
             }
             fhat_blocks<V>(nr, ux, uy, vmul(Ts, bc<V>(c.inv_m[s])), c.dpi[s], cb);
             if constexpr (X::on) {
@@ -944,9 +996,10 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
                     const float v = c.vr[s][i >> 2];
-                    e = i == 0 ? vmul(bc<V>(c.qr[s][0]), f0[0]) : vfma(bc<V>(c.qr[s][i >> 2]), f0[i], e);
-                    if (dir_x(i) != 0) jx = i == 0 ? vmul(bc<V>(dir_x(i) * v), f0[i]) : vfma(bc<V>(dir_x(i) * v), f0[i], jx);
-                    if (dir_y(i) != 0) jy = i == 1 ? vmul(bc<V>(dir_y(i) * v), f0[i]) : vfma(bc<V>(dir_y(i) * v), f0[i], jy);
+                    const V fi = my_ring(i >> 2) ? f0[i] : ts.ld(s * Q + i, 0, 0);
+                    e = i == 0 ? vmul(bc<V>(c.qr[s][0]), fi) : vfma(bc<V>(c.qr[s][i >> 2]), fi, e);
+                    if (dir_x(i) != 0) jx = i == 0 ? vmul(bc<V>(dir_x(i) * v), fi) : vfma(bc<V>(dir_x(i) * v), fi, jx);
+                    if (dir_y(i) != 0) jy = i == 1 ? vmul(bc<V>(dir_y(i) * v), fi) : vfma(bc<V>(dir_y(i) * v), fi, jy);
                 }
                 V usx, usy, th;
 #pragma unroll
@@ -987,6 +1040,7 @@ __device__ __forceinline__ void step_cell(const K &c, const G &g, const Tile &t,
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int p = s * Q + i, r = i >> 2;
+            if (!my_ring(r)) continue;
             // 6. forward Euler: f + dt/tau (f^eq,tot - f) - dt v . grad f,
             // with the 5. NND advection terms of x and y each applied as one
             // fused multiply-add (no product is left for the compiler to fuse)
@@ -1393,6 +1447,151 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     }
 }
 
+// ---------------------------------------------------------------------------
+// The two-thread step of small grids: a pair of cells takes two threads, each
+// with two of the four rings of every species.  On a grid that leaves the chip
+// idle the time is one thread's chain of instructions: about 1560 for a cell
+// of two species, 1900 for a pair, 1030 for half of a pair (f-hat and half of
+// the block solve are formed twice).  A warp is two rows of 16 pairs and one
+// half, so the rings' constants stay constant-bank operands; the two warps of
+// a row pair exchange, through shared memory and a barrier of their 64
+// threads, the partial moment sums (half 0 to half 1, which adds its rings in
+// the same order as one thread would) and the mixture (back).  A boundary
+// tile's halo is loaded beside its copies.  Same bits.  Two species, us a
+// step: 128^2 7.4 (one cell) -> 5.8.  On grids that fill the chip the second
+// copy of the step's code and the exchange cost more than the shorter threads
+// give (three species 1024^2 97 -> 119).
+// the tile, then the exchange area: 4 S pairs per pair of cells
+constexpr size_t half_smem(int S, int TX, int TY)
+{
+    return (size_t)(TX + 8) * (TY + 4) * S * Q * sizeof(float) + (size_t)TX / 2 * TY * 4 * S * sizeof(float2);
+}
+
+template <class Base, int HALF>
+struct HalfTile : Base {
+    static constexpr int kHalf = HALF;
+    float2 *ex;  // this pair's column of the exchange area
+    int stride;  // pairs of the tile
+    int id;      // named barriers id (partial sums) and id + 4 (mixture) of the two warps
+    __device__ __forceinline__ void partials_done() const  // half 0
+    {
+        asm volatile("barrier.arrive %0, 64;" ::"r"(id) : "memory");
+    }
+    __device__ __forceinline__ void partials_wait() const  // half 1
+    {
+        asm volatile("barrier.sync %0, 64;" ::"r"(id) : "memory");
+    }
+    __device__ __forceinline__ void give(int s, float2 n, float2 jx, float2 jy, float2 e) const
+    {
+        float2 *q = ex + 4 * s * stride;
+        q[0] = n, q[stride] = jx, q[2 * stride] = jy, q[3 * stride] = e;
+    }
+    __device__ __forceinline__ void take(int s, float2 &n, float2 &jx, float2 &jy, float2 &e) const
+    {
+        const float2 *q = ex + 4 * s * stride;
+        n = q[0], jx = q[stride], jy = q[2 * stride], e = q[3 * stride];
+    }
+    // half 1, after its last take: the area now carries the mixture back
+    template <int S>
+    __device__ __forceinline__ void give_mixture(const float2 n[S], float2 ux, float2 uy, float2 T, float2 om,
+                                                 float2 dT) const
+    {
+        static_assert(5 + S <= 4 * S, "exchange area");
+        ex[0] = ux, ex[stride] = uy, ex[2 * stride] = T, ex[3 * stride] = om, ex[4 * stride] = dT;
+#pragma unroll
+        for (int s = 0; s < S; ++s) ex[(5 + s) * stride] = n[s];
+        asm volatile("barrier.arrive %0, 64;" ::"r"(id + 4) : "memory");
+    }
+    template <int S>
+    __device__ __forceinline__ void take_mixture(float2 n[S], float2 &ux, float2 &uy, float2 &T, float2 &om,
+                                                 float2 &dT) const
+    {
+        asm volatile("barrier.sync %0, 64;" ::"r"(id + 4) : "memory");
+        ux = ex[0], uy = ex[stride], T = ex[2 * stride], om = ex[3 * stride], dT = ex[4 * stride];
+#pragma unroll
+        for (int s = 0; s < S; ++s) n[s] = ex[(5 + s) * stride];
+    }
+};
+
+// Output of a kernel whose every thread runs the step because its barriers
+// sit inside it: one outside the domain (the ragged edge of a tile) computes
+// on in-range shared-memory values and stores nothing.
+struct MaskedOut : StateOutNoImages {
+    bool live;
+    template <class G>
+    __device__ __forceinline__ void put(const Site &w, int p, G g, G e) const
+    {
+        if (live) StateOutNoImages::put(w, p, g, e);
+    }
+};
+
+template <int S, int TX, int TY>
+__global__ void __launch_bounds__(TX *TY, 2)
+    k_step_half(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
+                const __grid_constant__ CUtensorMap tmap_in, const float *__restrict__ fin, float *__restrict__ fout,
+                unsigned *__restrict__ flag)
+{
+    constexpr int BX = TX + 8, BY = TY + 4, NP = S * Q, NT = TX * TY, W = NT / 64;
+    constexpr unsigned BYTES = (unsigned)(BX * BY * Q * sizeof(float));  // one species
+    static_assert(TX == 32 && TY % 2 == 0 && TY <= 8, "a warp is two rows of 16 pairs; barriers 1 .. 8");
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) unsigned long long bar[S];
+    __shared__ unsigned health_sink;
+    float *tile = reinterpret_cast<float *>(smem_raw);
+    float2 *ex = reinterpret_cast<float2 *>(tile + NP * BX * BY);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = warp / W, wl = warp - half * W;
+    const int bx0 = blockIdx.x * TX, by0 = blockIdx.y * TY;
+    const unsigned b = smem_u32(&bar[0]);
+    if (tid == 0) {
+        for (int s = 0; s < S; ++s)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b + 8u * s) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    chain_begin();
+    if (tid == 0) {
+        for (int s = 0; s < S; ++s)
+            tma_tile_load(tile + s * Q * BX * BY, reinterpret_cast<unsigned long long>(&tmap), bx0, by0, b + 8u * s,
+                          BYTES, s * Q);
+        prefetch_ahead<S, TX, TY>(c.prefetch, reinterpret_cast<unsigned long long>(&tmap_in));
+    }
+    __syncthreads();
+    const HaloSides hs = halo_sides<TX, TY>(bx0, by0, c.nx, c.ny);
+    HaloRegs<NP, TX, TY, NT> hr;  // a boundary tile's halo, fetched beside its copies
+    if (hs.any())
+        halo_load(hr, hs, fin, bx0, by0, c.nx, c.ny, c.pitch, c.plane, c.bc_x, c.bc_y, tid, flag);
+    const bool ok = mbar_wait(b, 0, c.wait_polls);
+    if (__syncthreads_or(!ok)) {
+        // as in k_step_tma
+        if (tid == 0) raise_flag(flag, DBM_HEALTH_TIMEOUT);
+        for (int s = 0; s < S; ++s) mbar_wait(b + 8u * s, 0, TMA_WAIT_LIMIT);
+        return;
+    }
+    if (hs.any()) {
+        for (int s = 1; s < S; ++s)
+            if (!mbar_wait(b + 8u * s, 0, TMA_WAIT_LIMIT)) raise_flag(flag, DBM_HEALTH_TIMEOUT);
+        halo_store(hr, hs, tile, bx0, by0, c.nx, c.ny, tid, flag);
+    }
+    if (by0 + 2 * wl >= c.ny) {  // both warps of a row pair outside the domain leave
+        for (int s = 1; s < S; ++s) mbar_wait(b + 8u * s, 0, TMA_WAIT_LIMIT);
+        return;
+    }
+    const int row = 2 * wl + (lane >> 4), col = 2 * (lane & 15);
+    const int x = bx0 + col, y = by0 + row;
+    const bool live = x < c.nx && y < c.ny;
+    const MaskedOut o{{fout, c.plane, (long long)NP * c.plane, flag}, live};
+    unsigned *health = live ? flag : &health_sink;
+    const float *base = tile + (row + 2) * BX + (col + 4);
+    const SplitTile<SmemTile2> t{{base, BY * BX, BX, tile, NP * BY * BX, flag}, b, 0u};
+    float2 *mine = ex + row * (TX / 2) + (lane & 15);
+    if (half == 0) {
+        const HalfTile<SplitTile<SmemTile2>, 0> h0{t, mine, NT / 2, 1 + wl};
+        step_cell<S>(c, c, h0, x, y, live && x + 1 < c.nx, o, health);
+    } else {
+        const HalfTile<SplitTile<SmemTile2>, 1> h1{t, mine, NT / 2, 1 + wl};
+        step_cell<S>(c, c, h1, x, y, live && x + 1 < c.nx, o, health);
+    }
+}
+
 template <int S>
 int launch_step_t(dbm_handle *h, const void *fin, void *fout, cudaStream_t st)
 {
@@ -1527,20 +1726,6 @@ constexpr int staged_ctas_per_sm(int TX, int TY)
     return by_smem > 4 ? 4 : by_smem < 1 ? 1 : by_smem;
 }
 
-// Output of the species-staged kernel.  Its barriers are CTA-wide and sit
-// inside the step, so every thread runs the whole step, in the same order
-// of barrier instructions: a thread whose cells lie outside the domain (the
-// ragged edge of a tile) computes on the in-range shared-memory values at
-// its position and stores nothing.
-struct StagedOut : StateOutNoImages {
-    bool live;
-    template <class G>
-    __device__ __forceinline__ void put(const Site &w, int p, G g, G e) const
-    {
-        if (live) StateOutNoImages::put(w, p, g, e);
-    }
-};
-
 template <int S, int TX, int TY>
 __global__ void __launch_bounds__(TX / 2 * TY, staged_ctas_per_sm(TX, TY))
     k_step_staged(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
@@ -1583,12 +1768,12 @@ __global__ void __launch_bounds__(TX / 2 * TY, staged_ctas_per_sm(TX, TY))
         t.issue(0);
         t.issue(1);
     }
-    // every thread steps (see StagedOut); one outside the domain stores
+    // every thread steps (see MaskedOut); one outside the domain stores
     // nothing and sends its health bits to a sink
     __shared__ unsigned health_sink;
     const int x = t.bx0 + 2 * tx, y = t.by0 + ty;
     const bool live = x < c.nx && y < c.ny;
-    const StagedOut o{{fout, c.plane, (long long)S * Q * c.plane, flag}, live};
+    const MaskedOut o{{fout, c.plane, (long long)S * Q * c.plane, flag}, live};
     step_cell<S>(c, c, t, x, y, live && x + 1 < c.nx, o, live ? flag : &health_sink);
     t.drain();
 }
@@ -1612,6 +1797,28 @@ int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorM
     return set_cuda_error(h, launch_chained(k_step_staged<S, TX, TY>, grid, block, smem, st, c, *tmap, *tmap_in,
                                             (const float *)fin, (float *)fout, (unsigned *)h->scratch),
                           "staged step kernel launch");
+}
+
+template <int S, int TX, int TY>
+int launch_step_half_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin, void *fout,
+                       cudaStream_t st)
+{
+    constexpr size_t need = half_smem(S, TX, TY), most = need > ALONE_SMEM ? need : ALONE_SMEM;
+    static bool attr_set = false;  // per instantiation, set once per process
+    if (!attr_set) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k_step_half<S, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        if (e != cudaSuccess) return set_cuda_error(h, e, "two-thread step kernel shared-memory attribute");
+        attr_set = true;
+    }
+    StepConsts<float, S> c;
+    fill_step_consts<float, S>(h, c);
+    c.prefetch = (unsigned)h->sms;
+    dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
+    const size_t smem = (long long)grid.x * grid.y <= h->sms ? most : need;
+    return set_cuda_error(h, launch_chained(k_step_half<S, TX, TY>, grid, dim3(TX * TY), smem, st, c, *tmap, *tmap_in,
+                                            (const float *)fin, (float *)fout, (unsigned *)h->scratch),
+                          "two-thread step kernel launch");
 }
 
 }  // namespace dbm

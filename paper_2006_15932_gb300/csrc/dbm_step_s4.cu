@@ -7,4 +7,6 @@ template int launch_step_tma_t<4, tma_tile_x(4), tma_tile_y(4), 1, 0>(dbm_handle
                                      cudaStream_t);
 template int launch_step_staged_t<4, STAGED_TX, STAGED_TY>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
                                                                 const void *, void *, cudaStream_t);
+template int launch_step_half_t<4, SMALL_TX, SMALL_TY>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
+                                     const void *, void *, cudaStream_t);
 }  // namespace dbm

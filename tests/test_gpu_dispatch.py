@@ -13,7 +13,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,ns,bc", [
     (513, 113, 2, (W.PERIODIC, W.OUTFLOW)),  # 9 x 15 pair tiles, ragged both ways
     (512, 128, 2, (W.OUTFLOW, W.PERIODIC)),  # exactly 128 pair tiles
-    (510, 119, 2, (W.OUTFLOW, W.OUTFLOW)),   # 120: one cell per thread
+    (510, 119, 2, (W.OUTFLOW, W.OUTFLOW)),   # 120: two threads per pair
+    (67, 9, 2, (W.PERIODIC, W.PERIODIC)), (33, 5, 2, (W.OUTFLOW, W.PERIODIC)), (1, 1, 2, (W.PERIODIC, W.OUTFLOW)),
+    (31, 6, 4, (W.OUTFLOW, W.OUTFLOW)), (97, 75, 4, (W.PERIODIC, W.PERIODIC)),
     (1025, 65, 1, (W.PERIODIC, W.PERIODIC)),
     (321, 200, 3, (W.OUTFLOW, W.PERIODIC)),
     (130, 300, 4, (W.PERIODIC, W.OUTFLOW)),
