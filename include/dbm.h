@@ -127,10 +127,13 @@ enum dbm_step_kernel {
                                  DBM_KERNEL_TMA                                      */
     DBM_KERNEL_GENERIC = 1,   /* stencil read from global memory                      */
     DBM_KERNEL_TMA = 2,       /* tile + halo staged in shared memory by TMA copies:
-                                 S = 1, 3, 4: one cell per thread; S = 2: two cells
+                                 S = 1, 3: one cell per thread; S = 2: two cells
                                  per thread on grids of at least 128 tiles of 64 x 8
-                                 cells (4096 with the thermo or rounding option),
-                                 else one cell per thread; S >= 5: as
+                                 cells, two threads per pair of cells on smaller ones
+                                 (with the thermo or rounding option: from 4096
+                                 tiles, else one cell per thread); S = 4: one cell per
+                                 thread, or two threads per pair on small grids;
+                                 S >= 5: as
                                  DBM_KERNEL_TMA_STAGED                               */
     DBM_KERNEL_TMA_CELL = 3,  /* TMA-staged, all planes in one copy, one cell per
                                  thread (S <= 4)                                     */
@@ -389,8 +392,10 @@ long long dbm_steps_taken(const dbm_handle *h);
  * cells_per_thread 1 or 2 (adjacent cells of a row, packed FP32x2
  * arithmetic).  Two species below 4096 tiles of 64 x 8 cells answer with
  * their one-cell tile, 32 x 7; the step itself runs pairs on 64 x 8 tiles
- * there as well from 128 such tiles up, unless DBM_KERNEL_TMA_CELL asks for
- * one cell (same bits).
+ * there as well from 128 such tiles up, and two threads per pair on smaller
+ * grids, unless DBM_KERNEL_TMA_CELL asks for one cell; four species answer
+ * 32 x 6 and run 32 x 7 (or two threads per pair on a small grid).  The bits
+ * are the same.
  * All three 0 when the step runs a kernel without a tile
  * (generic global-memory stencil, FP64, BF16DEV).  Null outputs are
  * skipped.  DBM_ERR_UNBOUND before dbm_bind. */

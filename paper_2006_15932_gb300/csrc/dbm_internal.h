@@ -131,9 +131,9 @@ namespace dbm {
 // thread updates (CW: 1, or 2 adjacent cells of a row with packed FP32x2
 // arithmetic).  One cell per thread: 64 x 4 cells for one species (4 CTAs of
 // 256 threads per SM), 32 x 8 for three (92 KB of shared memory, two CTAs),
-// 32 x 6 for four (102 KB, two CTAs of 192 threads; 29.4 G/s on 2048 x 2048
-// against 22.3 G/s for the generic kernel; 32x4, 64x4, 32x2, 32x3 and 64x2
-// were slower).  Measured fastest among 32x16, 32x12, 32x10, 32x9, 32x8,
+// 32 x 7 for four (113 KB, two CTAs of 224 threads, the tallest that fits
+// twice; us a step against 32 x 6: 2048 x 1024 242 / 254, 777 x 413 56.7 / 58.9;
+// 32x4, 64x4, 32x2, 32x3 and 64x2 were slower than that).  Measured fastest among 32x16, 32x12, 32x10, 32x9, 32x8,
 // 32x7, 32x6, 32x5, 32x4, 40x8, 48x6, 64x8, 64x6, 64x5, 64x4, 128x4 and
 // others on 4096 x 4096 (two species) and 4096 x 2048 (one) grids: more
 // resident CTAs per SM hide each CTA's wait for its tile.  For three species
@@ -150,7 +150,7 @@ namespace dbm {
 // per SM and ran slower (64 x 4 and 32 x 8: 12.4 and 15.5 G/s against 21.4
 // on the 1024 x 256 reactive gas, 25.2 and 26.6 against 31.2 on 2048 x 1024).
 constexpr int tma_tile_x(int S) { return S == 1 ? 64 : 32; }
-constexpr int tma_tile_y(int S) { return S == 1 ? 4 : S == 2 ? 7 : S == 3 ? 8 : 6; }
+constexpr int tma_tile_y(int S) { return S == 1 ? 4 : S == 3 ? 8 : 7; }
 constexpr int PAIR_TX = 64, PAIR_TY = 8;
 // The species-staged step (two cells per thread, the tile passing through
 // shared memory one species at a time in two buffers; k_step_staged): its

@@ -84,7 +84,8 @@ static bool staged_supported(const dbm_params &p)
 //
 // dbm_step_tile's answer is fixed by its own rule, older than pairs on small
 // grids: it names the pair tile for two species from PAIR_MIN_TILES tiles up
-// (or when pairs are asked for) and the one-cell tile below.
+// (or when pairs are asked for) and the one-cell tile below, and for four
+// species the one-cell tile's former 32 x 6.
 static void choose_tile(dbm_handle *h)
 {
     const dbm_params &p = h->p;
@@ -113,7 +114,7 @@ static void choose_tile(dbm_handle *h)
     h->tma_ty = pair ? PAIR_TY : h->tma_half ? SMALL_TY : tma_tile_y(p.nspecies);
     h->tma_cw = pair ? 2 : 1;
     h->told_tx = told_pair ? PAIR_TX : tma_tile_x(p.nspecies);
-    h->told_ty = told_pair ? PAIR_TY : tma_tile_y(p.nspecies);
+    h->told_ty = told_pair ? PAIR_TY : p.nspecies == 4 ? 6 : tma_tile_y(p.nspecies);
     h->told_cw = told_pair ? 2 : 1;
 }
 

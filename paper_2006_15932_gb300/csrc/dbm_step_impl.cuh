@@ -1417,6 +1417,14 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     __syncthreads();
     const int tid = ty * (TX / CW) + tx;
     const HaloSides hs = halo_sides<TX, TY>(bx0, by0, c.nx, c.ny);
+    // one cell per thread: a boundary tile's halo is loaded beside its copies
+    // (us a step: 1024 x 256, three species 28.2 -> 27.0; 777 x 413, four 61.6 ->
+    // 58.9); a pair's registers are full and its halo is filled afterwards
+    // (256^2, two species 8.2, loaded beside 8.5)
+    constexpr bool EARLY = CW == 1;
+    HaloRegs<NP, TX, TY, NT> hr;
+    if (EARLY && hs.any())
+        halo_load(hr, hs, fin, bx0, by0, c.nx, c.ny, c.pitch, c.plane, c.bc_x, c.bc_y, tid, flag);
     const bool ok = mbar_wait(b, 0, c.wait_polls);
     if (__syncthreads_or(!ok)) {
         // the copy did not land: report, give the copies one more bounded wait
@@ -1429,7 +1437,11 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     if (hs.any()) {
         for (int s = 1; s < S; ++s)
             if (!mbar_wait(b + 8u * s, 0, TMA_WAIT_LIMIT)) raise_flag(flag, DBM_HEALTH_TIMEOUT);
-        halo_fill<NP, TX, TY, NT>(hs, tile, fin, bx0, by0, c.nx, c.ny, c.pitch, c.plane, c.bc_x, c.bc_y, tid, flag);
+        if constexpr (EARLY)
+            halo_store(hr, hs, tile, bx0, by0, c.nx, c.ny, tid, flag);
+        else
+            halo_fill<NP, TX, TY, NT>(hs, tile, fin, bx0, by0, c.nx, c.ny, c.pitch, c.plane, c.bc_x, c.bc_y, tid,
+                                      flag);
     }
     const int x = bx0 + CW * tx, y = by0 + ty;
     if (x >= c.nx || y >= c.ny) {

@@ -51,9 +51,10 @@ from . import workloads as W
 # of the compiled shapes with one CTA per tile on mixes of sides 64 to 512
 # (us a step, best shape / 64 x 4 one cell, the former shape of all: two
 # species, 64 instances 358 / 386; three species, 30 instances of 100 to 400
-# 203 / 221; four 290 / 410; one species 64 x 4 stays)
+# 202 / 221; four 291 / 411; one species 64 x 4 stays)
 DEFAULT_CONFIG = {"tile": (64, 8), "cells": 2, "persistent": 0, "promote": 1,
-                  "by_species": {1: {"tile": (64, 4), "cells": 1}, 3: {"tile": (32, 8), "cells": 1}}}
+                  "by_species": {1: {"tile": (64, 4), "cells": 1}, 3: {"tile": (32, 8), "cells": 1},
+                                 4: {"tile": (32, 7), "cells": 1}}}
 
 
 class Admission:
