@@ -131,12 +131,19 @@ def kernel_source_sha():
 
 def step_kernel_name(pb, precision, solver):
     """The step kernel dbm_step dispatches for this problem (DBM_KERNEL_AUTO);
-    the TMA tile as the library reports it."""
+    the TMA tile as the library reports it, where the step runs that one."""
     if precision == "fp64":
         return f"k_step_f64<{pb.ns}>"
     if precision == "bf16dev":
         return f"k_step_bf16<{pb.ns},32,16,2>"
     tx, ty, cw = solver.step_tile()
+    if tx and pb.ns >= 5:  # one cell per thread, one species at a time
+        return f"k_step_staged<{pb.ns},32,8,1>"
+    if tx and pb.ns == 2:  # pairs, or two threads per pair below 128 pair tiles
+        pairs = -(-pb.nx // 64) * -(-pb.ny // 8) >= 128
+        return "k_step_tma<2,64,8,2>" if pairs else "k_step_half<2,32,4>"
+    if tx and pb.ns == 4:
+        ty = 7
     if tx and cw == 2 and pb.ns >= 3:  # two cells per thread for three or more species: species-staged
         return f"k_step_staged<{pb.ns},{tx},{ty}>"
     if tx:

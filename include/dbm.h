@@ -142,8 +142,8 @@ enum dbm_step_kernel {
     DBM_KERNEL_TMA_STAGED = 5 /* TMA-staged one species at a time through two shared-
                                  memory buffers (each species copied for its moment
                                  sums and again for its update), two adjacent cells
-                                 per thread on 64 x 8 tiles; 2 <= S <= 8, without the
-                                 thermo and rounding options                         */
+                                 per thread on 64 x 8 tiles (S >= 5: one on 32 x 8);
+                                 2 <= S <= 8, without the thermo and rounding options */
 };
 
 /* Constants of one species sigma. */
@@ -394,8 +394,9 @@ long long dbm_steps_taken(const dbm_handle *h);
  * their one-cell tile, 32 x 7; the step itself runs pairs on 64 x 8 tiles
  * there as well from 128 such tiles up, and two threads per pair on smaller
  * grids, unless DBM_KERNEL_TMA_CELL asks for one cell; four species answer
- * 32 x 6 and run 32 x 7 (or two threads per pair on a small grid).  The bits
- * are the same.
+ * 32 x 6 and run 32 x 7 (or two threads per pair on a small grid); the
+ * species-staged step answers 64 x 8 pairs and runs 32 x 8 cells for five or
+ * more species.  The bits are the same.
  * All three 0 when the step runs a kernel without a tile
  * (generic global-memory stencil, FP64, BF16DEV).  Null outputs are
  * skipped.  DBM_ERR_UNBOUND before dbm_bind. */

@@ -152,18 +152,18 @@ namespace dbm {
 constexpr int tma_tile_x(int S) { return S == 1 ? 64 : 32; }
 constexpr int tma_tile_y(int S) { return S == 1 ? 4 : S == 3 ? 8 : 7; }
 constexpr int PAIR_TX = 64, PAIR_TY = 8;
-// The species-staged step (two cells per thread, the tile passing through
-// shared memory one species at a time in two buffers; k_step_staged): its
-// tile, 64 x 8 cells in two buffers of 55 KB, two CTAs of 256 threads per
-// SM.  A build may set another with -DDBM_STAGED_TX=.. -DDBM_STAGED_TY=..
-// (TX a multiple of 8).
-#ifndef DBM_STAGED_TX
-#define DBM_STAGED_TX 64
-#endif
-#ifndef DBM_STAGED_TY
-#define DBM_STAGED_TY 8
-#endif
-constexpr int STAGED_TX = DBM_STAGED_TX, STAGED_TY = DBM_STAGED_TY;
+// The species-staged step (the tile passing through shared memory one species
+// at a time in two buffers; k_step_staged).  Five or more species: one cell
+// per thread on 32 x 8 cells, two buffers of 31 KB, three CTAs of 256 threads
+// per SM; its waits for copies want warps more than it wants fewer
+// instructions (us a step, two cells per thread on 64 x 8 with two CTAs / this:
+// 1024^2, five 197 / 193; 777 x 413, six 121 / 106; 1024 x 512, eight 200 / 183;
+// 128^2, five 31 / 20; 32 x 7, 32 x 6, 32 x 10 and 64 x 4 were slower).  Two to
+// four, when asked for: two cells per thread on 64 x 8 (2048 x 1024, three
+// 202 / 212, four 274 / 303).
+constexpr int staged_cw(int S) { return S >= 5 ? 1 : 2; }
+constexpr int staged_tile_x(int S) { return S >= 5 ? 32 : 64; }
+constexpr int staged_tile_y(int) { return 8; }
 constexpr long long PAIR_MIN_TILES = 4096, PAIR_MIN_RUN = 128;
 // Small grids of two and four species: two threads per pair of cells on
 // SMALL_TX x SMALL_TY tiles (k_step_half; 32 x 8 on 128^2, two species, 6.6 us

@@ -16,22 +16,29 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
 template <int S, int TX, int TY>
 int launch_step_half_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin, void *fout,
                        cudaStream_t st);
-template <int S, int TX, int TY>
+template <int S, int TX, int TY, int CW>
 int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin,
                          void *fout, cudaStream_t st);
+
+template <int S>
+static int launch_staged_s(dbm_handle *h, const CUtensorMap *tm, const CUtensorMap *ti, const void *fin, void *fout,
+                           cudaStream_t st)
+{
+    return launch_step_staged_t<S, staged_tile_x(S), staged_tile_y(S), staged_cw(S)>(h, tm, ti, fin, fout, st);
+}
 
 // The species-staged step of the handle's tile (no arithmetic options).
 static int launch_staged(dbm_handle *h, int cur, const void *fin, void *fout, cudaStream_t st)
 {
     const CUtensorMap *tm = &h->tmap[cur], *ti = &h->tmap_in[cur];
     switch (h->p.nspecies) {
-    case 2: return launch_step_staged_t<2, STAGED_TX, STAGED_TY>(h, tm, ti, fin, fout, st);
-    case 3: return launch_step_staged_t<3, STAGED_TX, STAGED_TY>(h, tm, ti, fin, fout, st);
-    case 4: return launch_step_staged_t<4, STAGED_TX, STAGED_TY>(h, tm, ti, fin, fout, st);
-    case 5: return launch_step_staged_t<5, STAGED_TX, STAGED_TY>(h, tm, ti, fin, fout, st);
-    case 6: return launch_step_staged_t<6, STAGED_TX, STAGED_TY>(h, tm, ti, fin, fout, st);
-    case 7: return launch_step_staged_t<7, STAGED_TX, STAGED_TY>(h, tm, ti, fin, fout, st);
-    case 8: return launch_step_staged_t<8, STAGED_TX, STAGED_TY>(h, tm, ti, fin, fout, st);
+    case 2: return launch_staged_s<2>(h, tm, ti, fin, fout, st);
+    case 3: return launch_staged_s<3>(h, tm, ti, fin, fout, st);
+    case 4: return launch_staged_s<4>(h, tm, ti, fin, fout, st);
+    case 5: return launch_staged_s<5>(h, tm, ti, fin, fout, st);
+    case 6: return launch_staged_s<6>(h, tm, ti, fin, fout, st);
+    case 7: return launch_staged_s<7>(h, tm, ti, fin, fout, st);
+    case 8: return launch_staged_s<8>(h, tm, ti, fin, fout, st);
     }
     return DBM_ERR_INVALID;
 }
@@ -84,8 +91,8 @@ static bool staged_supported(const dbm_params &p)
 //
 // dbm_step_tile's answer is fixed by its own rule, older than pairs on small
 // grids: it names the pair tile for two species from PAIR_MIN_TILES tiles up
-// (or when pairs are asked for) and the one-cell tile below, and for four
-// species the one-cell tile's former 32 x 6.
+// (or when pairs are asked for) and the one-cell tile below, for four species
+// the one-cell tile's former 32 x 6, for the species-staged step 64 x 8 pairs.
 static void choose_tile(dbm_handle *h)
 {
     const dbm_params &p = h->p;
@@ -95,9 +102,12 @@ static void choose_tile(dbm_handle *h)
     const bool staged_asked = want == DBM_KERNEL_TMA_STAGED || (p.nspecies >= 3 && want == DBM_KERNEL_TMA_PAIR);
     if (staged_supported(p) && (staged_by_default || staged_asked)) {
         h->tma_staged = 1;
-        h->tma_tx = h->told_tx = STAGED_TX;
-        h->tma_ty = h->told_ty = STAGED_TY;
-        h->tma_cw = h->told_cw = 2;
+        h->tma_tx = staged_tile_x(p.nspecies);
+        h->tma_ty = staged_tile_y(p.nspecies);
+        h->tma_cw = staged_cw(p.nspecies);
+        h->told_tx = PAIR_TX;
+        h->told_ty = PAIR_TY;
+        h->told_cw = 2;
         return;
     }
     bool told_pair = false, pair = false;

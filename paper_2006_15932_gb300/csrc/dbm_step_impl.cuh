@@ -195,7 +195,7 @@ struct SmemTile2 {
 };
 
 // A tile that passes through shared memory one species at a time
-// (StagedTile2, the species-staged step) declares kStaged; step_cell then
+// (StagedTile, the species-staged step) declares kStaged; step_cell then
 // brackets the reads of each species with acquire / release and reads
 // through view(k, s), the buffer of use k.  Other tiles hold every species
 // at once and are read as they are.
@@ -1646,9 +1646,10 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
 // The species-staged step.  The tile and its radius-2 halo pass through
 // shared memory one species at a time, in two buffers that each hold the Q
 // planes of one species (BX x BY cells), so the shared memory of a CTA does
-// not grow with the species count: three and more species run two cells per
-// thread at two CTAs per SM (the all-species tile of three species in pairs
-// would hold one).  Each species is copied twice per tile: for its moment
+// not grow with the species count: five and more species, whose all-species
+// tile fits no useful shape, run one cell per thread at three CTAs per SM, fewer
+// (when asked for) two cells per thread at two (staged_cw has the figures).
+// Each species is copied twice per tile: for its moment
 // sums only its TX x TY own cells (a second descriptor, an interior box; no
 // halo), for its update the tile and its halo.  Use k = 0 .. 2S-1 takes
 // species k mod S from buffer k & 1,
@@ -1656,21 +1657,22 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
 // computed the copy of the next one is in flight, and once every thread is
 // done with a buffer (the barrier in release) the leader refills it for use
 // k + 2.  A tile at the domain boundary fills each copy's halo from the
-// interior of the input (halo_fill on that species' planes).
+// interior of the input (that species' planes).
 //
 // Waits are bounded.  The first one takes c.wait_polls polls (a test can
 // make it run out); a wait that runs out raises DBM_HEALTH_TIMEOUT, and the
 // first one then waits once more, with the full limit.  A thread whose wait
 // ran out for good stops waiting, the leader stops issuing copies, and at
 // the end the leader waits (bounded) for the copies it left in flight.
-template <int S, int TX, int TY>
-struct StagedTile2 {
+template <int S, int TX, int TY, int CW>
+struct StagedTile {
     static constexpr bool kStaged = true;
-    static constexpr int BX = TX + 8, BY = TY + 4, PS = BX * BY, NT = TX / 2 * TY;
+    static constexpr int BX = TX + 8, BY = TY + 4, PS = BX * BY, NT = TX / CW * TY;
     static constexpr int PI = TX * TY;  // plane of an interior copy
     static constexpr unsigned BYTES = (unsigned)(PS * Q * sizeof(float));
     static constexpr unsigned BYTES_IN = (unsigned)(PI * Q * sizeof(float));
-    using V = float2;
+    using V = typename std::conditional<CW == 2, float2, float>::type;
+    using View = typename std::conditional<CW == 2, SmemTile2, SmemTile>::type;
     float *buf;         // buffer 0 (buffer 1 follows at Q * PS)
     const float *cell;  // buffer 0, plane 0, this thread's row and first column
     const float *own;   // the same cells in the interior layout [plane][TY][TX]
@@ -1684,10 +1686,10 @@ struct StagedTile2 {
 
     // view of use k: plane s * Q + i of species s read from buffer k & 1
     // (interior layout for the moment sums, k < S)
-    __device__ __forceinline__ SmemTile2 view(int k, int s) const
+    __device__ __forceinline__ View view(int k, int s) const
     {
-        if (k < S) return SmemTile2{own + (k & 1) * Q * PS - s * Q * PI, PI, TX, buf, 2 * Q * PS, flag};
-        return SmemTile2{cell + ((k & 1) - s) * Q * PS, PS, BX, buf, 2 * Q * PS, flag};
+        if (k < S) return View{own + (k & 1) * Q * PS - s * Q * PI, PI, TX, buf, 2 * Q * PS, flag};
+        return View{cell + ((k & 1) - s) * Q * PS, PS, BX, buf, 2 * Q * PS, flag};
     }
     __device__ __forceinline__ static bool leader() { return threadIdx.x == 0 && threadIdx.y == 0; }
     // leader: the copy of use k into its buffer
@@ -1709,10 +1711,12 @@ struct StagedTile2 {
                 if (!ok) failed_at = k;
             }
         }
+        // (loading a boundary tile's halo beside the copy, as the one-cell kernel
+        // does, costs this one registers: 1024^2, five species 194 -> 214 us)
         const HaloSides hs = halo_sides<TX, TY>(bx0, by0, nx, ny);
         if (k >= S && hs.any())
             halo_fill<Q, TX, TY, NT>(hs, buf + (k & 1) * Q * PS, fin + (long long)(k % S) * Q * plane, bx0, by0,
-                                     nx, ny, pitch, plane, bc_x, bc_y, threadIdx.y * (TX / 2) + threadIdx.x, flag);
+                                     nx, ny, pitch, plane, bc_x, bc_y, threadIdx.y * (TX / CW) + threadIdx.x, flag);
     }
     __device__ __forceinline__ void release(int k) const
     {
@@ -1738,14 +1742,14 @@ constexpr int staged_ctas_per_sm(int TX, int TY)
     return by_smem > 4 ? 4 : by_smem < 1 ? 1 : by_smem;
 }
 
-template <int S, int TX, int TY>
-__global__ void __launch_bounds__(TX / 2 * TY, staged_ctas_per_sm(TX, TY))
+template <int S, int TX, int TY, int CW>
+__global__ void __launch_bounds__(TX / CW * TY, staged_ctas_per_sm(TX, TY))
     k_step_staged(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
                   const __grid_constant__ CUtensorMap tmap_in, const float *__restrict__ fin,
                   float *__restrict__ fout, unsigned *__restrict__ flag)
 {
     static_assert(S >= 2 && TX % 8 == 0, "two or more species; 16-byte aligned tile columns");
-    using T = StagedTile2<S, TX, TY>;
+    using T = StagedTile<S, TX, TY, CW>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long bars[2];
     float *buf = reinterpret_cast<float *>(smem_raw);
@@ -1759,8 +1763,8 @@ __global__ void __launch_bounds__(TX / 2 * TY, staged_ctas_per_sm(TX, TY))
     __syncthreads();
     chain_begin();
     const T t{buf,
-              buf + (ty + 2) * T::BX + (2 * tx + 4),
-              buf + ty * TX + 2 * tx,
+              buf + (ty + 2) * T::BX + (CW * tx + 4),
+              buf + ty * TX + CW * tx,
               reinterpret_cast<unsigned long long>(&tmap),
               reinterpret_cast<unsigned long long>(&tmap_in),
               b0,
@@ -1783,30 +1787,30 @@ __global__ void __launch_bounds__(TX / 2 * TY, staged_ctas_per_sm(TX, TY))
     // every thread steps (see MaskedOut); one outside the domain stores
     // nothing and sends its health bits to a sink
     __shared__ unsigned health_sink;
-    const int x = t.bx0 + 2 * tx, y = t.by0 + ty;
+    const int x = t.bx0 + CW * tx, y = t.by0 + ty;
     const bool live = x < c.nx && y < c.ny;
     const MaskedOut o{{fout, c.plane, (long long)S * Q * c.plane, flag}, live};
-    step_cell<S>(c, c, t, x, y, live && x + 1 < c.nx, o, live ? flag : &health_sink);
+    step_cell<S>(c, c, t, x, y, CW == 2 ? live && x + 1 < c.nx : true, o, live ? flag : &health_sink);
     t.drain();
 }
 
-template <int S, int TX, int TY>
+template <int S, int TX, int TY, int CW>
 int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap *tmap_in, const void *fin,
                          void *fout, cudaStream_t st)
 {
     constexpr size_t smem = (size_t)2 * (TX + 8) * (TY + 4) * Q * sizeof(float);
     static bool attr_set = false;  // per instantiation, set once per process
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_step_staged<S, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_step_staged<S, TX, TY, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return set_cuda_error(h, e, "staged step kernel shared-memory attribute");
         attr_set = true;
     }
     StepConsts<float, S> c;
     fill_step_consts<float, S>(h, c);
-    dim3 block(TX / 2, TY);
+    dim3 block(TX / CW, TY);
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
-    return set_cuda_error(h, launch_chained(k_step_staged<S, TX, TY>, grid, block, smem, st, c, *tmap, *tmap_in,
+    return set_cuda_error(h, launch_chained(k_step_staged<S, TX, TY, CW>, grid, block, smem, st, c, *tmap, *tmap_in,
                                             (const float *)fin, (float *)fout, (unsigned *)h->scratch),
                           "staged step kernel launch");
 }
