@@ -37,11 +37,11 @@ BYTES_PER_UPDATE = {"fp64": 256, "fp32": 128}
 FALLBACK_HBM_GBS = 6800.0
 # The FP64 step (oracle operation order, no fused multiply-add) is bound by
 # the FP64 pipe, not by HBM.  Its FP64 operations per species-cell update,
-# from the ncu counts of one 1024 x 1024 two-species launch (DADD 85.8 +
-# DMUL 80.1 + 2 x DFMA 46.2 flop per cycle over 12.24 ms at 2.06 GHz for
-# 2.10 M updates), and the nominal FP64 peak of a GB300 (no measured FP64
+# from the ncu counts of one 512 x 384 two-species launch (DADD 127.6 + DMUL
+# 75.8 + 2 x DFMA 43.3 flop per cycle over 748 us at 2.05 GHz for 0.393 M
+# updates), and the nominal FP64 peak of a GB300 (no measured FP64
 # figure exists for this pool).
-FP64_FLOPS_PER_UPDATE = 3107.0
+FP64_FLOPS_PER_UPDATE = 1130.0
 FP64_PEAK_TFLOPS = 1.25
 
 
@@ -689,7 +689,7 @@ def main():
                     "frac": tflops / FP64_PEAK_TFLOPS, "traffic": None,
                     "peak_source": "nominal GB300 FP64 (no measured FP64 peak); the kernel keeps the oracle's "
                                    "operation order, so separate adds and multiplies fill the FP64 pipe "
-                                   "(84.5 % busy per ncu) at half the flops of fused multiply-adds",
+                                   "(82 % busy per ncu, the rate back-to-back additions reach)",
                     "kernel": step_kernel_name(pb, args.precision, solver), "flops_per_update": FP64_FLOPS_PER_UPDATE,
                     "hbm_gbs": achieved, "median_launch_ms": statistics.median(per_launch)}
     else:

@@ -354,15 +354,23 @@ inline NoneqConsts<S> noneq_consts(const OutConsts<S> &c)
 }
 
 // m times the moments of rows 5..16 of M (xx, xy, yy, q x, q y, xxx, xxy, xyy,
-// yyy, q xx, q xy, q yy) of one species' values.
-template <int S>
-__device__ __forceinline__ void high_moments(const NoneqConsts<S> &k, int s, const double f[Q], double t[12])
+// yyy, q xx, q xy, q yy) of one species' values; with LOW also n, j_x, j_y, E.
+template <bool LOW, int S>
+__device__ __forceinline__ void high_moments(const NoneqConsts<S> &k, int s, const double f[Q], double t[12],
+                                             double low[4])
 {
 #pragma unroll
     for (int j = 0; j < 12; ++j) t[j] = 0.0;
+    if (LOW) low[0] = low[1] = low[2] = low[3] = 0.0;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const RingSums g = ring_sums(r, f + 4 * r);
+        if (LOW) {
+            low[0] += g.all;
+            low[1] += k.c.vr[s][r] * g.rx;
+            low[2] += k.c.vr[s][r] * g.ry;
+            low[3] += k.c.qr[s][r] * g.all;
+        }
         if (r & 1) {  // xx and yy are the ring's sum, xxx = xyy, xxy = yyy
             const double e2 = k.v2[s][r] * g.all, e4 = k.qv2[s][r] * g.all;
             const double cx = k.v3[s][r] * g.rx, cy = k.v3[s][r] * g.ry;
@@ -395,8 +403,8 @@ __device__ __forceinline__ void high_moments(const NoneqConsts<S> &k, int s, con
 // over it is needed, and M f comes from ring sums: under 200 FP64 operations
 // per species and cell where summing f - f^eq over the velocities took 1400
 // (the FP64 pipe bounds this kernel: 2048 x 1024, two species, 7.9 -> 1.63
-// ms).  Up to two species keep their values in registers until the mixture u
-// and T are known; more load them again.
+// ms).  Up to two species keep their sums in registers until the mixture u and
+// T are known; more load their values again.
 template <int S, class Src>
 __global__ void __launch_bounds__(128)
     k_noneq(const __grid_constant__ NoneqConsts<S> k, const __grid_constant__ Src src,
@@ -409,19 +417,36 @@ __global__ void __launch_bounds__(128)
     const long long N = (long long)c.nx * c.ny;
     const long long d = (long long)y * c.nx + x;
     const long long cell = (long long)(y + GY) * c.pitch + (x + GX);
-    double n[S], jx[S], jy[S], en[S];
-    cell_moments<S>(c, src, cell, n, jx, jy, en);
+    constexpr bool KEEP = S <= 2;
+    double n[S], jx[S], jy[S], en[S], kept[KEEP ? S : 1][12], low[4];
+    if constexpr (KEEP) {
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            double fc[Q];
+            src.load16(s, cell, fc);
+            high_moments<true>(k, s, fc, kept[s], low);
+            n[s] = low[0], jx[s] = low[1], jy[s] = low[2], en[s] = low[3];
+        }
+    } else {
+        cell_moments<S>(c, src, cell, n, jx, jy, en);
+    }
     double ux, uy, T;
     cell_mixture<S>(c, n, jx, jy, en, ux, uy, T);
 #pragma unroll(S <= 2 ? S : 1)
     for (int s = 0; s < S; ++s) {
-        double fc[Q], fh[Q], t[12];
+        double fh[Q], t[12];
         double ns = n[0];  // selected, not indexed
 #pragma unroll
         for (int j = 1; j < S; ++j)
             if (s == j) ns = n[j];
-        src.load16(s, cell, fc);
-        high_moments<S>(k, s, fc, t);
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int j = 0; j < 12; ++j) t[j] = kept[s][j];
+        } else {
+            double fc[Q];
+            src.load16(s, cell, fc);
+            high_moments<false>(k, s, fc, t, low);
+        }
         // f-hat is linear in n: m f-hat is that of m n
         fhat16<double>(c.m[s] * ns, ux, uy, T * k.inv_m[s], c.dpi[s], fh);
         double *o = out + 20LL * s * N + d;

@@ -196,13 +196,9 @@ template <int S>
 static int step_bf16_t(dbm_handle *h, int cur, cudaStream_t st)
 {
     constexpr size_t smem = (size_t)(BF_TX + 4) * (BF_TY + 4) * S * Q * sizeof(float);
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_step_bf16<S, BF_TX, BF_TY, BF_CW>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return set_cuda_error(h, e, "BF16 step kernel shared-memory attribute");
-        attr_set = true;
-    }
+    static std::atomic<unsigned long long> allowed{0};
+    const cudaError_t e = allow_smem(k_step_bf16<S, BF_TX, BF_TY, BF_CW>, smem, allowed);
+    if (e != cudaSuccess) return set_cuda_error(h, e, "BF16 step kernel shared-memory attribute");
     StepConsts<float, S> c;
     fill_step_consts<float, S>(h, c);
     dim3 block(BF_TX / BF_CW, BF_TY);

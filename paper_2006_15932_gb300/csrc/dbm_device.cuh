@@ -1,8 +1,10 @@
 // dbm_device.cuh -- device building blocks of the D2V16 DBM step:
-// the equilibrium moments f-hat, the minmod limiter of the NND scheme and
+// chained launches, the equilibrium moments f-hat, conversions by bits and
 // the ghost-image bookkeeping of the boundary conditions.  The NND flux
 // differences are in dbm_step_impl.cuh.
 #pragma once
+
+#include <atomic>
 
 #include "dbm_internal.h"
 
@@ -20,6 +22,21 @@ namespace dbm {
 // let in at once).
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_end() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+// Raise a kernel's dynamic shared-memory limit, once per device (`done`: one
+// bit per device, a static of the launcher).
+template <class K>
+cudaError_t allow_smem(K kernel, size_t bytes, std::atomic<unsigned long long> &done)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (bit != 0 && (done.load(std::memory_order_relaxed) & bit) != 0) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 
 // Dynamic shared memory that keeps a grid of at most one CTA per SM from
 // doubling up: more than half of an SM's.
@@ -88,22 +105,6 @@ __device__ __forceinline__ double widen_bits(float x)
     return __hiloint2double((int)hi, (int)(u << 29));
 }
 __device__ __forceinline__ double widen(float x) { return widens_by_bits(x) ? widen_bits(x) : (double)x; }
-
-// minmod(a, b): the argument of smaller magnitude when both have the same
-// sign, else 0 (limiter of the NND scheme).
-__device__ __forceinline__ double minmod(double a, double b)
-{
-    const double s = copysign(1.0, a);
-    return s * fmax(fmin(fabs(a), s * b), 0.0);
-}
-__device__ __forceinline__ float minmod(float a, float b)
-{
-    // t = min(|a|, |b|) carrying the sign (sgn a) xor (sgn b): positive
-    // exactly when a and b agree in sign
-    float t;
-    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
-    return copysignf(fmaxf(t, 0.0f), a);
-}
 
 // Ghost images of interior index k along an axis of n cells: the ghost
 // indices g in {-2, -1, n, n+1} whose source cell is k (periodic wrap, or

@@ -451,13 +451,9 @@ static int launch_f64_wide(dbm_handle *h, const F64Consts<S> &c, int sets, const
     constexpr int CELLS = 32;
     const size_t smem = f64_smem<S>(CELLS, sets);
     if (smem > 48 * 1024) {
-        static bool attr_set = false;  // per instantiation, set once per process
-        if (!attr_set) {
-            cudaError_t e = cudaFuncSetAttribute(k_step_f64<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)f64_smem<S>(CELLS, 4));
-            if (e != cudaSuccess) return set_cuda_error(h, e, "FP64 step kernel shared-memory attribute");
-            attr_set = true;
-        }
+        static std::atomic<unsigned long long> allowed{0};
+        const cudaError_t e = allow_smem(k_step_f64<S>, f64_smem<S>(CELLS, 4), allowed);
+        if (e != cudaSuccess) return set_cuda_error(h, e, "FP64 step kernel shared-memory attribute");
     }
     const long long cells = (long long)h->p.nx * h->p.ny;
     return set_cuda_error(h, launch_chained(k_step_f64<S>, dim3((unsigned)((cells + CELLS - 1) / CELLS)),
@@ -722,13 +718,9 @@ static int launch_f64_t(dbm_handle *h, const double *fin, double *fout, cudaStre
     const long long cells = (long long)h->p.nx * h->p.ny;
     if (cells > SMALL_GRID)
         return launch_f64_wide<S>(h, c, 1 + (c.has_reaction ? 1 : 0) + (c.has_force ? 2 : 0), fin, fout, st);
-    static bool attr_set = false;  // per instantiation, set once per process
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_step_f64_small<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)ALONE_SMEM);
-        if (e != cudaSuccess) return set_cuda_error(h, e, "FP64 small-grid step kernel shared-memory attribute");
-        attr_set = true;
-    }
+    static std::atomic<unsigned long long> allowed{0};
+    const cudaError_t e = allow_smem(k_step_f64_small<S>, ALONE_SMEM, allowed);
+    if (e != cudaSuccess) return set_cuda_error(h, e, "FP64 small-grid step kernel shared-memory attribute");
     const long long ctas = (cells + SMALL_CELLS - 1) / SMALL_CELLS;
     return set_cuda_error(h, launch_chained(k_step_f64_small<S>, dim3((unsigned)ctas),
                                             dim3(128 + 32 * small_ring_warps(S)), ctas <= h->sms ? ALONE_SMEM : 0, st, c,

@@ -1622,13 +1622,9 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
 {
     using X = typename std::conditional<MODE != 0, AccConsts<S, MODE>, NoAcc>::type;
     constexpr size_t smem = (size_t)(TX + 8) * (TY + 4) * S * Q * sizeof(float);
-    static bool attr_set = false;  // per instantiation, set once per process
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_step_tma<S, TX, TY, CW, X>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return set_cuda_error(h, e, "TMA step kernel shared-memory attribute");
-        attr_set = true;
-    }
+    static std::atomic<unsigned long long> allowed{0};
+    const cudaError_t e = allow_smem(k_step_tma<S, TX, TY, CW, X>, smem, allowed);
+    if (e != cudaSuccess) return set_cuda_error(h, e, "TMA step kernel shared-memory attribute");
     StepConsts<float, S> c;
     fill_step_consts<float, S>(h, c);
     c.prefetch = (unsigned)(h->sms * tma_ctas_per_sm(S, TX, TY) / 2);
@@ -1799,13 +1795,9 @@ int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorM
                          void *fout, cudaStream_t st)
 {
     constexpr size_t smem = (size_t)2 * (TX + 8) * (TY + 4) * Q * sizeof(float);
-    static bool attr_set = false;  // per instantiation, set once per process
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_step_staged<S, TX, TY, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return set_cuda_error(h, e, "staged step kernel shared-memory attribute");
-        attr_set = true;
-    }
+    static std::atomic<unsigned long long> allowed{0};
+    const cudaError_t e = allow_smem(k_step_staged<S, TX, TY, CW>, smem, allowed);
+    if (e != cudaSuccess) return set_cuda_error(h, e, "staged step kernel shared-memory attribute");
     StepConsts<float, S> c;
     fill_step_consts<float, S>(h, c);
     dim3 block(TX / CW, TY);
@@ -1820,13 +1812,9 @@ int launch_step_half_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap
                        cudaStream_t st)
 {
     constexpr size_t need = half_smem(S, TX, TY), most = need > ALONE_SMEM ? need : ALONE_SMEM;
-    static bool attr_set = false;  // per instantiation, set once per process
-    if (!attr_set) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_step_half<S, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
-        if (e != cudaSuccess) return set_cuda_error(h, e, "two-thread step kernel shared-memory attribute");
-        attr_set = true;
-    }
+    static std::atomic<unsigned long long> allowed{0};
+    const cudaError_t e = allow_smem(k_step_half<S, TX, TY>, most, allowed);
+    if (e != cudaSuccess) return set_cuda_error(h, e, "two-thread step kernel shared-memory attribute");
     StepConsts<float, S> c;
     fill_step_consts<float, S>(h, c);
     c.prefetch = (unsigned)h->sms;
