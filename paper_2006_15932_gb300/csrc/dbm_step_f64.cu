@@ -33,7 +33,7 @@
 //   - a division by a constant b is a product with 1/b and two multiply-adds
 //     (Markstein 1990: with y = RN(1/b), q = RN(a y), r = RN(a - q b) exact,
 //     RN(q + r y) is the rounded quotient).
-// About 900 FP64 instructions per species and cell; the plain form of the same
+// About 1000 FP64 instructions per species and cell; the plain form of the same
 // arithmetic had 2500 (two species, 512 x 384: 2342 us a step, now 745,
 // with the pipe at the rate that back-to-back additions reach, one warp
 // instruction in 19 cycles).
@@ -443,7 +443,6 @@ __global__ void __launch_bounds__(128 * f64_side(S))
     }
 }
 
-// Grids of up to this many cells take the 8-cell split.
 template <int S>
 static int launch_f64_wide(dbm_handle *h, const F64Consts<S> &c, int sets, const double *fin, double *fout,
                            cudaStream_t st)

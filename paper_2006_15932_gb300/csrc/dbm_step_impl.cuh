@@ -16,8 +16,9 @@
 //   6. the forward-Euler update, stored to the other buffer, then the ghost
 //      images the boundary conditions ask for (edge cells only).
 // The inputs come from a Tile policy: straight from global memory (k_step)
-// or from a shared-memory tile that one TMA bulk copy filled (k_step_tma,
-// one cell or a pair of cells per thread);
+// or from a shared-memory tile that TMA bulk copies filled (k_step_tma, one
+// cell or a pair of cells per thread; k_step_half, two threads per pair;
+// k_step_staged, one species at a time);
 // the outputs go through an Out policy (FP32 state, or the BF16-deviation
 // state of dbm_bf16.cuh).
 //
@@ -1121,11 +1122,12 @@ __global__ void __launch_bounds__(256)
 
 // ---------------------------------------------------------------------------
 // TMA-staged kernel: one CTA steps a TX x TY tile of cells, CW (1 or 2)
-// adjacent cells of a row per thread.  One thread issues a single
-// cp.async.bulk.tensor copy of the tile plus its radius-2 halo (all 16 S
+// adjacent cells of a row per thread.  One thread issues a
+// cp.async.bulk.tensor copy per species of the tile plus its radius-2 halo (16
 // planes, columns x0-4 .. x0+TX+3 so that the copy starts on a 16-byte
-// boundary) into shared memory, completing on an mbarrier; every thread then
-// reads its stencil from shared memory.
+// boundary) into shared memory, each completing on an mbarrier of its own, so
+// that the moment sums of a species start when it has landed; every thread
+// then reads its stencil from shared memory.
 // ---------------------------------------------------------------------------
 
 __device__ __forceinline__ unsigned smem_u32(const void *p)
