@@ -5,6 +5,7 @@
 #pragma once
 
 #include <atomic>
+#include <type_traits>
 
 #include "dbm_internal.h"
 
@@ -13,13 +14,35 @@ namespace dbm {
 // Chained launches: a step kernel launched with programmatic serialization
 // may start while the kernel before it on the stream still drains.  It sets
 // up its barriers and touches no memory that another kernel reads or writes
-// before chain_begin has returned: by then the kernel before it has completed
-// and its writes are visible.  Its own successor may start once every CTA has
-// passed chain_end, which sits late in the step: CTAs that start early take
-// the free SMs and the rest of their grid doubles up on others, which costs
-// a grid of fewer CTAs than the chip holds more than the launch it hides
-// (FP64, 64 x 64, two species: 29 us a step unchained, 54 with the successor
-// let in at once).
+// before its wait (ChainedIn::wait, chain_begin) has returned: by then the
+// kernel before it has completed and its writes are visible.  Its own successor
+// may start once every CTA has passed chain_end, which sits late in the step:
+// CTAs that start early take the free SMs and the rest of their grid doubles up
+// on others, which costs a grid of fewer CTAs than the chip holds more than the
+// launch it hides (FP64, 64 x 64, two species: 29 us a step unchained, 54 with
+// the successor let in at once).
+//
+// The input of a chained kernel is still being written when the kernel starts,
+// so it is not read-only for the kernel's lifetime: a const __restrict__
+// parameter would promise that, and would let the compiler move loads above the
+// wait or send them through the non-coherent cache.  A chained kernel takes it
+// as ChainedIn, which gives the pointer out of the wait itself: every load
+// depends on the wait's result.  launch_chained takes no bare pointer to const.
+// (Plain pointers in a struct, as the compact step's BfState, promise nothing:
+// their loads stay behind the memory clobber of chain_begin.)
+template <class T>
+class ChainedIn {
+    const T *p;
+
+  public:
+    explicit ChainedIn(const void *q) : p(static_cast<const T *>(q)) {}
+    __device__ __forceinline__ const T *wait() const  // chain_begin, and the input after it
+    {
+        size_t g = __cvta_generic_to_global(p);  // stays a global address across the asm
+        asm volatile("griddepcontrol.wait;" : "+l"(g)::"memory");
+        return static_cast<const T *>(__cvta_global_to_generic(g));
+    }
+};
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_end() { asm volatile("griddepcontrol.launch_dependents;"); }
 
@@ -42,9 +65,16 @@ cudaError_t allow_smem(K kernel, size_t bytes, std::atomic<unsigned long long> &
 // doubling up: more than half of an SM's.
 constexpr size_t ALONE_SMEM = 116 * 1024;
 
+template <class P>
+constexpr bool bare_input()  // a pointer to const
+{
+    return std::is_pointer<P>::value && std::is_const<typename std::remove_pointer<P>::type>::value;
+}
+
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
 {
+    static_assert(!(bare_input<P>() || ...), "a chained kernel takes its input as ChainedIn");
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;

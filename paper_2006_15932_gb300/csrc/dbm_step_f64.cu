@@ -224,7 +224,7 @@ constexpr size_t f64_smem(int cells, int sets)
 
 template <int S>
 __global__ void __launch_bounds__(128 * f64_side(S))
-    k_step_f64(const __grid_constant__ F64Consts<S> c, const double *__restrict__ fin,
+    k_step_f64(const __grid_constant__ F64Consts<S> c, const ChainedIn<double> in,
                double *__restrict__ fout, unsigned *__restrict__ flag)
 {
     constexpr int CELLS = 32, SW = f64_side(S), NT = 128 * SW, V = 4;
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(128 * f64_side(S))
         return (long long)(y + GY) * c.pitch + (x + GX);
     };
 
-    chain_begin();
+    const double *fin = in.wait();
 
     // 1. moment sums
 #pragma unroll 1
@@ -456,7 +456,8 @@ static int launch_f64_wide(dbm_handle *h, const F64Consts<S> &c, int sets, const
     }
     const long long cells = (long long)h->p.nx * h->p.ny;
     return set_cuda_error(h, launch_chained(k_step_f64<S>, dim3((unsigned)((cells + CELLS - 1) / CELLS)),
-                                            dim3(128 * f64_side(S)), smem, st, c, fin, fout, (unsigned *)h->scratch),
+                                            dim3(128 * f64_side(S)), smem, st, c, ChainedIn<double>(fin), fout,
+                                            (unsigned *)h->scratch),
                           "FP64 step kernel launch");
 }
 
@@ -479,7 +480,7 @@ __host__ __device__ constexpr int small_ring_warps(int S) { return 4 * ((S + 1) 
 
 template <int S>
 __global__ void __launch_bounds__(128 + 32 * small_ring_warps(S))
-    k_step_f64_small(const __grid_constant__ F64Consts<S> c, const double *__restrict__ fin,
+    k_step_f64_small(const __grid_constant__ F64Consts<S> c, const ChainedIn<double> in,
                      double *__restrict__ fout, unsigned *__restrict__ flag)
 {
     constexpr int C = SMALL_CELLS, PHASE = 128;
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(128 + 32 * small_ring_warps(S))
         x = d - y * (unsigned)c.nx;
         return (long long)(y + GY) * c.pitch + (x + GX);
     };
-    chain_begin();
+    const double *fin = in.wait();
 
     if (tid < PHASE) {
         auto phase_sync = [] { asm volatile("barrier.sync 1, 128;" ::: "memory"); };
@@ -723,7 +724,7 @@ static int launch_f64_t(dbm_handle *h, const double *fin, double *fout, cudaStre
     const long long ctas = (cells + SMALL_CELLS - 1) / SMALL_CELLS;
     return set_cuda_error(h, launch_chained(k_step_f64_small<S>, dim3((unsigned)ctas),
                                             dim3(128 + 32 * small_ring_warps(S)), ctas <= h->sms ? ALONE_SMEM : 0, st, c,
-                                            fin, fout, (unsigned *)h->scratch),
+                                            ChainedIn<double>(fin), fout, (unsigned *)h->scratch),
                           "FP64 small-grid step kernel launch");
 }
 

@@ -1248,7 +1248,7 @@ __device__ __forceinline__ HaloSides halo_sides(int bx0, int by0, int nx, int ny
 
 template <int NP, int TX, int TY, int NT>
 __device__ __forceinline__ void halo_load(HaloRegs<NP, TX, TY, NT> &hr, const HaloSides &hs,
-                                          const float *__restrict__ fin, int bx0, int by0, int nx, int ny,
+                                          const float *fin, int bx0, int by0, int nx, int ny,
                                           int pitch, long long plane, int bc_x, int bc_y, int tid, unsigned *flag)
 {
     using H = HaloRegs<NP, TX, TY, NT>;
@@ -1293,7 +1293,7 @@ __device__ __forceinline__ void halo_load(HaloRegs<NP, TX, TY, NT> &hr, const Ha
 // registers would cost every tile).  All threads of the CTA call this for a
 // boundary tile.
 template <int NP, int TX, int TY, int NT>
-__device__ __forceinline__ void halo_fill(const HaloSides &hs, float *tile, const float *__restrict__ fin, int bx0,
+__device__ __forceinline__ void halo_fill(const HaloSides &hs, float *tile, const float *fin, int bx0,
                                           int by0, int nx, int ny, int pitch, long long plane, int bc_x, int bc_y,
                                           int tid, unsigned *flag)
 {
@@ -1391,7 +1391,7 @@ struct SplitTile : Base {
 template <int S, int TX, int TY, int CW, class X>
 __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     k_step_tma(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
-               const __grid_constant__ CUtensorMap tmap_in, const float *__restrict__ fin, float *__restrict__ fout,
+               const __grid_constant__ CUtensorMap tmap_in, const ChainedIn<float> in, float *__restrict__ fout,
                unsigned *__restrict__ flag, const __grid_constant__ X xa)
 {
     static_assert(CW == 1 || CW == 2, "one or two cells per thread");
@@ -1409,7 +1409,7 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b + 8u * s) : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    chain_begin();
+    const float *fin = in.wait();
     if (leader) {
         for (int s = 0; s < S; ++s)
             tma_tile_load(tile + s * Q * BX * BY, reinterpret_cast<unsigned long long>(&tmap), bx0, by0, b + 8u * s,
@@ -1542,7 +1542,7 @@ struct MaskedOut : StateOutNoImages {
 template <int S, int TX, int TY>
 __global__ void __launch_bounds__(TX *TY, 2)
     k_step_half(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
-                const __grid_constant__ CUtensorMap tmap_in, const float *__restrict__ fin, float *__restrict__ fout,
+                const __grid_constant__ CUtensorMap tmap_in, const ChainedIn<float> in, float *__restrict__ fout,
                 unsigned *__restrict__ flag)
 {
     constexpr int BX = TX + 8, BY = TY + 4, NP = S * Q, NT = TX * TY, W = NT / 64;
@@ -1561,7 +1561,7 @@ __global__ void __launch_bounds__(TX *TY, 2)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b + 8u * s) : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    chain_begin();
+    const float *fin = in.wait();
     if (tid == 0) {
         for (int s = 0; s < S; ++s)
             tma_tile_load(tile + s * Q * BX * BY, reinterpret_cast<unsigned long long>(&tmap), bx0, by0, b + 8u * s,
@@ -1635,7 +1635,7 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
     dim3 block(TX / CW, TY);
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
     return set_cuda_error(h, launch_chained(k_step_tma<S, TX, TY, CW, X>, grid, block, smem, st, c, *tmap, *tmap_in,
-                                            (const float *)fin, (float *)fout, (unsigned *)h->scratch, xa),
+                                            ChainedIn<float>(fin), (float *)fout, (unsigned *)h->scratch, xa),
                           "TMA step kernel launch");
 }
 
@@ -1743,7 +1743,7 @@ constexpr int staged_ctas_per_sm(int TX, int TY)
 template <int S, int TX, int TY, int CW>
 __global__ void __launch_bounds__(TX / CW * TY, staged_ctas_per_sm(TX, TY))
     k_step_staged(const __grid_constant__ StepConsts<float, S> c, const __grid_constant__ CUtensorMap tmap,
-                  const __grid_constant__ CUtensorMap tmap_in, const float *__restrict__ fin,
+                  const __grid_constant__ CUtensorMap tmap_in, const ChainedIn<float> in,
                   float *__restrict__ fout, unsigned *__restrict__ flag)
 {
     static_assert(S >= 2 && TX % 8 == 0, "two or more species; 16-byte aligned tile columns");
@@ -1759,7 +1759,7 @@ __global__ void __launch_bounds__(TX / CW * TY, staged_ctas_per_sm(TX, TY))
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
-    chain_begin();
+    const float *fin = in.wait();
     const T t{buf,
               buf + (ty + 2) * T::BX + (CW * tx + 4),
               buf + ty * TX + CW * tx,
@@ -1805,7 +1805,7 @@ int launch_step_staged_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorM
     dim3 block(TX / CW, TY);
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
     return set_cuda_error(h, launch_chained(k_step_staged<S, TX, TY, CW>, grid, block, smem, st, c, *tmap, *tmap_in,
-                                            (const float *)fin, (float *)fout, (unsigned *)h->scratch),
+                                            ChainedIn<float>(fin), (float *)fout, (unsigned *)h->scratch),
                           "staged step kernel launch");
 }
 
@@ -1823,7 +1823,7 @@ int launch_step_half_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
     const size_t smem = (long long)grid.x * grid.y <= h->sms ? most : need;
     return set_cuda_error(h, launch_chained(k_step_half<S, TX, TY>, grid, dim3(TX * TY), smem, st, c, *tmap, *tmap_in,
-                                            (const float *)fin, (float *)fout, (unsigned *)h->scratch),
+                                            ChainedIn<float>(fin), (float *)fout, (unsigned *)h->scratch),
                           "two-thread step kernel launch");
 }
 
