@@ -468,68 +468,79 @@ __global__ void __launch_bounds__(128)
 // adds the block partials in a fixed order.  The result is independent of
 // timing.
 //
-// The totals are linear in f, so a thread only adds up the ring sums of its
-// cells (12 sums a species) and the block forms mass, momentum and energy
-// from them once.  Float states: a ring sum and its running total over 16
-// cells are exact float-float pairs but for the last bits of the low parts
-// (about 2^-47 of the sum, below the rounding of the FP64 total they are
-// added to), on the FP32 pipes; the FP64 pipe, two lanes per SM and cycle,
-// then gets 1.5 additions per species and cell.  Multiplying every value by
-// its weights in FP64 took 190 (4096^2, two species: 8.7 -> 0.65 ms).
-struct FloatPair {
-    float h, l;
-    __device__ __forceinline__ void add(float s, float e)  // += s + e
+// The totals are linear in f, so a thread only adds up its cells (float states:
+// each velocity; FP64 states: 12 ring sums a species) and the block forms mass,
+// momentum and energy from the sums once.  Float states: a velocity's running
+// total over 32 cells is three floats, h + l + t: h and l take each value by
+// exact two-sums and only t, at most 2^-38 of the magnitudes added, is rounded,
+// 2^-57 of them in the worst case, so nothing is lost that FP64 additions of
+// the values would keep; a total past the float range is formed again in FP64.
+// This runs on the FP32 pipes, 13 additions a value; the FP64 pipe, two lanes
+// per SM and cycle, gets 2 per species and cell.  Multiplying every value by its weights in FP64
+// took 190 (4096^2, two species: 8.7 -> 0.67 ms; in two
+// floats, 48 bits, 0.65).
+struct FloatTriple {
+    float h, l, t;
+    __device__ __forceinline__ void add(float f)
     {
-        float e2;
-        h = ff_sum(h, s, e2);
-        l = __fadd_rn(l, __fadd_rn(e, e2));
+        float e, e2;
+        h = ff_sum(h, f, e);
+        l = ff_sum(l, e, e2);
+        t = __fadd_rn(t, e2);
     }
+    __device__ __forceinline__ double value() const { return widen(h) + (widen(l) + widen(t)); }
 };
 
-// Running sums of one ring: all, rx, ry.
-struct RingTotalF {
-    FloatPair a[3];
+// Running totals of a species over a thread's cells.
+struct SpeciesTotalF {
+    FloatTriple a[Q];
     __device__ __forceinline__ void clear()
     {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) a[k].h = a[k].l = 0.0f;
+        for (int i = 0; i < Q; ++i) a[i].h = a[i].l = a[i].t = 0.0f;
     }
-    template <bool DIAG>
-    __device__ __forceinline__ void add(float f0, float f1, float f2, float f3)
+    __device__ __forceinline__ void add_ring(int r, float f0, float f1, float f2, float f3)
     {
-        float e0, e1, e2, e3, e4;
-        const float a02 = ff_sum(f0, f2, e0), a13 = ff_sum(f1, f3, e1), all = ff_sum(a02, a13, e2);
-        a[0].add(all, __fadd_rn(__fadd_rn(e0, e1), e2));
-        if (DIAG) {
-            const float p = ff_sum(f0, -f2, e0), q = ff_sum(f3, -f1, e1);
-            const float rx = ff_sum(p, q, e2), ry = ff_sum(p, -q, e3);
-            a[1].add(rx, __fadd_rn(__fadd_rn(e0, e1), e2));
-            a[2].add(ry, __fadd_rn(__fsub_rn(e0, e1), e3));
-        } else {
-            const float rx = ff_sum(f0, -f2, e3), ry = ff_sum(f1, -f3, e4);
-            a[1].add(rx, e3);
-            a[2].add(ry, e4);
+        a[4 * r].add(f0), a[4 * r + 1].add(f1), a[4 * r + 2].add(f2), a[4 * r + 3].add(f3);
+    }
+    // adds the ring sums; false, and nothing added, when a value was infinite or
+    // NaN or a float total overflowed
+    __device__ __forceinline__ bool flush(double acc[4][3]) const
+    {
+        bool finite = true;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) finite = finite && isfinite(a[i].h + a[i].t);
+        if (!finite) return false;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            double f[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) f[i] = a[4 * r + i].value();
+            const RingSums g = ring_sums(r, f);
+            acc[r][0] += g.all, acc[r][1] += g.rx, acc[r][2] += g.ry;
         }
-    }
-    // an infinite or NaN total has no error part
-    __device__ __forceinline__ double value(int k) const
-    {
-        return isfinite(a[k].h) ? widen(a[k].h) + widen(a[k].l) : (double)a[k].h;
+        return true;
     }
 };
-struct RingTotalD {
-    double a[3];
-    __device__ __forceinline__ void clear() { a[0] = a[1] = a[2] = 0.0; }
-    template <bool DIAG>
-    __device__ __forceinline__ void add(double f0, double f1, double f2, double f3)
+struct SpeciesTotalD {
+    double a[4][3];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) a[r][0] = a[r][1] = a[r][2] = 0.0;
+    }
+    __device__ __forceinline__ void add_ring(int r, double f0, double f1, double f2, double f3)
     {
         const double f[4] = {f0, f1, f2, f3};
-        const RingSums g = ring_sums<DIAG>(f);
-        a[0] += g.all;
-        a[1] += g.rx;
-        a[2] += g.ry;
+        const RingSums g = ring_sums(r, f);
+        a[r][0] += g.all, a[r][1] += g.rx, a[r][2] += g.ry;
     }
-    __device__ __forceinline__ double value(int k) const { return a[k]; }
+    __device__ __forceinline__ bool flush(double acc[4][3]) const
+    {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r][0] += a[r][0], acc[r][1] += a[r][1], acc[r][2] += a[r][2];
+        return true;
+    }
 };
 
 // The values of velocities 4 r .. 4 r + 3 of four cells in a row, v[velocity][cell]
@@ -553,7 +564,7 @@ __device__ __forceinline__ void load_ring4(const double *p, long long plane, dou
 }
 
 template <class Total, typename real>
-__device__ __forceinline__ void total_cells(const PlainSrc<real> &src, int s, long long cell, int live, Total tot[4])
+__device__ __forceinline__ void total_cells(const PlainSrc<real> &src, int s, long long cell, int live, Total &tot)
 {
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -562,24 +573,19 @@ __device__ __forceinline__ void total_cells(const PlainSrc<real> &src, int s, lo
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (j >= live) break;
-            if (r & 1)
-                tot[r].template add<true>(v[0][j], v[1][j], v[2][j], v[3][j]);
-            else
-                tot[r].template add<false>(v[0][j], v[1][j], v[2][j], v[3][j]);
+            tot.add_ring(r, v[0][j], v[1][j], v[2][j], v[3][j]);
         }
     }
 }
 template <class Total, int S>
-__device__ __forceinline__ void total_cells(const BfSrc<S> &src, int s, long long cell, int live, Total tot[4])
+__device__ __forceinline__ void total_cells(const BfSrc<S> &src, int s, long long cell, int live, Total &tot)
 {
 #pragma unroll 1
     for (int j = 0; j < live; ++j) {
         float f[Q];
         src.load16f(s, cell + j, f);
-        tot[0].template add<false>(f[0], f[1], f[2], f[3]);
-        tot[1].template add<true>(f[4], f[5], f[6], f[7]);
-        tot[2].template add<false>(f[8], f[9], f[10], f[11]);
-        tot[3].template add<true>(f[12], f[13], f[14], f[15]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) tot.add_ring(r, f[4 * r], f[4 * r + 1], f[4 * r + 2], f[4 * r + 3]);
     }
 }
 
@@ -600,35 +606,44 @@ __device__ __forceinline__ double warp_total(double v)
 }
 
 template <int S, class Src>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
     k_cons_partial(const __grid_constant__ OutConsts<S> c, const __grid_constant__ Src src,
                    double *__restrict__ partial)
 {
     constexpr bool DOUBLE = std::is_same<typename Src::value, double>::value;
-    using Total = typename std::conditional<DOUBLE, RingTotalD, RingTotalF>::type;
-    constexpr int FLUSH = 4;  // vectors of four cells between additions to the FP64 sums
+    using Total = typename std::conditional<DOUBLE, SpeciesTotalD, SpeciesTotalF>::type;
+    constexpr unsigned FLUSH = 8;  // vectors of four cells between additions to the FP64 sums
     const int s = blockIdx.y;
     double acc[4][3];
-    Total tot[4];
+    Total tot;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        acc[r][0] = acc[r][1] = acc[r][2] = 0.0;
-        tot[r].clear();
-    }
+    for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = acc[r][2] = 0.0;
     const unsigned nv = (unsigned)(c.nx + 3) / 4u, count = nv * (unsigned)c.ny;
     const unsigned stride = gridDim.x * 256u;
-    int held = 0;
-    for (unsigned t = blockIdx.x * 256u + threadIdx.x; t < count; t += stride) {
-        const unsigned y = t / nv, x = 4u * (t - y * nv);
-        const long long cell = (long long)(y + GY) * c.pitch + (x + GX);
-        total_cells(src, s, cell, min(4, c.nx - (int)x), tot);
-        if (++held == FLUSH) {
-            held = 0;
+    unsigned t = blockIdx.x * 256u + threadIdx.x;
+    while (t < count) {
+        const unsigned first = t;
+        tot.clear();
+#pragma unroll 1
+        for (unsigned k = 0; k < FLUSH && t < count; ++k, t += stride) {
+            const unsigned y = t / nv, x = 4u * (t - y * nv);
+            total_cells(src, s, (long long)(y + GY) * c.pitch + (x + GX), min(4, c.nx - (int)x), tot);
+        }
+        if (tot.flush(acc)) continue;
+        // the same cells value by value in FP64
+#pragma unroll 1
+        for (unsigned q = first; q < t; q += stride) {
+            const unsigned y = q / nv, x = 4u * (q - y * nv);
+            const long long cell = (long long)(y + GY) * c.pitch + (x + GX);
+#pragma unroll 1
+            for (int j = 0; j < min(4, c.nx - (int)x); ++j) {
+                double f[Q];
+                src.load16(s, cell + j, f);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) acc[r][k] += tot[r].value(k);
-                tot[r].clear();
+                for (int r = 0; r < 4; ++r) {
+                    const RingSums g = ring_sums(r, f + 4 * r);
+                    acc[r][0] += g.all, acc[r][1] += g.rx, acc[r][2] += g.ry;
+                }
             }
         }
     }
@@ -637,7 +652,7 @@ __global__ void __launch_bounds__(256)
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const double v = warp_total(acc[r][k] + tot[r].value(k));
+            const double v = warp_total(acc[r][k]);
             if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][3 * r + k] = v;
         }
     __syncthreads();
