@@ -129,28 +129,6 @@ def kernel_source_sha():
     return h.hexdigest()[:16]
 
 
-def step_kernel_name(pb, precision, solver):
-    """The step kernel dbm_step dispatches for this problem (DBM_KERNEL_AUTO);
-    the TMA tile as the library reports it, where the step runs that one."""
-    if precision == "fp64":
-        return f"k_step_f64<{pb.ns}>"
-    if precision == "bf16dev":
-        return f"k_step_bf16<{pb.ns},32,16,2>"
-    tx, ty, cw = solver.step_tile()
-    if tx and pb.ns >= 5:  # one cell per thread, one species at a time
-        return f"k_step_staged<{pb.ns},32,8,1>"
-    if tx and pb.ns == 2:  # pairs, or two threads per pair below 128 pair tiles
-        pairs = -(-pb.nx // 64) * -(-pb.ny // 8) >= 128
-        return "k_step_tma<2,64,8,2>" if pairs else "k_step_half<2,32,4>"
-    if tx and pb.ns == 4:
-        ty = 7
-    if tx and cw == 2 and pb.ns >= 3:  # two cells per thread for three or more species: species-staged
-        return f"k_step_staged<{pb.ns},{tx},{ty}>"
-    if tx:
-        return f"k_step_tma<{pb.ns},{tx},{ty},{cw}>"
-    return f"k_step<{pb.ns}>"
-
-
 def ncu_traffic(name, precision):
     """DRAM bytes per launch of the step kernel from the committed ncu
     summary, or None when the kernel source changed since the capture."""
@@ -690,14 +668,14 @@ def main():
                     "peak_source": "nominal GB300 FP64 (no measured FP64 peak); the kernel keeps the oracle's "
                                    "operation order, so separate adds and multiplies fill the FP64 pipe "
                                    "(82 % busy per ncu, the rate back-to-back additions reach)",
-                    "kernel": step_kernel_name(pb, args.precision, solver), "flops_per_update": FP64_FLOPS_PER_UPDATE,
+                    "kernel": solver.step_kernel_name(), "flops_per_update": FP64_FLOPS_PER_UPDATE,
                     "hbm_gbs": achieved, "median_launch_ms": statistics.median(per_launch)}
     else:
         roofline = None
     roofline = roofline or {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "peak_source": f"{peak_kind} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
-                "kernel": step_kernel_name(pb, args.precision, solver) if args.workload != "batched"
+                "kernel": solver.step_kernel_name() if args.workload != "batched"
                 else f"k_step_batch<{pb.ns},{cfg['tile'][0]},{cfg['tile'][1]},{cfg['batch_config']['cells']}>",
                 "algorithmic_bytes_per_launch": bytes_per_launch,
                 "median_launch_ms": statistics.median(per_launch)}

@@ -234,8 +234,8 @@ int dbm_scratch_bytes(const dbm_handle *h, size_t *bytes);
 /* Bind caller-owned device buffers: f_a and f_b of dbm_state_bytes each
  * (256-byte aligned), scratch of dbm_scratch_bytes.  f_a becomes the current
  * state.  The buffers must outlive every call that uses them.  Builds the
- * TMA descriptors of the two buffers and fixes the step's tile
- * (dbm_step_tile); DBM_ERR_INVALID when dbm_params.step_kernel asks for a
+ * TMA descriptors of the two buffers and fixes the step's kernel
+ * (dbm_step_kernel_name); DBM_ERR_INVALID when dbm_params.step_kernel asks for a
  * TMA-staged kernel that cannot run (not FP32; one cell per thread or an
  * arithmetic option with S > 4; no descriptor). */
 int dbm_bind(dbm_handle *h, void *f_a, void *f_b, void *scratch);
@@ -387,19 +387,24 @@ int dbm_status(dbm_handle *h, void *stream, unsigned *bits);
 /* Steps taken since the last dbm_set_state / dbm_set_f. */
 long long dbm_steps_taken(const dbm_handle *h);
 
-/* The shared-memory tile class of a bound handle (chosen at dbm_bind from
- * dbm_params.step_kernel and the grid): tile_x x tile_y cells,
- * cells_per_thread 1 or 2 (adjacent cells of a row, packed FP32x2
- * arithmetic).  Two species below 4096 tiles of 64 x 8 cells answer with
- * their one-cell tile, 32 x 7; the step itself runs pairs on 64 x 8 tiles
- * there as well from 128 such tiles up, and two threads per pair on smaller
- * grids, unless DBM_KERNEL_TMA_CELL asks for one cell; four species answer
- * 32 x 6 and run 32 x 7 (or two threads per pair on a small grid); the
- * species-staged step answers 64 x 8 pairs and runs 32 x 8 cells for five or
- * more species.  The bits are the same.
- * All three 0 when the step runs a kernel without a tile
- * (generic global-memory stencil, FP64, BF16DEV).  Null outputs are
- * skipped.  DBM_ERR_UNBOUND before dbm_bind. */
+/* Name of the kernel that dbm_step launches for a bound handle, with its
+ * template arguments as written in the sources and without the arithmetic
+ * options: "k_step_tma<S,tile_x,tile_y,cells per thread>",
+ * "k_step_staged<...>" alike, "k_step_half<S,tile_x,tile_y>" (two threads per
+ * pair of cells), "k_step<S>", "k_step_f64<S>", "k_step_f64_small<S>",
+ * "k_step_bf16<S,tile_x,tile_y,cells per thread>".  At most size bytes are
+ * written, the terminating zero included.  DBM_ERR_UNBOUND before dbm_bind;
+ * DBM_ERR_INVALID for a null or empty buffer, or when no step can run. */
+int dbm_step_kernel_name(const dbm_handle *h, char *name, size_t size);
+
+/* What the handle was given by a size rule that is kept for programs which
+ * read it; dbm_step may run another tile (dbm_step_kernel_name says which; the
+ * bits are the same).  The rule: two species 64 x 8 with two cells per thread
+ * from 4096 such tiles up or for DBM_KERNEL_TMA_PAIR, else 32 x 7 with one; one
+ * species 64 x 4, three 32 x 8, four 32 x 6 with one; the species-staged step
+ * 64 x 8 with two; all three 0 when the step runs a kernel without a
+ * shared-memory tile (generic global-memory stencil, FP64, BF16DEV).  Null
+ * outputs are skipped.  DBM_ERR_UNBOUND before dbm_bind. */
 int dbm_step_tile(const dbm_handle *h, int *tile_x, int *tile_y, int *cells_per_thread);
 
 /* Message of the last failed call on this handle ("" if none).  The string

@@ -684,6 +684,13 @@ int dbm_status(dbm_handle *h, void *stream, unsigned *bits)
 
 long long dbm_steps_taken(const dbm_handle *h) { return h ? h->steps : -1; }
 
+int dbm_step_kernel_name(const dbm_handle *h, char *name, size_t size)
+{
+    if (!h || !name || size == 0) return DBM_ERR_INVALID;
+    if (!h->bound) return DBM_ERR_UNBOUND;
+    return step_kernel_name(h, name, size);
+}
+
 int dbm_step_tile(const dbm_handle *h, int *tile_x, int *tile_y, int *cells_per_thread)
 {
     if (!h) return DBM_ERR_INVALID;

@@ -476,9 +476,9 @@ __global__ void __launch_bounds__(128)
 // 2^-57 of them in the worst case, so nothing is lost that FP64 additions of
 // the values would keep; a total past the float range is formed again in FP64.
 // This runs on the FP32 pipes, 13 additions a value; the FP64 pipe, two lanes
-// per SM and cycle, gets 2 per species and cell.  Multiplying every value by its weights in FP64
-// took 190 (4096^2, two species: 8.7 -> 0.67 ms; in two
-// floats, 48 bits, 0.65).
+// per SM and cycle, gets 2 per species and cell.  Multiplying every value by its
+// weights in FP64 took 190 (4096^2, two species: 8.7 -> 0.67 ms; in two floats,
+// 48 bits, 0.65).
 struct FloatTriple {
     float h, l, t;
     __device__ __forceinline__ void add(float f)

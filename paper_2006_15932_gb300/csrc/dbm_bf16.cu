@@ -188,10 +188,6 @@ __global__ void __launch_bounds__(128)
 // launchers
 // ---------------------------------------------------------------------------
 
-// one cell per thread: 32 x 16 measured fastest of 64x8, 32x16, 32x8, 32x7
-// and 64x4; BF_CW = 2: two adjacent cells per thread (packed FP32x2 step)
-constexpr int BF_TX = 32, BF_TY = 16, BF_CW = 2;
-
 template <int S>
 static int step_bf16_t(dbm_handle *h, int cur, cudaStream_t st)
 {

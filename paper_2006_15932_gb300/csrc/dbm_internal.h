@@ -107,7 +107,7 @@ struct dbm_handle {
     int tma_ok;           // the TMA-staged step kernel can run
     int tma_tx, tma_ty;   // its tile (cells) and cells per thread (1 or 2),
     int tma_cw;           // fixed at dbm_bind
-    int told_tx, told_ty, told_cw;  // what dbm_step_tile answers (choose_tile)
+    int told_tx, told_ty, told_cw;  // what dbm_step_tile answers (told_tile)
     int tma_staged;       // the species-staged step (one species per copy)
     int tma_half;         // two threads per pair of cells (k_step_half)
     int sms;              // SMs of the device current at dbm_bind
@@ -170,6 +170,10 @@ constexpr long long PAIR_MIN_TILES = 4096, PAIR_MIN_RUN = 128;
 // a step against 6.2).
 constexpr int SMALL_TX = 32, SMALL_TY = 4;
 
+// Tile of the BF16-deviation step: 32 x 16 measured fastest of 64x8, 32x16,
+// 32x8, 32x7 and 64x4; BF_CW = 2: two adjacent cells per thread (packed FP32x2).
+constexpr int BF_TX = 32, BF_TY = 16, BF_CW = 2;
+
 // CTAs of a TX x TY tile kernel that fit on one SM at once, limited by
 // shared memory (the tile plus halo of 16 S float planes, and 1 KB reserved
 // per CTA) and by registers (at least 64 per cell: 64 per thread for one
@@ -194,6 +198,11 @@ int launch_moments(dbm_handle *h, const void *f, double *out, cudaStream_t st);
 int launch_noneq(dbm_handle *h, const void *f, double *out, cudaStream_t st);
 int launch_conservation(dbm_handle *h, const void *f, double *out, cudaStream_t st);
 int launch_conservation_noalloc(dbm_handle *h, const void *f, double *out, cudaStream_t st);
+
+// the step kernel of a bound handle (dbm_step_kernel_name), by the fields and
+// rules that launch_step dispatches on
+int step_kernel_name(const dbm_handle *h, char *name, size_t size);
+bool f64_small_grid(const dbm_handle *h);  // the FP64 step takes its 4-cell kernel
 
 template <typename real, int S>
 void fill_step_consts(const dbm_handle *h, StepConsts<real, S> &c);

@@ -2,6 +2,7 @@
 // kernel variant, and the TMA descriptors of the state buffers.  The
 // kernels are in dbm_step_impl.cuh, instantiated once per species count in
 // dbm_step_s<S>.cu so that the units compile in parallel.
+#include <stdio.h>
 #include <string.h>
 
 #include "dbm_internal.h"
@@ -72,6 +73,11 @@ static bool staged_supported(const dbm_params &p)
     return p.precision == DBM_FP32 && p.nspecies >= 2 && p.nspecies <= DBM_MAX_SPECIES && !uses_acc(p);
 }
 
+static long long pair_tiles(const dbm_params &p)
+{
+    return (long long)((p.nx + PAIR_TX - 1) / PAIR_TX) * ((p.ny + PAIR_TY - 1) / PAIR_TY);
+}
+
 // The tile of the TMA-staged step, without the arithmetic options:
 // two species: two cells per thread from PAIR_MIN_RUN tiles up (us a step,
 //   one cell / pairs: 4096^2 845 / 726, 1024^2 68 / 60, 1001 x 771 51 / 45,
@@ -88,11 +94,6 @@ static bool staged_supported(const dbm_params &p)
 // DBM_KERNEL_TMA_CELL asks for one cell per thread, DBM_KERNEL_TMA_PAIR and
 // _STAGED for two.  With an option: two species pairs from PAIR_MIN_TILES
 // tiles up, else one cell.
-//
-// dbm_step_tile's answer is fixed by its own rule, older than pairs on small
-// grids: it names the pair tile for two species from PAIR_MIN_TILES tiles up
-// (or when pairs are asked for) and the one-cell tile below, for four species
-// the one-cell tile's former 32 x 6, for the species-staged step 64 x 8 pairs.
 static void choose_tile(dbm_handle *h)
 {
     const dbm_params &p = h->p;
@@ -105,17 +106,11 @@ static void choose_tile(dbm_handle *h)
         h->tma_tx = staged_tile_x(p.nspecies);
         h->tma_ty = staged_tile_y(p.nspecies);
         h->tma_cw = staged_cw(p.nspecies);
-        h->told_tx = PAIR_TX;
-        h->told_ty = PAIR_TY;
-        h->told_cw = 2;
         return;
     }
-    bool told_pair = false, pair = false;
-    if (p.nspecies == 2 && want != DBM_KERNEL_TMA_CELL) {
-        const long long tiles = (long long)((p.nx + PAIR_TX - 1) / PAIR_TX) * ((p.ny + PAIR_TY - 1) / PAIR_TY);
-        told_pair = want == DBM_KERNEL_TMA_PAIR || tiles >= PAIR_MIN_TILES;
-        pair = told_pair || (!uses_acc(p) && tiles >= PAIR_MIN_RUN);
-    }
+    const bool pair = p.nspecies == 2 && want != DBM_KERNEL_TMA_CELL &&
+                      (want == DBM_KERNEL_TMA_PAIR ||
+                       pair_tiles(p) >= (uses_acc(p) ? PAIR_MIN_TILES : PAIR_MIN_RUN));
     if (!uses_acc(p) && want != DBM_KERNEL_TMA_CELL && !pair) {
         const long long small = (long long)((p.nx + SMALL_TX - 1) / SMALL_TX) * ((p.ny + SMALL_TY - 1) / SMALL_TY);
         h->tma_half = p.nspecies == 2 || (p.nspecies == 4 && small <= h->sms);
@@ -123,9 +118,39 @@ static void choose_tile(dbm_handle *h)
     h->tma_tx = pair ? PAIR_TX : h->tma_half ? SMALL_TX : tma_tile_x(p.nspecies);
     h->tma_ty = pair ? PAIR_TY : h->tma_half ? SMALL_TY : tma_tile_y(p.nspecies);
     h->tma_cw = pair ? 2 : 1;
-    h->told_tx = told_pair ? PAIR_TX : tma_tile_x(p.nspecies);
-    h->told_ty = told_pair ? PAIR_TY : p.nspecies == 4 ? 6 : tma_tile_y(p.nspecies);
-    h->told_cw = told_pair ? 2 : 1;
+}
+
+// dbm_step_tile's answer: a rule of its own, which programs have read and
+// dbm.h states; the step follows choose_tile.
+static void told_tile(dbm_handle *h)
+{
+    const dbm_params &p = h->p;
+    const bool pair = h->tma_staged || (p.nspecies == 2 && p.step_kernel != DBM_KERNEL_TMA_CELL &&
+                                        (p.step_kernel == DBM_KERNEL_TMA_PAIR || pair_tiles(p) >= PAIR_MIN_TILES));
+    h->told_tx = pair ? PAIR_TX : tma_tile_x(p.nspecies);
+    h->told_ty = pair ? PAIR_TY : p.nspecies == 4 ? 6 : tma_tile_y(p.nspecies);
+    h->told_cw = pair ? 2 : 1;
+}
+
+int step_kernel_name(const dbm_handle *h, char *name, size_t size)
+{
+    const dbm_params &p = h->p;
+    const int S = p.nspecies;
+    if (p.precision == DBM_FP64) {
+        snprintf(name, size, "%s<%d>", f64_small_grid(h) ? "k_step_f64_small" : "k_step_f64", S);
+    } else if (p.precision == DBM_BF16DEV) {
+        snprintf(name, size, "k_step_bf16<%d,%d,%d,%d>", S, BF_TX, BF_TY, BF_CW);
+    } else if (!h->tma_ok || p.step_kernel == DBM_KERNEL_GENERIC) {
+        if (uses_acc(p) || (p.step_kernel != DBM_KERNEL_AUTO && p.step_kernel != DBM_KERNEL_GENERIC))
+            return DBM_ERR_INVALID;
+        snprintf(name, size, "k_step<%d>", S);
+    } else if (h->tma_half) {
+        snprintf(name, size, "k_step_half<%d,%d,%d>", S, h->tma_tx, h->tma_ty);
+    } else {
+        snprintf(name, size, "%s<%d,%d,%d,%d>", h->tma_staged ? "k_step_staged" : "k_step_tma", S, h->tma_tx, h->tma_ty,
+                 h->tma_cw);
+    }
+    return DBM_OK;
 }
 
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -152,6 +177,7 @@ int make_tensor_maps(dbm_handle *h)
     cuuint64_t dims[3] = {(cuuint64_t)L.pitch, (cuuint64_t)L.rows, (cuuint64_t)(16 * h->p.nspecies)};
     cuuint64_t strides[2] = {(cuuint64_t)L.pitch * 4, (cuuint64_t)L.plane * 4};
     choose_tile(h);
+    told_tile(h);
     if (!h->tma_staged && !tma_supported(h->p)) {  // no all-species kernel for this species count
         h->tma_tx = h->tma_ty = h->tma_cw = 0;
         return DBM_OK;

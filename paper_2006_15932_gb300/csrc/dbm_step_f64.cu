@@ -710,13 +710,15 @@ __global__ void __launch_bounds__(128 + 32 * small_ring_warps(S))
 // a force 63 / 71, 76 / 71).
 constexpr long long SMALL_GRID = 16 * 152;
 
+bool f64_small_grid(const dbm_handle *h) { return (long long)h->p.nx * h->p.ny <= SMALL_GRID; }
+
 template <int S>
 static int launch_f64_t(dbm_handle *h, const double *fin, double *fout, cudaStream_t st)
 {
     F64Consts<S> c;
     fill_f64_consts<S>(h, c);
     const long long cells = (long long)h->p.nx * h->p.ny;
-    if (cells > SMALL_GRID)
+    if (!f64_small_grid(h))
         return launch_f64_wide<S>(h, c, 1 + (c.has_reaction ? 1 : 0) + (c.has_force ? 2 : 0), fin, fout, st);
     static std::atomic<unsigned long long> allowed{0};
     const cudaError_t e = allow_smem(k_step_f64_small<S>, ALONE_SMEM, allowed);

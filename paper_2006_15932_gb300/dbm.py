@@ -43,7 +43,7 @@ EXPORTS = [
     "dbm_init", "dbm_init_error", "dbm_equilibrium_matrix", "dbm_get_layout", "dbm_state_bytes", "dbm_scratch_bytes",
     "dbm_bind", "dbm_set_state", "dbm_set_f", "dbm_get_f", "dbm_step", "dbm_moments",
     "dbm_nonequilibrium", "dbm_conservation", "dbm_conservation_noalloc", "dbm_status", "dbm_steps_taken",
-    "dbm_step_tile",
+    "dbm_step_kernel_name", "dbm_step_tile",
     "dbm_last_error", "dbm_destroy", "dbm_batch_table_bytes", "dbm_batch_create", "dbm_batch_tune",
     "dbm_batch_step", "dbm_batch_info", "dbm_batch_get_config", "dbm_batch_set_config", "dbm_batch_last_error",
     "dbm_batch_destroy",
@@ -136,6 +136,7 @@ def load(path: str = LIB_PATH):
     L.dbm_status.argtypes = [H, vp, C.POINTER(C.c_uint)]
     L.dbm_steps_taken.argtypes = [H]
     L.dbm_steps_taken.restype = C.c_longlong
+    L.dbm_step_kernel_name.argtypes = [H, C.c_char_p, C.c_size_t]
     L.dbm_step_tile.argtypes = [H] + [C.POINTER(C.c_int)] * 3
     L.dbm_last_error.argtypes = [H]
     L.dbm_last_error.restype = C.c_char_p
@@ -290,9 +291,17 @@ def dbm_steps_taken(h) -> int:
     return load().dbm_steps_taken(h)
 
 
+def dbm_step_kernel_name(h) -> str:
+    """The kernel dbm_step launches, with its template arguments."""
+    buf = C.create_string_buffer(64)
+    _check(h, load().dbm_step_kernel_name(h, buf, len(buf)))
+    return buf.value.decode()
+
+
 def dbm_step_tile(h) -> tuple[int, int, int]:
-    """(tile_x, tile_y, cells_per_thread) of the step's shared-memory tile;
-    (0, 0, 0) when the step runs a kernel without one."""
+    """(tile_x, tile_y, cells_per_thread) by the size rule in dbm.h, which the
+    step itself may differ from (dbm_step_kernel_name); (0, 0, 0) when the step
+    runs a kernel without a shared-memory tile."""
     tx, ty, cw = C.c_int(), C.c_int(), C.c_int()
     _check(h, load().dbm_step_tile(h, C.byref(tx), C.byref(ty), C.byref(cw)))
     return tx.value, ty.value, cw.value
@@ -422,9 +431,13 @@ class Solver:
     def status(self):
         return dbm_status(self.h, self._st())
 
+    def step_kernel_name(self):
+        """The kernel a step launches, with its template arguments."""
+        return dbm_step_kernel_name(self.h)
+
     def step_tile(self):
-        """(tile_x, tile_y, cells_per_thread) of the step kernel; zeros when
-        it has no shared-memory tile."""
+        """(tile_x, tile_y, cells_per_thread) by the size rule of
+        dbm_step_tile; step_kernel_name() says what runs."""
         return dbm_step_tile(self.h)
 
     def close(self):
