@@ -142,8 +142,9 @@ enum dbm_step_kernel {
     DBM_KERNEL_TMA_STAGED = 5 /* TMA-staged one species at a time through two shared-
                                  memory buffers (each species copied for its moment
                                  sums and again for its update), two adjacent cells
-                                 per thread on 64 x 8 tiles (S >= 5: one on 32 x 8);
-                                 2 <= S <= 8, without the thermo and rounding options */
+                                 per thread on 64 x 8 tiles (S >= 5: one on 32 x 8,
+                                 two for DBM_KERNEL_TMA_PAIR); 2 <= S <= 8, without
+                                 the thermo and rounding options                     */
 };
 
 /* Constants of one species sigma. */

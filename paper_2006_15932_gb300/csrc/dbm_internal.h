@@ -159,11 +159,10 @@ constexpr int PAIR_TX = 64, PAIR_TY = 8;
 // instructions (us a step, two cells per thread on 64 x 8 with two CTAs / this:
 // 1024^2, five 197 / 193; 777 x 413, six 121 / 106; 1024 x 512, eight 200 / 183;
 // 128^2, five 31 / 20; 32 x 7, 32 x 6, 32 x 10 and 64 x 4 were slower).  Two to
-// four, when asked for: two cells per thread on 64 x 8 (2048 x 1024, three
+// four when asked for, and more when two cells per thread are asked for
+// (DBM_KERNEL_TMA_PAIR): two cells per thread on PAIR_TX x PAIR_TY (2048 x 1024, three
 // 202 / 212, four 274 / 303).
-constexpr int staged_cw(int S) { return S >= 5 ? 1 : 2; }
-constexpr int staged_tile_x(int S) { return S >= 5 ? 32 : 64; }
-constexpr int staged_tile_y(int) { return 8; }
+constexpr int STAGED_TX = 32, STAGED_TY = 8;
 constexpr long long PAIR_MIN_TILES = 4096, PAIR_MIN_RUN = 128;
 // Small grids of two and four species: two threads per pair of cells on
 // SMALL_TX x SMALL_TY tiles (k_step_half; 32 x 8 on 128^2, two species, 6.6 us

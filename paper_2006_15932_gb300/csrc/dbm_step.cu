@@ -25,7 +25,9 @@ template <int S>
 static int launch_staged_s(dbm_handle *h, const CUtensorMap *tm, const CUtensorMap *ti, const void *fin, void *fout,
                            cudaStream_t st)
 {
-    return launch_step_staged_t<S, staged_tile_x(S), staged_tile_y(S), staged_cw(S)>(h, tm, ti, fin, fout, st);
+    if constexpr (S >= 5)
+        if (h->tma_cw == 1) return launch_step_staged_t<S, STAGED_TX, STAGED_TY, 1>(h, tm, ti, fin, fout, st);
+    return launch_step_staged_t<S, PAIR_TX, PAIR_TY, 2>(h, tm, ti, fin, fout, st);
 }
 
 // The species-staged step of the handle's tile (no arithmetic options).
@@ -91,8 +93,10 @@ static long long pair_tiles(const dbm_params &p)
 //   per pair on grids of at most a small tile per SM (128^2 10.7 / 8.3, 777 x
 //   413 62 / 91);
 // five or more: the species-staged kernel, the only TMA-staged one.
-// DBM_KERNEL_TMA_CELL asks for one cell per thread, DBM_KERNEL_TMA_PAIR and
-// _STAGED for two.  With an option: two species pairs from PAIR_MIN_TILES
+// DBM_KERNEL_TMA_CELL asks for one cell per thread, DBM_KERNEL_TMA_PAIR for two
+// (three and more species: staged), DBM_KERNEL_TMA_STAGED for the
+// species-staged kernel, in pairs up to four species and one cell per thread
+// from five on.  With an option: two species pairs from PAIR_MIN_TILES
 // tiles up, else one cell.
 static void choose_tile(dbm_handle *h)
 {
@@ -103,9 +107,10 @@ static void choose_tile(dbm_handle *h)
     const bool staged_asked = want == DBM_KERNEL_TMA_STAGED || (p.nspecies >= 3 && want == DBM_KERNEL_TMA_PAIR);
     if (staged_supported(p) && (staged_by_default || staged_asked)) {
         h->tma_staged = 1;
-        h->tma_tx = staged_tile_x(p.nspecies);
-        h->tma_ty = staged_tile_y(p.nspecies);
-        h->tma_cw = staged_cw(p.nspecies);
+        const bool pair = p.nspecies < 5 || want == DBM_KERNEL_TMA_PAIR;
+        h->tma_tx = pair ? PAIR_TX : STAGED_TX;
+        h->tma_ty = pair ? PAIR_TY : STAGED_TY;
+        h->tma_cw = pair ? 2 : 1;
         return;
     }
     const bool pair = p.nspecies == 2 && want != DBM_KERNEL_TMA_CELL &&

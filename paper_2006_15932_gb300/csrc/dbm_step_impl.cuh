@@ -1646,7 +1646,7 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
 // planes of one species (BX x BY cells), so the shared memory of a CTA does
 // not grow with the species count: five and more species, whose all-species
 // tile fits no useful shape, run one cell per thread at three CTAs per SM, fewer
-// (when asked for) two cells per thread at two (staged_cw has the figures).
+// (when asked for) two cells per thread at two (STAGED_TX has the figures).
 // Each species is copied twice per tile: for its moment
 // sums only its TX x TY own cells (a second descriptor, an interior box; no
 // halo), for its update the tile and its halo.  Use k = 0 .. 2S-1 takes

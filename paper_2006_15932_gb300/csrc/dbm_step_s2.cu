@@ -7,8 +7,8 @@ template int launch_step_tma_t<2, tma_tile_x(2), tma_tile_y(2), 1, 0>(dbm_handle
                                      cudaStream_t);
 template int launch_step_tma_t<2, PAIR_TX, PAIR_TY, 2, 0>(dbm_handle *, const CUtensorMap *, const CUtensorMap *, const void *, void *,
                                      cudaStream_t);
-template int launch_step_staged_t<2, staged_tile_x(2), staged_tile_y(2), staged_cw(2)>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
-                                                                const void *, void *, cudaStream_t);
+template int launch_step_staged_t<2, PAIR_TX, PAIR_TY, 2>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
+                                     const void *, void *, cudaStream_t);
 template int launch_step_half_t<2, SMALL_TX, SMALL_TY>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
                                      const void *, void *, cudaStream_t);
 }  // namespace dbm

@@ -3,6 +3,8 @@
 
 namespace dbm {
 template int launch_step_t<6>(dbm_handle *, const void *, void *, cudaStream_t);
-template int launch_step_staged_t<6, staged_tile_x(6), staged_tile_y(6), staged_cw(6)>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
-                                                                const void *, void *, cudaStream_t);
+template int launch_step_staged_t<6, PAIR_TX, PAIR_TY, 2>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
+                                     const void *, void *, cudaStream_t);
+template int launch_step_staged_t<6, STAGED_TX, STAGED_TY, 1>(dbm_handle *, const CUtensorMap *, const CUtensorMap *,
+                                     const void *, void *, cudaStream_t);
 }  // namespace dbm
