@@ -1419,11 +1419,14 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
     __syncthreads();
     const int tid = ty * (TX / CW) + tx;
     const HaloSides hs = halo_sides<TX, TY>(bx0, by0, c.nx, c.ny);
-    // one cell per thread: a boundary tile's halo is loaded beside its copies
-    // (us a step: 1024 x 256, three species 28.2 -> 27.0; 777 x 413, four 61.6 ->
-    // 58.9); a pair's registers are full and its halo is filled afterwards
-    // (256^2, two species 8.2, loaded beside 8.5)
-    constexpr bool EARLY = CW == 1;
+    // one cell per thread, two species and more: a boundary tile's halo is loaded
+    // beside its copies (us a step: 256^2, two species 8.1 -> 7.3; 1024 x 256,
+    // three 28.2 -> 27.0; 777 x 413, four 61.6 -> 58.9).  A pair's registers are
+    // full and its halo is filled afterwards (256^2, two species 8.2, loaded
+    // beside 8.5); so are one species' 64 registers, four CTAs of 256 threads,
+    // where the halo spilled (filled / loaded beside: 4096^2 421 / 425, 1025 x 771
+    // 26.4 / 26.9, 256^2 4.5 / 4.3, with the FP64 thermo 17.2 / 19.9)
+    constexpr bool EARLY = CW == 1 && S >= 2;
     HaloRegs<NP, TX, TY, NT> hr;
     if (EARLY && hs.any())
         halo_load(hr, hs, fin, bx0, by0, c.nx, c.ny, c.pitch, c.plane, c.bc_x, c.bc_y, tid, flag);
