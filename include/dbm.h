@@ -127,12 +127,13 @@ enum dbm_step_kernel {
                                  DBM_KERNEL_TMA                                      */
     DBM_KERNEL_GENERIC = 1,   /* stencil read from global memory                      */
     DBM_KERNEL_TMA = 2,       /* tile + halo staged in shared memory by TMA copies:
-                                 S = 1, 3: one cell per thread; S = 2: two cells
-                                 per thread on grids of at least 128 tiles of 64 x 8
-                                 cells, two threads per pair of cells on smaller ones
-                                 (with the thermo or rounding option: from 4096
-                                 tiles, else one cell per thread); S = 4: one cell per
-                                 thread, or two threads per pair on small grids;
+                                 S = 1, 3: one cell per thread; S = 2: two threads
+                                 per pair of cells on grids of up to three tiles of
+                                 32 x 4 cells per SM, else two cells per thread (with
+                                 the thermo or rounding option: from 4096 tiles of
+                                 64 x 8 cells, else one cell per thread); S = 4: two
+                                 threads per pair on grids of up to one such tile
+                                 per SM, else one cell per thread;
                                  S >= 5: as
                                  DBM_KERNEL_TMA_STAGED                               */
     DBM_KERNEL_TMA_CELL = 3,  /* TMA-staged, all planes in one copy, one cell per

@@ -163,11 +163,14 @@ constexpr int PAIR_TX = 64, PAIR_TY = 8;
 // (DBM_KERNEL_TMA_PAIR): two cells per thread on PAIR_TX x PAIR_TY (2048 x 1024, three
 // 202 / 212, four 274 / 303).
 constexpr int STAGED_TX = 32, STAGED_TY = 8;
-constexpr long long PAIR_MIN_TILES = 4096, PAIR_MIN_RUN = 128;
+constexpr long long PAIR_MIN_TILES = 4096;  // with an arithmetic option
 // Small grids of two and four species: two threads per pair of cells on
 // SMALL_TX x SMALL_TY tiles (k_step_half; 32 x 8 on 128^2, two species, 6.6 us
-// a step against 6.2).
+// a step against 6.2), while the grid's tiles are on the chip at once: three
+// CTAs of 128 threads per SM by registers with two species, and no more than
+// one with four, whose threads then have the SM's issue slots to themselves.
 constexpr int SMALL_TX = 32, SMALL_TY = 4;
+constexpr int small_tiles_per_sm(int S) { return S == 2 ? 3 : S == 4 ? 1 : 0; }
 
 // Tile of the BF16-deviation step: 32 x 16 measured fastest of 64x8, 32x16,
 // 32x8, 32x7 and 64x4; BF_CW = 2: two adjacent cells per thread (packed FP32x2).

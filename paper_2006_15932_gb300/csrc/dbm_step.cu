@@ -81,16 +81,17 @@ static long long pair_tiles(const dbm_params &p)
 }
 
 // The tile of the TMA-staged step, without the arithmetic options:
-// two species: two cells per thread from PAIR_MIN_RUN tiles up (us a step,
-//   one cell / pairs: 4096^2 845 / 726, 1024^2 68 / 60, 1001 x 771 51 / 45,
-//   512^2 20.0 / 17.7, 256^2, 128 tiles, 9.1 / 8.1), below that two threads per
-//   pair, whose chain is the shortest (one cell / two threads: 256 x 200 9.1 /
-//   6.4, 128^2 7.4 / 5.8, 64^2 7.4 / 4.4, 400 x 1 6.6 / 5.3);
+// two species: two threads per pair, whose chain is the shortest, while three
+//   small tiles per SM hold the grid (us a step, two threads / pairs, on 152 SMs:
+//   256 x 128 6.1 / 8.0, 256 x 200, 400 tiles, 6.3 / 8.1, 704 x 80, 440 tiles, 6.4 /
+//   8.3; past 456 tiles a second wave: 832 x 72, 468, 9.3 / 8.3, 768 x 80, 480, 9.8 /
+//   8.4), then two cells per thread (one cell / pairs: 4096^2 845 / 726, 1024^2
+//   68 / 60, 1001 x 771 51 / 45, 512^2 20.0 / 17.7);
 // one and three species: one cell per thread (three species, two threads per
 //   pair: 128^2 7.5 / 8.0, 256^2 9.9 / 14.6; species-staged: 2048 x 1024 174 /
 //   201);
 // four: one cell per thread (2048 x 1024 261, species-staged 265), two threads
-//   per pair on grids of at most a small tile per SM (128^2 10.7 / 8.3, 777 x
+//   per pair on grids of at most one small tile per SM (128^2 10.7 / 8.3, 777 x
 //   413 62 / 91);
 // five or more: the species-staged kernel, the only TMA-staged one.
 // DBM_KERNEL_TMA_CELL asks for one cell per thread, DBM_KERNEL_TMA_PAIR for two
@@ -113,13 +114,11 @@ static void choose_tile(dbm_handle *h)
         h->tma_cw = pair ? 2 : 1;
         return;
     }
-    const bool pair = p.nspecies == 2 && want != DBM_KERNEL_TMA_CELL &&
-                      (want == DBM_KERNEL_TMA_PAIR ||
-                       pair_tiles(p) >= (uses_acc(p) ? PAIR_MIN_TILES : PAIR_MIN_RUN));
-    if (!uses_acc(p) && want != DBM_KERNEL_TMA_CELL && !pair) {
-        const long long small = (long long)((p.nx + SMALL_TX - 1) / SMALL_TX) * ((p.ny + SMALL_TY - 1) / SMALL_TY);
-        h->tma_half = p.nspecies == 2 || (p.nspecies == 4 && small <= h->sms);
-    }
+    const long long small = (long long)((p.nx + SMALL_TX - 1) / SMALL_TX) * ((p.ny + SMALL_TY - 1) / SMALL_TY);
+    h->tma_half = !uses_acc(p) && want != DBM_KERNEL_TMA_CELL && want != DBM_KERNEL_TMA_PAIR &&
+                  small <= (long long)small_tiles_per_sm(p.nspecies) * h->sms;
+    const bool pair = p.nspecies == 2 && want != DBM_KERNEL_TMA_CELL && !h->tma_half &&
+                      (want == DBM_KERNEL_TMA_PAIR || !uses_acc(p) || pair_tiles(p) >= PAIR_MIN_TILES);
     h->tma_tx = pair ? PAIR_TX : h->tma_half ? SMALL_TX : tma_tile_x(p.nspecies);
     h->tma_ty = pair ? PAIR_TY : h->tma_half ? SMALL_TY : tma_tile_y(p.nspecies);
     h->tma_cw = pair ? 2 : 1;

@@ -705,12 +705,14 @@ __global__ void __launch_bounds__(128 + 32 * small_ring_warps(S))
     if (mx | my) store_images(po, (int)x, (int)y, c.nx, c.ny, c.pitch, mx, my, fnew);
 }
 
-// Grids of up to this many cells take the 4-cell kernel (us a step, 4 cells /
-// 32 cells: two species 2048 cells 20.2 / 25.7, 3000 cells 27.6 / 25.8; four under
-// a force 63 / 71, 76 / 71).
-constexpr long long SMALL_GRID = 16 * 152;
+// Grids of up to four 4-cell CTAs per SM take the 4-cell kernel (us a step on 152
+// SMs, 4 cells / 32 cells: two species 2048 cells 20.2 / 25.7, 3000 cells 27.6 /
+// 25.8; four under a force 63 / 71, 76 / 71; either side of the line, 2432 and
+// 2433 cells: one species 18.8 / 19.8, two 20.2 / 26.1, eight under a force 122 /
+// 136).
+constexpr int SMALL_CELLS_PER_SM = 4 * SMALL_CELLS;
 
-bool f64_small_grid(const dbm_handle *h) { return (long long)h->p.nx * h->p.ny <= SMALL_GRID; }
+bool f64_small_grid(const dbm_handle *h) { return (long long)h->p.nx * h->p.ny <= (long long)SMALL_CELLS_PER_SM * h->sms; }
 
 template <int S>
 static int launch_f64_t(dbm_handle *h, const double *fin, double *fout, cudaStream_t st)
