@@ -7,8 +7,8 @@
 // holds, for every instance of the chunk, its step constants, the TMA
 // descriptor of its input buffer and its output pointers.  A CTA takes one
 // tile (or a contiguous range of tiles) from the device tile list, stages
-// the tile plus halo with one TMA copy through its instance's descriptor
-// and runs the same per-cell arithmetic as the single-problem kernel, with
+// the tile plus halo with one TMA copy per species through its instance's
+// descriptor and runs the same per-cell arithmetic as the single-problem kernel, with
 // the constants read from the constant bank (shared-memory copies of them
 // would compete with the stencil reads).  Pairs of steps are replayed from
 // a CUDA graph in which each chunk is an independent two-launch chain; the

@@ -133,22 +133,21 @@ namespace dbm {
 // 256 threads per SM), 32 x 8 for three (92 KB of shared memory, two CTAs),
 // 32 x 7 for four (113 KB, two CTAs of 224 threads, the tallest that fits
 // twice; us a step against 32 x 6: 2048 x 1024 242 / 254, 777 x 413 56.7 / 58.9;
-// 32x4, 64x4, 32x2, 32x3 and 64x2 were slower than that).  Measured fastest among 32x16, 32x12, 32x10, 32x9, 32x8,
+// 32x4, 64x4, 32x2, 32x3 and 64x2 were slower than that), 32 x 7 for two (56 KB,
+// four CTAs of 224 threads).  Chosen among 32x16, 32x12, 32x10, 32x9, 32x8,
 // 32x7, 32x6, 32x5, 32x4, 40x8, 48x6, 64x8, 64x6, 64x5, 64x4, 128x4 and
 // others on 4096 x 4096 (two species) and 4096 x 2048 (one) grids: more
 // resident CTAs per SM hide each CTA's wait for its tile.  For three species
-// 64 x 4 is 3 % faster on 2048 x 2048 but 10 % slower on the 1024 x 256
-// reactive gas, whose halo re-reads (2.25x against 1.9x) come from L2.  Two
-// species: 32 x 7 with one cell per thread (56 KB, four CTAs of 224
-// threads), or two cells per thread on PAIR_TX x PAIR_TY =
-// 64 x 8 cells (110 KB, two CTAs of 256 threads): one thread per cell runs
-// 812 instructions per species-cell and is issue-bound; pairs run 528, and
-// the taller tile keeps 16 warps per SM (on 4096 x 4096: 42.0 G/s against
-// 37.7; pairs on 64 x 4, 64 x 6 and 64 x 7 gave 39.6, 36.1 and 39.9).
-// Pairs win on small grids too since the limiter's and the copies' cost came
-// down (choose_tile has the figures).  Three species in pairs hold half the warps
-// per SM and ran slower (64 x 4 and 32 x 8: 12.4 and 15.5 G/s against 21.4
-// on the 1024 x 256 reactive gas, 25.2 and 26.6 against 31.2 on 2048 x 1024).
+// 64 x 4 was 3 % faster on 2048 x 2048 but 10 % slower on the 1024 x 256
+// reactive gas, whose halo re-reads (2.25x against 1.9x) come from L2.
+//
+// Two species on grids that fill the chip: two cells per thread on PAIR_TX x
+// PAIR_TY = 64 x 8 cells (110 KB, two CTAs of 256 threads).  One thread per cell
+// runs 762 instructions per species-cell and is issue-bound; pairs run 469, and
+// the taller tile keeps 16 warps per SM (4096 x 4096 726 us a step, one cell 845;
+// when the tile was chosen, G/s: 64 x 8 42.0, 64 x 4 39.6, 64 x 6 36.1, 64 x 7
+// 39.9).  Three species in pairs held half the warps per SM and ran slower (64 x 4
+// and 32 x 8 then 12.4 and 15.5 G/s against 21.4 on the 1024 x 256 reactive gas).
 constexpr int tma_tile_x(int S) { return S == 1 ? 64 : 32; }
 constexpr int tma_tile_y(int S) { return S == 1 ? 4 : S == 3 ? 8 : 7; }
 constexpr int PAIR_TX = 64, PAIR_TY = 8;

@@ -91,8 +91,8 @@ static long long pair_tiles(const dbm_params &p)
 //   pair: 128^2 7.5 / 8.0, 256^2 9.9 / 14.6; species-staged: 2048 x 1024 174 /
 //   201);
 // four: one cell per thread (2048 x 1024 261, species-staged 265), two threads
-//   per pair on grids of at most one small tile per SM (128^2 10.7 / 8.3, 777 x
-//   413 62 / 91);
+//   per pair on grids of at most one small tile per SM (one cell / two threads:
+//   64^2 8.7 / 7.7, 128^2 8.4 / 8.1, 777 x 413 57 / 91);
 // five or more: the species-staged kernel, the only TMA-staged one.
 // DBM_KERNEL_TMA_CELL asks for one cell per thread, DBM_KERNEL_TMA_PAIR for two
 // (three and more species: staged), DBM_KERNEL_TMA_STAGED for the

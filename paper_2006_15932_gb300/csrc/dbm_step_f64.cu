@@ -82,9 +82,9 @@ __device__ __forceinline__ double minmod_bits(double a, double b)
     return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(m);
 }
 
-// d(c f)/dx of one velocity component of magnitude v at the cell p points
-// to; e: element offset of the neighbour downwind (the sign of c times the
-// stride), g0 = v f.  Seen along c, both signs have the same flux
+// d(c f)/dx of one velocity component of magnitude v at a cell: fm2, fm1, fp1
+// are f two cells and one cell upwind and one downwind, g0 = v f at the cell, h
+// the grid spacing.  Seen along c, both signs have the same flux
 // H = v f + minmod(...)/2.
 __device__ __forceinline__ double nnd_dflux(double fm2, double fm1, double fp1, double g0, double v,
                                             const ConstDiv &h)

@@ -1475,7 +1475,9 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
 // threads, the partial moment sums (half 0 to half 1, which adds its rings in
 // the same order as one thread would) and the mixture (back).  A boundary
 // tile's halo is loaded beside its copies.  Same bits.  Two species, us a
-// step: 128^2 7.4 (one cell) -> 5.8.  On grids that fill the chip the second
+// step: 128^2 7.4 (one cell, its halo filled after the copy) -> 5.8; with its
+// halo loaded beside the copies the one-cell step takes 4.4 there, 256 x 128 5.5
+// against 6.1, 256 x 200 6.4 against 6.3.  On grids that fill the chip the second
 // copy of the step's code and the exchange cost more than the shorter threads
 // give (three species 1024^2 97 -> 119).
 // the tile, then the exchange area: 4 S pairs per pair of cells
@@ -1649,12 +1651,11 @@ int launch_step_tma_t(dbm_handle *h, const CUtensorMap *tmap, const CUtensorMap 
 // planes of one species (BX x BY cells), so the shared memory of a CTA does
 // not grow with the species count: five and more species, whose all-species
 // tile fits no useful shape, run one cell per thread at three CTAs per SM, fewer
-// (when asked for) two cells per thread at two (STAGED_TX has the figures).
-// Each species is copied twice per tile: for its moment
-// sums only its TX x TY own cells (a second descriptor, an interior box; no
-// halo), for its update the tile and its halo.  Use k = 0 .. 2S-1 takes
-// species k mod S from buffer k & 1,
-// whose mbarrier completes its phase k >> 1 with that copy; while a use is
+// (and any count that asks for pairs) two cells per thread at two (STAGED_TX has
+// the figures).  Each species is copied twice per tile: for its moment sums only
+// its TX x TY own cells (a second descriptor, an interior box; no halo), for its
+// update the tile and its halo.  Use k = 0 .. 2S-1 takes species k mod S from
+// buffer k & 1, whose mbarrier completes its phase k >> 1 with that copy; while a use is
 // computed the copy of the next one is in flight, and once every thread is
 // done with a buffer (the barrier in release) the leader refills it for use
 // k + 2.  A tile at the domain boundary fills each copy's halo from the
