@@ -476,9 +476,9 @@ __global__ void __launch_bounds__(128)
 // 2^-57 of them in the worst case, so nothing is lost that FP64 additions of
 // the values would keep; a total past the float range is formed again in FP64.
 // This runs on the FP32 pipes, 13 additions a value; the FP64 pipe, two lanes
-// per SM and cycle, gets 2 per species and cell.  Multiplying every value by its
-// weights in FP64 took 190 (4096^2, two species: 8.7 -> 0.67 ms; in two floats,
-// 48 bits, 0.65).
+// per SM and cycle, gets one per species and cell.  Multiplying every value by its
+// weights in FP64 took 190 (4096^2, two species: 8.7 -> 0.59 ms; with the ring
+// sums of a group and twelve trees a warp in FP64 0.67).
 struct FloatTriple {
     float h, l, t;
     __device__ __forceinline__ void add(float f)
@@ -489,7 +489,19 @@ struct FloatTriple {
         t = __fadd_rn(t, e2);
     }
     __device__ __forceinline__ double value() const { return widen(h) + (widen(l) + widen(t)); }
+    __device__ __forceinline__ float size() const { return fabsf(h) + fabsf(t); }  // not finite when any part is not
 };
+// a + sign b, exactly but for the rounding of t
+__device__ __forceinline__ FloatTriple triple_sum(const FloatTriple &a, const FloatTriple &b, float sign)
+{
+    FloatTriple s;
+    float e, e1, e2;
+    s.h = ff_sum(a.h, sign * b.h, e);
+    const float m = ff_sum(a.l, sign * b.l, e1);
+    s.l = ff_sum(m, e, e2);
+    s.t = __fadd_rn(__fmaf_rn(sign, b.t, a.t), __fadd_rn(e1, e2));
+    return s;
+}
 
 // Running totals of a species over a thread's cells.
 struct SpeciesTotalF {
@@ -504,20 +516,24 @@ struct SpeciesTotalF {
         a[4 * r].add(f0), a[4 * r + 1].add(f1), a[4 * r + 2].add(f2), a[4 * r + 3].add(f3);
     }
     // adds the ring sums; false, and nothing added, when a value was infinite or
-    // NaN or a float total overflowed
+    // NaN or a float total left the range (a running total that overflowed stays
+    // infinite or NaN)
     __device__ __forceinline__ bool flush(double acc[4][3]) const
     {
         bool finite = true;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) finite = finite && isfinite(a[i].h + a[i].t);
+        for (int r = 0; r < 4; ++r)  // of a ring's sums, so of its four totals
+            finite = finite && a[4 * r].size() + a[4 * r + 1].size() + a[4 * r + 2].size() + a[4 * r + 3].size() < 0x1p127f;
         if (!finite) return false;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            double f[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) f[i] = a[4 * r + i].value();
-            const RingSums g = ring_sums(r, f);
-            acc[r][0] += g.all, acc[r][1] += g.rx, acc[r][2] += g.ry;
+            // the ring's sums as in ring_sums
+            const FloatTriple *f = a + 4 * r;
+            const FloatTriple p = triple_sum(f[0], f[2], 1.0f), q = triple_sum(f[1], f[3], 1.0f);
+            const FloatTriple d = triple_sum(f[0], f[2], -1.0f), e = triple_sum(f[3], f[1], -1.0f);
+            acc[r][0] += triple_sum(p, q, 1.0f).value();
+            acc[r][1] += (r & 1) ? triple_sum(d, e, 1.0f).value() : d.value();
+            acc[r][2] += (r & 1) ? triple_sum(d, e, -1.0f).value() : -e.value();
         }
         return true;
     }
@@ -605,6 +621,33 @@ __device__ __forceinline__ double warp_total(double v)
     return v;
 }
 
+// The totals of twelve values over a warp, to out[0 .. 11].  Each exchange also
+// halves what a lane goes on with (12, 6, 3, 2, 1 values), so a lane makes 13
+// FP64 additions where twelve trees of their own take 60; the additions of a
+// value, and so its bits, are those of warp_total.
+__device__ __forceinline__ void warp_totals(const double *v, double *out)
+{
+    const int lane = threadIdx.x & 31;
+    double a[6], b[3];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const bool up = lane & 16;
+        a[i] = (up ? v[6 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[6 + i], 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const bool up = lane & 8;
+        b[i] = (up ? a[3 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[3 + i], 8);
+    }
+    const bool third = lane & 4, second = lane & 2;
+    const double c0 = (third ? b[2] : b[0]) + __shfl_xor_sync(0xffffffffu, third ? b[0] : b[2], 4);
+    const double c1 = b[1] + __shfl_xor_sync(0xffffffffu, b[1], 4);
+    double d = (second ? c1 : c0) + __shfl_xor_sync(0xffffffffu, second ? c0 : c1, 2);
+    d += __shfl_xor_sync(0xffffffffu, d, 1);
+    if ((lane & 1) == 0 && !(third && second))
+        out[(lane & 16 ? 6 : 0) + (lane & 8 ? 3 : 0) + (third ? 2 : second ? 1 : 0)] = d;
+}
+
 template <int S, class Src>
 __global__ void __launch_bounds__(256, 2)
     k_cons_partial(const __grid_constant__ OutConsts<S> c, const __grid_constant__ Src src,
@@ -648,13 +691,7 @@ __global__ void __launch_bounds__(256, 2)
         }
     }
     __shared__ double red[8][12];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double v = warp_total(acc[r][k]);
-            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][3 * r + k] = v;
-        }
+    warp_totals(&acc[0][0], red[threadIdx.x >> 5]);
     __syncthreads();
     if (threadIdx.x == 0) {
         double n = 0.0, jx = 0.0, jy = 0.0, en = 0.0;
