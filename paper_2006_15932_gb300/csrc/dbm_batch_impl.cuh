@@ -170,8 +170,7 @@ __global__ void __launch_bounds__(TX / CW * TY, tma_ctas_per_sm(S, TX, TY))
         const int x = cur.bx0 + CW * tx, y = cur.by0 + ty;
         const bool inside = x < g.nx && y < g.ny;
         if (hs.any() || !inside)
-            for (int s = 1; s < S; ++s)
-                if (!mbar_wait(b + 8u * s, phase, TMA_WAIT_LIMIT)) raise_flag(e.flag, DBM_HEALTH_TIMEOUT);
+            for (int s = 1; s < S; ++s) mbar_land(b + 8u * s, phase, e.flag);
         if (hs.any()) halo_store(hr, hs, tile, cur.bx0, cur.by0, g.nx, g.ny, tid, e.flag);
         if (inside) {
             StateOutNoImages o{e.fout, g.plane, (long long)NP * g.plane, e.flag};

@@ -1,4 +1,7 @@
-"""A chained step kernel (launched with programmatic serialization) starts
+"""Rules of the step kernels that no safe run can show broken, checked on the
+source.
+
+A chained step kernel (launched with programmatic serialization) starts
 while the kernel before it still writes the chained kernel's input.  A const
 __restrict__ parameter would promise that the input never changes while the
 kernel runs, and would allow its loads to move above the wait or to go through
@@ -38,3 +41,12 @@ cudaError_t go(const float *in, float *out) { return dbm::launch_chained(k_bare,
     r = subprocess.run([B.nvcc(), *B.ARCH, *B.NVCC_FLAGS, "-c", str(src), "-o", str(tmp_path / "bare.o")],
                        capture_output=True, text=True)
     assert r.returncode != 0 and "ChainedIn" in r.stdout + r.stderr, r.stderr
+
+
+def test_later_waits_have_the_limit_of_the_first_wait_and_its_second():
+    """A wait that gives up must not let the CTA leave with a copy in flight: a
+    step's first wait and the species-staged buffers have a second wait behind
+    them; the wait for a later species of a tile has both limits at once."""
+    every = "\n".join(open(f).read() for f in glob.glob(os.path.join(B.CSRC, "*.cu*")))
+    reported = re.findall(r"!\s*mbar_wait\(([^;]*?)\)\)\s*raise_flag", every)
+    assert reported and all(r.endswith("2 * TMA_WAIT_LIMIT") for r in reported), reported
